@@ -135,16 +135,26 @@ static int grid_for(long long n) {
 }
 
 // ----------------------------------------------------------------------------- SIMT GEMM
-template <typename T, typename OutT, int BM, int BN, int BK, int TM, int TN>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN))
+// Bound by the FP64 pipe: an FP64 warp instruction holds a sub-partition's pipe for 64
+// cycles (76 with four warps on an SM, 1.68 FMA per clock and SM), so a tile of BM x BN
+// costs BM * BN * K / 1.68 cycles on its SM whatever its shape, and what counts is that all
+// SMs have the same share of the outputs (pick_tile).  KG thread groups split the K indices
+// of a tile (group g takes kk = g mod KG of every K chunk) and add up in a fixed order, so
+// that small tiles still give every sub-partition a warp.  The next K chunk is fetched
+// into registers while the current one is multiplied.
+template <typename T, typename OutT, int BM, int BN, int BK, int TM, int TN, int KG>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG)
 simt_gemm_kernel(SimtGemm<T, OutT> g) {
-  constexpr int NT = (BM / TM) * (BN / TN);
+  constexpr int NT = (BM / TM) * (BN / TN) * KG;
+  constexpr int NG = NT / KG;            // threads of one K group
   constexpr int GX = BN / TN;            // threads along n
   constexpr int GY = BM / TM;            // threads along m
+  constexpr int EA = (BM * BK + NT - 1) / NT, EB = (BN * BK + NT - 1) / NT;
   __shared__ T As[BK][BM + 1];
   __shared__ T Bs[BK][BN + 1];
   const int tid = threadIdx.x;
-  const int tx = tid % GX, ty = tid / GX;
+  const int kg = tid / NG, tg = tid % NG;
+  const int tx = tg % GX, ty = tg / GX;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   const int z = blockIdx.z;
   const int b = z / g.splitk, sk = z % g.splitk;
@@ -161,35 +171,90 @@ simt_gemm_kernel(SimtGemm<T, OutT> g) {
     for (int j = 0; j < TN; ++j) acc[i][j] = T(0);
   const bool a_kfast = (g.sak == 1);
   const bool b_kfast = (g.sbk == 1);
+  T pa[EA], pb[EB];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < EA; ++q) {
+      const int e = tid + q * NT;
+      const int mm = a_kfast ? e / BK : e % BM, kk = a_kfast ? e % BK : e / BM;
+      const int m = m0 + mm, k = k0 + kk;
+      pa[q] = (e < BM * BK && m < g.M && k < kend)
+                  ? A[(long long)m * g.sam + (long long)k * g.sak] : T(0);
+    }
+#pragma unroll
+    for (int q = 0; q < EB; ++q) {
+      const int e = tid + q * NT;
+      const int nn = b_kfast ? e / BK : e % BN, kk = b_kfast ? e % BK : e / BN;
+      const int n = n0 + nn, k = k0 + kk;
+      pb[q] = (e < BN * BK && n < g.N && k < kend)
+                  ? B[(long long)n * g.sbn + (long long)k * g.sbk] : T(0);
+    }
+  };
+  fetch(kbeg);
   for (int k0 = kbeg; k0 < kend; k0 += BK) {
 #pragma unroll
-    for (int e = tid; e < BM * BK; e += NT) {
-      int mm, kk;
-      if (a_kfast) { mm = e / BK; kk = e % BK; } else { kk = e / BM; mm = e % BM; }
-      const int m = m0 + mm, k = k0 + kk;
-      As[kk][mm] = (m < g.M && k < kend) ? A[(long long)m * g.sam + (long long)k * g.sak] : T(0);
+    for (int q = 0; q < EA; ++q) {
+      const int e = tid + q * NT;
+      if (e < BM * BK) {
+        if (a_kfast) As[e % BK][e / BK] = pa[q];
+        else As[e / BM][e % BM] = pa[q];
+      }
     }
 #pragma unroll
-    for (int e = tid; e < BN * BK; e += NT) {
-      int nn, kk;
-      if (b_kfast) { nn = e / BK; kk = e % BK; } else { kk = e / BN; nn = e % BN; }
-      const int n = n0 + nn, k = k0 + kk;
-      Bs[kk][nn] = (n < g.N && k < kend) ? B[(long long)n * g.sbn + (long long)k * g.sbk] : T(0);
+    for (int q = 0; q < EB; ++q) {
+      const int e = tid + q * NT;
+      if (e < BN * BK) {
+        if (b_kfast) Bs[e % BK][e / BK] = pb[q];
+        else Bs[e / BN][e % BN] = pb[q];
+      }
     }
     __syncthreads();
+    if (k0 + BK < kend) fetch(k0 + BK);
+    const int kn = min(BK, kend - k0);   // the zero padding of a short chunk is not multiplied
+    if (kn == BK) {
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      T a[TM], bb[TN];
+      for (int q = 0; q < BK / KG; ++q) {
+        const int kk = q * KG + kg;
+        T a[TM], bb[TN];
 #pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + i * GY];
+        for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + i * GY];
 #pragma unroll
-      for (int j = 0; j < TN; ++j) bb[j] = Bs[kk][tx + j * GX];
+        for (int j = 0; j < TN; ++j) bb[j] = Bs[kk][tx + j * GX];
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+      }
+    } else {
+      for (int kk = kg; kk < kn; kk += KG) {
+        T a[TM], bb[TN];
+#pragma unroll
+        for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + i * GY];
+#pragma unroll
+        for (int j = 0; j < TN; ++j) bb[j] = Bs[kk][tx + j * GX];
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+      }
+    }
+    __syncthreads();
+  }
+  if constexpr (KG > 1) {   // sums of the K groups, in group order
+    __shared__ T red[KG - 1][NG][TM * TN + 1];
+    if (kg > 0)
 #pragma unroll
       for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
-    }
+        for (int j = 0; j < TN; ++j) red[kg - 1][tg][i * TN + j] = acc[i][j];
     __syncthreads();
+    if (kg > 0) return;
+#pragma unroll
+    for (int q = 0; q < KG - 1; ++q)
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] += red[q][tg][i * TN + j];
   }
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
@@ -208,20 +273,73 @@ simt_gemm_kernel(SimtGemm<T, OutT> g) {
   }
 }
 
+static int simt_sms() {
+  static int n = 0;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    int dev = 0;
+    A2_CUDA(cudaGetDevice(&dev));
+    A2_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+  });
+  return n > 0 ? n : 1;
+}
+
+template <typename T, typename OutT, int BM, int BN, int BK, int TM, int TN, int KG>
+static void simt_launch(const SimtGemm<T, OutT>& g, cudaStream_t s) {
+  dim3 grid(cdiv(g.N, BN), cdiv(g.M, BM), g.batch * g.splitk);
+  A2_REQUIRE(grid.y < 65536 && grid.z < 65536, "GEMM grid too large");
+  simt_gemm_kernel<T, OutT, BM, BN, BK, TM, TN, KG>
+      <<<grid, (BM / TM) * (BN / TN) * KG, 0, s>>>(g);
+}
+
+// Index of the tile edge (of `edges`, descending) with the least work on the busiest SM:
+// rounds of blocks over the SMs times the tile's area, divided by the tile's relative
+// efficiency.  A smaller tile also has to gain something (its loads per product are more).
+static int pick_tile(int M, int N, long long batch, const int* edges, const double* eff, int n) {
+  const int sms = simt_sms();
+  int best = 0;
+  double best_cost = 0.0;
+  for (int i = 0; i < n; ++i) {
+    const long long ty = cdiv(M, edges[i]), tiles = ty * cdiv(N, edges[i]) * batch;
+    if (i > 0 && ty >= 65536) break;
+    const double cost =
+        (double)((tiles + sms - 1) / sms) * edges[i] * edges[i] / eff[i];
+    if (i == 0 || cost < best_cost) {
+      best = i;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
+// FP64: S4 of the Heisenberg operator at D = 32 (M 128, N 32, K 160) takes 172 us on the
+// two 64 x 64 tiles it has and 6.5 us on 64 tiles of 8 x 8; S1 (160 x 128 x 32) 38 and
+// 4.8 us.  Products with many tiles run at the pipe's rate with every tile (P^T M of a
+// 1024 x 1024 split, 256 x 1024 x 1024: 64 tiles of 64 leave 88 SMs idle, 1.10 ms; 1024
+// tiles of 16: 0.46 ms), hence the small penalties.  FP32: the wide tiles reuse shared memory
+// more, which is what bounds them, hence the large ones.
 template <typename T, typename OutT>
 void simt_gemm(const SimtGemm<T, OutT>& g, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
   A2_REQUIRE(g.splitk == 1 || g.mode == GEMM_ATOMIC, "split-K needs atomic mode");
+  const long long nz = (long long)g.batch * g.splitk;
   if constexpr (sizeof(T) == 8) {
-    constexpr int BM = 64, BN = 64, BK = 8, TM = 4, TN = 4;
-    dim3 grid(cdiv(g.N, BN), cdiv(g.M, BM), g.batch * g.splitk);
-    A2_REQUIRE(grid.y < 65536 && grid.z < 65536, "GEMM grid too large");
-    simt_gemm_kernel<T, OutT, BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, s>>>(g);
+    static const int edges[4] = {64, 32, 16, 8};
+    static const double eff[4] = {1.0, 0.97, 0.9, 0.8};
+    switch (pick_tile(g.M, g.N, nz, edges, eff, 4)) {
+      case 0: simt_launch<T, OutT, 64, 64, 16, 4, 4, 1>(g, s); break;
+      case 1: simt_launch<T, OutT, 32, 32, 16, 2, 2, 1>(g, s); break;
+      case 2: simt_launch<T, OutT, 16, 16, 32, 2, 2, 4>(g, s); break;
+      default: simt_launch<T, OutT, 8, 8, 32, 1, 1, 4>(g, s); break;
+    }
   } else {
-    constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8;
-    dim3 grid(cdiv(g.N, BN), cdiv(g.M, BM), g.batch * g.splitk);
-    A2_REQUIRE(grid.y < 65536 && grid.z < 65536, "GEMM grid too large");
-    simt_gemm_kernel<T, OutT, BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, s>>>(g);
+    static const int edges[3] = {128, 64, 32};
+    static const double eff[3] = {1.0, 0.6, 0.3};
+    switch (pick_tile(g.M, g.N, nz, edges, eff, 3)) {
+      case 0: simt_launch<T, OutT, 128, 128, 8, 8, 8, 1>(g, s); break;
+      case 1: simt_launch<T, OutT, 64, 64, 16, 4, 4, 1>(g, s); break;
+      default: simt_launch<T, OutT, 32, 32, 32, 2, 2, 1>(g, s); break;
+    }
   }
   A2_CHECK_LAUNCH();
 }
