@@ -1099,19 +1099,19 @@ struct LanczosResult {
   bool converged = false;
 };
 
-// Restarted Lanczos with full re-orthogonalisation (twice) for the lowest eigenpair of
-// the operator `mv`, started from x0 (device, overwritten by the unit Ritz vector with
-// <x, x0> >= 0).  Scalars are reduced on the device and read back once per step.
+// Restarted Lanczos with full re-orthogonalisation for the lowest eigenpair of the operator
+// `mv`, started from x0 (device, overwritten by the unit Ritz vector with <x, x0> >= 0).
+// Everything after an application of the operator is one kernel (lanczos_step), whose four
+// scalars the host reads once per step.
 template <typename MV>
 LanczosResult lanczos(a2_ctx* c, MV&& mv, double* x, long long N, double tol, int max_krylov,
                       int max_cycles) {
   cudaStream_t s = c->stream;
   const int m = (int)std::min<long long>(std::min(max_krylov, 63), N);
-  c->wv.ensure(sizeof(double) * (size_t)(m + 3) * N, s);
+  c->wv.ensure(sizeof(double) * (size_t)(m + 2) * N, s);
   double* V = c->wv.as<double>();
   double* w = V + (size_t)m * N;
   double* x0 = w + N;
-  double* tmp = x0 + N;
   A2_CUDA(cudaMemcpyAsync(x0, x, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
   double nrm2 = dot_dev(c, x, x, N, 0);
   check_finite(nrm2, "Lanczos start vector");
@@ -1121,54 +1121,38 @@ LanczosResult lanczos(a2_ctx* c, MV&& mv, double* x, long long N, double tol, in
     A2_CUDA(cudaMemcpyAsync(x0, x, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
     nrm2 = dot_dev(c, x, x, N, 0);
   }
-  A2_CUDA(cudaMemcpyAsync(V, x, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
-  A2_CUDA(cudaMemcpyAsync(tmp, x, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
-  normalize_into(tmp, scal(c, 0), V, N, s);
+  normalize_into(x, scal(c, 0), V, N, s);
   LanczosResult res;
-  std::vector<double> alpha, beta;
-  std::vector<double> ev(65);
-  double* dev_ev = scal(c, 128);
+  double* tri = scal(c, 512);                 // a, b, eigenvector of the tridiagonal
+  unsigned* bar = reinterpret_cast<unsigned*>(scal(c, 704));   // two pairs of barrier words
+  A2_CUDA(cudaMemsetAsync(bar, 0, 4 * sizeof(unsigned), s));
+  double* out = c->h_scal + 32;
+  long long steps = 0;
   for (int cyc = 1; cyc <= max_cycles; ++cyc) {
     res.cycles = cyc;
-    alpha.clear();
-    beta.clear();
     int j = 0;
     bool conv = false;
-    double theta = 0.0;
-    std::vector<double> svec;
+    double theta = 0.0, beta = 0.0;
     for (j = 0; j < m; ++j) {
       double* vj = V + (size_t)j * N;
       mv(vj, w);
       ++res.matvecs;
-      // alpha_j = <v_j, w>; w -= alpha v_j + beta v_{j-1}
-      ProfScope ps(PK_LANCZOS, s, 2.0 * N * (2.0 * (j + 1) * 2 + 6), 8.0 * N * (4.0 * (j + 1) + 6));
-      dot_multi(vj, 0, 1, w, N, c->partial.as<double>(), scal(c, 1), s);
-      lanczos_update(w, vj, j > 0 ? V + (size_t)(j - 1) * N : nullptr, scal(c, 1),
-                     j > 0 ? beta.back() : 0.0, N, s);
-      for (int pass = 0; pass < 2; ++pass) {   // full re-orthogonalisation
-        dot_multi(V, N, j + 1, w, N, c->partial.as<double>(), scal(c, 8), s);
-        gemv_sub(V, N, j + 1, scal(c, 8), w, N, s);
+      const int k = j + 1;
+      out[4] = 0.0;
+      {
+        ProfScope ps(PK_LANCZOS, s, 2.0 * N * (2.0 * k + 6), 8.0 * N * (2.0 * k + 6));
+        lanczos_step(V, w, N, j, beta, k < m, tri, c->partial.as<double>(), bar + 2 * (steps & 1),
+                     bar + 2 * ((steps + 1) & 1), out, s);
       }
-      dot_multi(w, 0, 1, w, N, c->partial.as<double>(), scal(c, 2), s);
-      fetch_scalars(c, 1, 2);
-      const double a = c->h_scal[1];
-      const double b2 = c->h_scal[2];
-      check_finite(a, "Lanczos alpha");
+      ++steps;
+      A2_CUDA(cudaStreamSynchronize(s));
+      if (out[4] != 0.0) throw CudaError("Lanczos: a bounded grid barrier gave up");
+      const double b2 = out[1];
+      check_finite(out[0], "Lanczos alpha");
       check_finite(b2, "Lanczos beta");
       const double b = std::sqrt(std::max(b2, 0.0));
-      alpha.push_back(a);
-      // lowest eigenpair of the tridiagonal T_j (device bisection + inverse iteration)
-      const int k = j + 1;
-      TridiagIn tin;
-      tin.k = k;
-      for (int i = 0; i < k; ++i) tin.a[i] = alpha[i];
-      for (int i = 0; i + 1 < k; ++i) tin.b[i] = beta[i];
-      tridiag_lowest(tin, dev_ev, s);
-      A2_CUDA(cudaMemcpyAsync(ev.data(), dev_ev, sizeof(double) * (k + 1), cudaMemcpyDeviceToHost, s));
-      A2_CUDA(cudaStreamSynchronize(s));
-      theta = ev[0];
-      svec.assign(ev.begin() + 1, ev.begin() + 1 + k);
-      const double resid = std::fabs(b * svec[k - 1]);
+      theta = out[2];
+      const double resid = b * out[3];
       const bool breakdown = b <= 1e-14 * std::max(1.0, std::fabs(theta));
       if (resid <= tol * std::max(1.0, std::fabs(theta)) || breakdown || k == N) {
         conv = true;
@@ -1176,21 +1160,13 @@ LanczosResult lanczos(a2_ctx* c, MV&& mv, double* x, long long N, double tol, in
         break;
       }
       if (j == m - 1) { ++j; break; }
-      beta.push_back(b);
-      // v_{j+1} = w / b
-      A2_CUDA(cudaMemcpyAsync(scal(c, 3), &b2, sizeof(double), cudaMemcpyHostToDevice, s));
-      normalize_into(w, scal(c, 3), V + (size_t)(j + 1) * N, N, s);
-      A2_CUDA(cudaStreamSynchronize(s));   // b2 is a host stack value
+      beta = b;
     }
     // Ritz vector x = V s (unit), becomes the restart vector
-    A2_CUDA(cudaMemcpyAsync(scal(c, 8), svec.data(), sizeof(double) * svec.size(),
-                            cudaMemcpyHostToDevice, s));
-    gemv_set(V, N, (int)svec.size(), scal(c, 8), x, N, s);
-    double xn = dot_dev(c, x, x, N, 4);
-    A2_CUDA(cudaMemcpyAsync(V, x, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
+    gemv_set(V, N, j, tri + 128, x, N, s);
+    dot_multi(x, 0, 1, x, N, c->partial.as<double>(), scal(c, 4), s);
     normalize_into(x, scal(c, 4), V, N, s);
     A2_CUDA(cudaMemcpyAsync(x, V, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
-    (void)xn;
     res.theta = theta;
     if (conv) { res.converged = true; break; }
   }

@@ -1049,70 +1049,6 @@ template void convert_ld<float, __nv_bfloat16>(const float*, __nv_bfloat16*, lon
                                                long long, long long, cudaStream_t);
 
 // ----------------------------------------------------------------------------- vector kernels
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// partial[j * kReduceBlocks + block] = sum over the block's grid-stride slice of V_j . w
-__global__ void dot_multi_partial(const double* __restrict__ V, long long ldv, int k,
-                                  const double* __restrict__ w, long long n,
-                                  double* __restrict__ partial) {
-  __shared__ double red[8][64];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int j0 = 0; j0 < k; j0 += 8) {
-    const int jn = min(8, k - j0);
-    double acc[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-      const double wi = w[i];
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (q < jn) acc[q] = fma(V[(long long)(j0 + q) * ldv + i], wi, acc[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      double v = warp_sum(acc[q]);
-      if (lane == 0) red[q][wid] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < jn) {
-      double t = 0.0;
-      for (int ww = 0; ww < (int)(blockDim.x >> 5); ++ww) t += red[threadIdx.x][ww];
-      partial[(long long)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
-    }
-    __syncthreads();
-  }
-}
-
-__global__ void reduce_partials(const double* __restrict__ partial, int nb, int k,
-                                double* __restrict__ out) {
-  const int j = blockIdx.x;
-  double acc = 0.0;
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) acc += partial[(long long)j * nb + b];
-  __shared__ double red[32];
-  acc = warp_sum(acc);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    out[j] = t;
-  }
-}
-
-void dot_multi(const double* V, long long ldv, int k, const double* w, long long n,
-               double* partial, double* out, cudaStream_t s) {
-  if (k <= 0) return;
-  dot_multi_partial<<<kReduceBlocks, 256, 0, s>>>(V, ldv, k, w, n, partial);
-  A2_CHECK_LAUNCH();
-  reduce_partials<<<k, 256, 0, s>>>(partial, kReduceBlocks, k, out);
-  A2_CHECK_LAUNCH();
-}
-
 __global__ void gemv_sub_kernel(const double* __restrict__ V, long long ldv, int k,
                                 const double* __restrict__ h, double* __restrict__ w,
                                 long long n, int set_mode) {
@@ -1149,22 +1085,6 @@ __global__ void axpby_kernel(double a, const double* x, double b, double* y, lon
 void axpby(double a, const double* x, double b, double* y, long long n, cudaStream_t s) {
   if (!n) return;
   axpby_kernel<<<grid_for(n), 256, 0, s>>>(a, x, b, y, n);
-  A2_CHECK_LAUNCH();
-}
-
-__global__ void lanczos_update_kernel(double* w, const double* v, const double* vprev,
-                                      const double* alpha, double beta, long long n) {
-  const double a = *alpha;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    double t = w[i] - a * v[i];
-    if (vprev) t -= beta * vprev[i];
-    w[i] = t;
-  }
-}
-void lanczos_update(double* w, const double* v, const double* vprev, const double* alpha,
-                    double beta_prev, long long n, cudaStream_t s) {
-  lanczos_update_kernel<<<grid_for(n), 256, 0, s>>>(w, v, vprev, alpha, beta_prev, n);
   A2_CHECK_LAUNCH();
 }
 
@@ -1404,104 +1324,6 @@ void coarse_solve_dev(const double* A, const double* S, int m, double eps, doubl
                                  (int)sizeof(CoarseShared)));
   });
   coarse_kernel<<<1, 256, sizeof(CoarseShared), s>>>(A, S, m, eps, c, lam, rank, status);
-  A2_CHECK_LAUNCH();
-}
-
-// ----------------------------------------------------------------------------- tridiagonal
-// Lowest eigenpair of the symmetric tridiagonal T (diag a[0..k-1], off-diag b[0..k-2]):
-// bisection on the Sturm count of T - x I (Golub & Van Loan, Sec. 8.4; here 32-way
-// multisection by one warp), then inverse iteration with a partially pivoted tridiagonal
-// solve (one thread, shared-memory arrays).  k <= 64.
-__device__ int sturm_below(const double* a, const double* b, int k, double x) {
-  int cnt = 0;
-  double d = a[0] - x;
-  if (d < 0) ++cnt;
-  for (int i = 1; i < k; ++i) {
-    const double dd = (d == 0.0) ? 1e-300 : d;
-    d = a[i] - x - b[i - 1] * b[i - 1] / dd;
-    if (d < 0) ++cnt;
-  }
-  return cnt;
-}
-
-__global__ void tridiag_lowest_kernel(TridiagIn in, double* out) {
-  // multisection: the 32 lanes evaluate the Sturm count at 32 interior points of the
-  // bracket at once, so that every round shrinks it 33-fold
-  const int lane = threadIdx.x & 31;
-  const int k = in.k;
-  const double* a = in.a;
-  const double* b = in.b;
-  double lo = 1e300, hi = -1e300, scale = 0.0;
-  for (int i = 0; i < k; ++i) {
-    const double r = (i > 0 ? fabs(b[i - 1]) : 0.0) + (i + 1 < k ? fabs(b[i]) : 0.0);
-    lo = fmin(lo, a[i] - r);
-    hi = fmax(hi, a[i] + r);
-    scale = fmax(scale, fabs(a[i]) + r);
-  }
-  for (int it = 0; it < 40 && hi - lo > 4e-16 * fmax(scale, 1e-300); ++it) {
-    const double x = lo + (hi - lo) * (double)(lane + 1) / 33.0;
-    const bool above = sturm_below(a, b, k, x) >= 1;     // lowest eigenvalue <= x
-    const unsigned m = __ballot_sync(0xffffffffu, above);
-    const int j = m ? __ffs(m) - 1 : 32;                 // first point above the eigenvalue
-    const double nlo = j == 0 ? lo : lo + (hi - lo) * (double)j / 33.0;
-    const double nhi = j == 32 ? hi : lo + (hi - lo) * (double)(j + 1) / 33.0;
-    if (!(nlo >= lo && nhi <= hi && nlo < nhi)) break;  // no further progress in FP64
-    lo = nlo;
-    hi = nhi;
-  }
-  const double theta = 0.5 * (lo + hi);
-  if (lane != 0) return;
-  // inverse iteration: (T - theta I) y = v, partially pivoted tridiagonal elimination
-  __shared__ double y[64], v[64], dl[64], d[64], du[64], du2[64], rhs[64];
-  for (int i = 0; i < k; ++i) v[i] = 1.0 / sqrt((double)k) * (1.0 + 0.01 * i);
-  const double eps = 1e-14 * fmax(scale, 1e-300);
-  for (int rep = 0; rep < 3; ++rep) {
-    for (int i = 0; i < k; ++i) {
-      d[i] = a[i] - theta;
-      du[i] = (i + 1 < k) ? b[i] : 0.0;
-      dl[i] = (i + 1 < k) ? b[i] : 0.0;
-      du2[i] = 0.0;
-      rhs[i] = v[i];
-    }
-    for (int i = 0; i + 1 < k; ++i) {
-      if (fabs(d[i]) >= fabs(dl[i])) {
-        const double piv = (d[i] == 0.0) ? eps : d[i];
-        d[i] = piv;
-        const double f = dl[i] / piv;
-        d[i + 1] -= f * du[i];
-        rhs[i + 1] -= f * rhs[i];
-        dl[i] = 0.0;
-      } else {
-        const double f = d[i] / dl[i];
-        d[i] = dl[i];
-        double t = d[i + 1];
-        d[i + 1] = du[i] - f * t;
-        if (i + 2 < k) {
-          du2[i] = du[i + 1];
-          du[i + 1] = -f * du2[i];
-        }
-        du[i] = t;
-        t = rhs[i];
-        rhs[i] = rhs[i + 1];
-        rhs[i + 1] = t - f * rhs[i + 1];
-      }
-    }
-    if (d[k - 1] == 0.0) d[k - 1] = eps;
-    y[k - 1] = rhs[k - 1] / d[k - 1];
-    if (k > 1) y[k - 2] = (rhs[k - 2] - du[k - 2] * y[k - 1]) / d[k - 2];
-    for (int i = k - 3; i >= 0; --i) y[i] = (rhs[i] - du[i] * y[i + 1] - du2[i] * y[i + 2]) / d[i];
-    double nrm = 0.0;
-    for (int i = 0; i < k; ++i) nrm += y[i] * y[i];
-    const double inv = 1.0 / sqrt(nrm);
-    for (int i = 0; i < k; ++i) v[i] = y[i] * inv;
-  }
-  out[0] = theta;
-  for (int i = 0; i < k; ++i) out[1 + i] = v[i];
-}
-
-void tridiag_lowest(const TridiagIn& in, double* out, cudaStream_t s) {
-  A2_REQUIRE(in.k >= 1 && in.k <= 64, "tridiagonal size 1..64");
-  tridiag_lowest_kernel<<<1, 32, 0, s>>>(in, out);
   A2_CHECK_LAUNCH();
 }
 

@@ -101,8 +101,6 @@ void gemv_set(const double* V, long long ldv, int k, const double* h, double* ou
               cudaStream_t s);                                         // out = sum_j h[j] V_j
 void axpby(double a, const double* x, double b, double* y, long long n, cudaStream_t s);
 void scale_dev(double* x, const double* num, const double* den_sqrt, long long n, cudaStream_t s);
-void lanczos_update(double* w, const double* v, const double* vprev, const double* alpha,
-                    double beta_prev, long long n, cudaStream_t s);    // w -= a v + b vprev
 void normalize_into(const double* w, const double* nrm2, double* out, long long n, cudaStream_t s);
 
 // ---- small symmetric eigensolver (one CTA, cyclic Jacobi, m <= 64)
@@ -110,14 +108,18 @@ void normalize_into(const double* w, const double* nrm2, double* out, long long 
 // (evecs[j*m + i] = component i of eigenvector j).  status[0] = sweeps used (or -1).
 void jacobi_eig(double* A, int m, double* evals, double* evecs, int* status, cudaStream_t s);
 
-// Lowest eigenpair of a symmetric tridiagonal matrix passed by value (k <= 64):
-// out[0] = eigenvalue, out[1..k] = unit eigenvector (sign arbitrary).
-struct TridiagIn {
-  int k;
-  double a[64];
-  double b[64];
-};
-void tridiag_lowest(const TridiagIn& in, double* out, cudaStream_t s);
+// One Lanczos step after w = H v_j (lanczos.cu): alpha_j = <v_j, w>, w made orthogonal to
+// v_0 .. v_j, v_{j+1} = w / |w| stored if write_next (basis vector q at V + q * N, w may be
+// the slot behind the last of them), and the lowest eigenpair of the tridiagonal of size
+// j + 1 <= 63.  tri (192 doubles, kept from step to step): a[64], b[64], eigenvector[64].
+// partial: at least kReduceBlocks * 64 doubles.  bar, bar_next: two unsigned each, swapped by the
+// caller from step to step; bar is zero on entry, bar_next is zeroed.  out (pinned host
+// memory, 5 doubles, valid once the stream has completed the step): alpha, |w|^2, the
+// eigenvalue, the magnitude of the eigenvector's last component; out[4] is set to 1 if a
+// bounded wait gave up (zero it before).
+void lanczos_step(double* V, double* w, long long N, int j, double beta_prev, bool write_next,
+                  double* tri, double* partial, unsigned* bar, unsigned* bar_next,
+                  double* out, cudaStream_t s);
 
 // Coarse problem of Sec. 3.1 (m <= 63) in one CTA; outputs on the device.
 void coarse_solve_dev(const double* A, const double* S, int m, double eps, double* c,
