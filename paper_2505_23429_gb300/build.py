@@ -12,7 +12,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "liba2dmrg.so")
-SOURCES = ["kernels.cu", "lanczos.cu", "factor.cu", "tc_gemm.cu", "a2dmrg.cu"]
+SOURCES = ["kernels.cu", "lanczos.cu", "sparse.cu", "factor.cu", "tc_gemm.cu", "a2dmrg.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--diag-suppress=177"]

@@ -89,7 +89,8 @@ struct SiteOps {
   long long nnz_g = 0;
   struct Part {
     int nrows = 0, nnz = 0;
-    DevBuf ptr, rw, rs, nw, nt, v64, v32, v32lo;
+    int in_rows = 0, in_t = 1;
+    DevBuf ptr, rw, rs, nw, nt, v64, v32, v32lo, sell, sell_lo, sell_row;
     template <typename V> SparseRows<V> rows() const {
       SparseRows<V> r;
       r.nrows = nrows;
@@ -102,6 +103,11 @@ struct SiteOps {
       if constexpr (sizeof(V) == 8) r.nz_val = v64.as<double>();
       else r.nz_val = v32.as<float>();
       r.nz_lo = v32lo.as<float>();
+      r.sell = sell.as<int2>();
+      r.sell_lo = sell_lo.as<float>();
+      r.sell_row = sell_row.as<int4>();
+      r.in_rows = in_rows;
+      r.in_t = in_t;
       return r;
     }
   } lr, rl;
@@ -151,25 +157,57 @@ void upload(DevBuf& b, const void* h, size_t bytes, cudaStream_t s) {
   if (bytes) A2_CUDA(cudaMemcpyAsync(b.p, h, bytes, cudaMemcpyHostToDevice, s));
 }
 
+// The rows of a part on the device, sorted by falling number of nonzeros (rows that run side
+// by side in a warp then have the same length); win: input bond dimension, nt: physical
+// values t per bond index.
 void build_part(SiteOps::Part& part, const std::vector<std::vector<std::array<double, 3>>>& rows,
-                const std::vector<std::pair<int, int>>& rowid, cudaStream_t s) {
+                const std::vector<std::pair<int, int>>& rowid, int win, int nt_in,
+                cudaStream_t s) {
   part.nrows = (int)rows.size();
+  part.in_rows = win * nt_in;
+  part.in_t = nt_in;
+  std::vector<int> order(rows.size());
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int x, int y) { return rows[x].size() > rows[y].size(); });
   std::vector<int> ptr(rows.size() + 1, 0), rw, rs, nw, nt;
   std::vector<double> v64;
   std::vector<float> v32, v32lo;
-  for (size_t r = 0; r < rows.size(); ++r) {
+  for (size_t i = 0; i < rows.size(); ++i) {
+    const int r = order[i];
     rw.push_back(rowid[r].first);
     rs.push_back(rowid[r].second);
     for (auto& e : rows[r]) {
       nw.push_back((int)e[0]);
       nt.push_back((int)e[1]);
       v64.push_back(e[2]);
-      v32.push_back((float)e[2]);
-      v32lo.push_back((float)(e[2] - (double)(float)e[2]));
+      const float hi = (float)e[2];
+      v32.push_back(hi);
+      v32lo.push_back((float)(e[2] - (double)hi));
     }
-    ptr[r + 1] = (int)nw.size();
+    ptr[i + 1] = (int)nw.size();
   }
   part.nnz = (int)nw.size();
+  // the same entries interleaved over kSellRows rows (gaps behind the shorter rows)
+  std::vector<int4> meta(rows.size());
+  std::vector<int2> sell;
+  std::vector<float> sell_lo;
+  for (size_t i0 = 0; i0 < rows.size(); i0 += kSellRows) {
+    const size_t base = sell.size(), len0 = rows[order[i0]].size();   // the longest of them
+    sell.resize(base + len0 * kSellRows, int2{0, 0});
+    sell_lo.resize(sell.size(), 0.f);
+    for (size_t i = i0; i < std::min(rows.size(), i0 + kSellRows); ++i) {
+      const int len = ptr[i + 1] - ptr[i];
+      meta[i] = int4{len, (int)(base + (i - i0)), rw[i], rs[i]};
+      for (int e = 0; e < len; ++e) {
+        const int q = ptr[i] + e;
+        int2& k = sell[base + (size_t)e * kSellRows + (i - i0)];
+        k.x = nw[q] * nt_in + nt[q];
+        std::memcpy(&k.y, &v32[q], sizeof(float));
+        sell_lo[base + (size_t)e * kSellRows + (i - i0)] = v32lo[q];
+      }
+    }
+  }
   upload(part.ptr, ptr.data(), ptr.size() * sizeof(int), s);
   upload(part.rw, rw.data(), rw.size() * sizeof(int), s);
   upload(part.rs, rs.data(), rs.size() * sizeof(int), s);
@@ -178,6 +216,9 @@ void build_part(SiteOps::Part& part, const std::vector<std::vector<std::array<do
   upload(part.v64, v64.data(), v64.size() * sizeof(double), s);
   upload(part.v32, v32.data(), v32.size() * sizeof(float), s);
   upload(part.v32lo, v32lo.data(), v32lo.size() * sizeof(float), s);
+  upload(part.sell, sell.data(), sell.size() * sizeof(int2), s);
+  upload(part.sell_lo, sell_lo.data(), sell_lo.size() * sizeof(float), s);
+  upload(part.sell_row, meta.data(), meta.size() * sizeof(int4), s);
 }
 
 // Scan a dense core W[wl][s][t][wr] (minus `sub` = I (x) G when given) into the two
@@ -202,8 +243,8 @@ long long scan_actions(const double* W, const double* G, int Rl, int n, int Rr,
           lr[(size_t)wr * n + sx].push_back({(double)wl, (double)t, v});
           rl[(size_t)wl * n + sx].push_back({(double)wr, (double)t, v});
         }
-  build_part(plr, lr, lrid, s);
-  if (prl) build_part(*prl, rl, rlid, s);
+  build_part(plr, lr, lrid, Rl, n, s);
+  if (prl) build_part(*prl, rl, rlid, Rr, n, s);
   return nnz;
 }
 
@@ -226,8 +267,8 @@ void build_site(SiteOps& so, const double* W, int Rl, int n, int Rr, cudaStream_
       gc[wr].push_back({(double)wl, 0.0, v});
       gr[wl].push_back({(double)wr, 0.0, v});
     }
-  build_part(so.g_lr, gc, gcid, s);
-  build_part(so.g_rl, gr, grid, s);
+  build_part(so.g_lr, gc, gcid, Rl, 1, s);
+  build_part(so.g_rl, gr, grid, Rr, 1, s);
 }
 
 double* scal(a2_ctx* c, int i) { return c->scal.as<double>() + i; }

@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "kernels.cuh"
+#include "sparse.cuh"
 
 namespace a2 {
 
@@ -662,6 +663,10 @@ void sparse_rows_apply_split3(const SparseRows<V>& sp, const SparseGeom& g, cons
   if (sp.nrows == 0 || g.veclen == 0) return;
   constexpr int NV = Vec16<TI>::N;
   if constexpr (sizeof(TI) != 2) A2_REQUIRE(in_plane == 0, "input planes need BF16 input");
+  if constexpr (sizeof(V) == 4 && sizeof(TI) == 2) {
+    if (in_plane && !add && sparse_staged(sp, g, ST_PLANES, in, in_plane, ST_PLANES, out, plane, s))
+      return;
+  }
   auto al = [](long long x) { return x % NV == 0; };
   if (!(al(g.veclen) && al(g.in_sw) && al(g.in_st) && al(g.in_b1) && al(g.in_b2) &&
         al(in_plane) && reinterpret_cast<uintptr_t>(in) % 16 == 0 && al(g.out_sw) &&
@@ -770,6 +775,11 @@ void sparse_rows_apply(const SparseRows<V>& sp, const SparseGeom& g, const TI* i
                        cudaStream_t s) {
   if (sp.nrows == 0 || g.veclen == 0) return;
   constexpr int NV = Vec16<TI>::N;
+  if constexpr (sizeof(V) == 4 && sizeof(TI) == 2 && sizeof(TO) == 2) {
+    if ((const void*)in != (const void*)out &&
+        sparse_staged(sp, g, ST_BF16, in, 0, ST_BF16, out, 0, s))
+      return;
+  }
   auto al = [](long long x) { return x % NV == 0; };
   const bool vec_ok = al(g.veclen) && al(g.in_sw) && al(g.in_st) && al(g.out_sw) &&
                       al(g.out_ss) && al(g.in_b1) && al(g.in_b2) && al(g.out_b1) &&
@@ -883,6 +893,9 @@ void sparse_rows_apply_df(const SparseRows<float>& sp, const SparseGeom& g, cons
                           cudaStream_t s) {
   if (sp.nrows == 0 || g.veclen == 0) return;
   A2_REQUIRE(sp.nz_lo && !g.accumulate, "double-float sparse action: bad arguments");
+  if (out64 ? sparse_staged(sp, g, ST_DF, in_hi, in_plane, ST_F64, out64, 0, s)
+            : sparse_staged(sp, g, ST_DF, in_hi, in_plane, ST_DF, out_hi, out_plane, s))
+    return;
   auto al = [](long long x) { return x % 4 == 0; };
   const bool vec = al(g.veclen) && al(g.in_sw) && al(g.in_st) && al(g.out_sw) &&
                    al(g.out_ss) && al(g.in_b1) && al(g.in_b2) && al(g.out_b1) &&

@@ -41,7 +41,16 @@ struct SparseRows {
   const V* nz_val = nullptr;        // nnz
   long long nnz_total = 0;
   const float* nz_lo = nullptr;     // nnz: FP64 value - (float)value (double-float kernels)
+  // staged kernel (sparse.cu).  The rows are sorted by falling length; the entries of
+  // kSellRows consecutive rows are interleaved: entry e of row r at sell[sell_row[r].y + e *
+  // kSellRows] = {input row nz_w * in_t + nz_t, FP32 value bits}, sell_lo the low parts;
+  // sell_row[r] = {length, first entry, row_w, row_s}.  in_rows: number of input rows.
+  const int2* sell = nullptr;
+  const float* sell_lo = nullptr;
+  const int4* sell_row = nullptr;
+  int in_rows = 0, in_t = 1;
 };
+constexpr int kSellRows = 16;
 
 struct SparseGeom {
   int veclen = 0;
