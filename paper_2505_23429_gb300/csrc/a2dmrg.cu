@@ -448,8 +448,6 @@ void env_right(a2_ctx* c, const SiteOps& so, const T* Hin, const T* bra, int Dlb
 
 // ---- environment updates with FP32-accurate split products on tcgen05 (FP32 envs)
 inline long long round64(long long x) { return (x + 63) / 64 * 64; }
-static const int kPairA[6] = {0, 0, 1, 0, 1, 2};
-static const int kPairB[6] = {0, 1, 0, 2, 1, 0};
 
 struct Planes {   // three BF16 slices of a (rows x K) operand, row stride ld
   const __nv_bfloat16* p[3];
@@ -484,8 +482,7 @@ void env_left_emu(a2_ctx* c, const SiteOps& so, const float* Hin, const double* 
   transpose_split3<double>(ket, Dlk, n * Drk, Kp, ldK, pK, s);
   {  // E1: T1[(a w)][(t b')] = sum_a' Hin[(a w)][a'] ket[a'][(t b')]
     Planes A = planes_at(Hp, ldH, pH), B = planes_at(Kp, ldK, pK);
-    tc_gemm_bf16_pairs(A.p, A.ld, B.p, B.ld, Dlb * Rl, n * Drk, Dlk, 6, kPairA, kPairB, T1,
-                       (long long)n * Drk, 1, 1, s);
+    tc_gemm_split3(A.p, A.ld, B.p, B.ld, Dlb * Rl, n * Drk, Dlk, T1, (long long)n * Drk, false, 1, s);
   }
   {  // E2 (FP32)
     SparseGeom gm;
@@ -499,8 +496,7 @@ void env_left_emu(a2_ctx* c, const SiteOps& so, const float* Hin, const double* 
   transpose_split3<float>(T2, Dlb * n, Rr * Drk, T2p, ldB, pT, s);
   {  // E3: Hout[b][(w' b')] = sum_{(a s)} bra[(a s)][b] T2[(a s)][(w' b')]
     Planes A = planes_at(Bp, ldB, pB), B = planes_at(T2p, ldB, pT);
-    tc_gemm_bf16_pairs(A.p, A.ld, B.p, B.ld, Drb, Rr * Drk, Dlb * n, 6, kPairA, kPairB, Hout,
-                       (long long)Rr * Drk, 1, 1, s);
+    tc_gemm_split3(A.p, A.ld, B.p, B.ld, Drb, Rr * Drk, Dlb * n, Hout, (long long)Rr * Drk, false, 1, s);
   }
 }
 
@@ -532,8 +528,7 @@ void env_right_emu(a2_ctx* c, const SiteOps& so, const float* Hin, const double*
   split3_ld<double>(Vt, (long long)n * Dlk, Drk, Vp, ldV, pV, s);
   {  // F1: T1[(b w')][(t a')] = sum_b' Hin[(b w')][b'] Vt[(t a')][b']
     Planes A = planes_at(Hp, ldH, pH), B = planes_at(Vp, ldV, pV);
-    tc_gemm_bf16_pairs(A.p, A.ld, B.p, B.ld, Drb * Rr, n * Dlk, Drk, 6, kPairA, kPairB, T1,
-                       (long long)n * Dlk, 1, 1, s);
+    tc_gemm_split3(A.p, A.ld, B.p, B.ld, Drb * Rr, n * Dlk, Drk, T1, (long long)n * Dlk, false, 1, s);
   }
   {  // F2 (FP32)
     SparseGeom gm;
@@ -547,8 +542,7 @@ void env_right_emu(a2_ctx* c, const SiteOps& so, const float* Hin, const double*
   transpose_split3<float>(T2, n * Drb, Rl * Dlk, T2p, ldB, pT, s);
   {  // F3: Hout[a][(w a')] = sum_{(s b)} bra[a][(s b)] T2[(s b)][(w a')]
     Planes A = planes_at(Bp, ldB, pB), B = planes_at(T2p, ldB, pT);
-    tc_gemm_bf16_pairs(A.p, A.ld, B.p, B.ld, Dlb, Rl * Dlk, n * Drb, 6, kPairA, kPairB, Hout,
-                       (long long)Rl * Dlk, 1, 1, s);
+    tc_gemm_split3(A.p, A.ld, B.p, B.ld, Dlb, Rl * Dlk, n * Drb, Hout, (long long)Rl * Dlk, false, 1, s);
   }
 }
 
@@ -564,25 +558,22 @@ void env_left_f64e(a2_ctx* c, const SiteOps& so, const double* Hin, const double
                       2.0 * Dlb * Rl * n * Drk + 2.0 * Dlb * n * Rr * Drk));
   const long long M1 = (long long)Dlb * Rl, N1 = (long long)n * Drk;
   const long long N3 = (long long)Rr * Drk, K3 = (long long)Dlb * n;
-  const long long ldH = pad8(Dlk), pH = round64(M1 * ldH);
-  const long long ldK = pad8(Dlk), pK = round64(N1 * ldK);
-  const long long ldB = pad8(K3), pB = round64((long long)Drb * ldB);
-  const long long pT = round64(N3 * ldB);
+  const long long pH = oz_elems(M1, Dlk), pK = oz_elems(N1, Dlk), pB = oz_elems(Drb, K3);
   const long long s1 = M1 * N1, p1 = (s1 + 3) / 4 * 4, s2 = K3 * N3;
-  c->cb.ensure(sizeof(__nv_bfloat16) * (size_t)(kOzSlices * (pH + pK + pB)), s);
+  c->cb.ensure(sizeof(__nv_bfloat16) * (size_t)(pH + pK + pB), s);
   __nv_bfloat16* Hp = c->cb.as<__nv_bfloat16>();
-  __nv_bfloat16* Kp = Hp + kOzSlices * pH;
-  __nv_bfloat16* Bp = Kp + kOzSlices * pK;
+  __nv_bfloat16* Kp = Hp + pH;
+  __nv_bfloat16* Bp = Kp + pK;
   c->tmp1.ensure(std::max(sizeof(float) * 2 * (size_t)p1, sizeof(double) * (size_t)s2), s);
   c->tmp2.ensure(sizeof(double) * (size_t)s2, s);
-  c->t3.ensure(sizeof(__nv_bfloat16) * (size_t)(kOzSlices * pT), s);
+  c->t3.ensure(sizeof(__nv_bfloat16) * (size_t)oz_elems(N3, K3), s);
   float* T1 = c->tmp1.as<float>();
   double* T2 = c->tmp2.as<double>();
   __nv_bfloat16* T2p = c->t3.as<__nv_bfloat16>();
-  ozaki_split(Hin, Dlk, 1, (int)M1, Dlk, Hp, ldH, pH, s);            // rows (a w), K = a'
-  ozaki_split(ket, 1, N1, (int)N1, Dlk, Kp, ldK, pK, s);             // rows (t b'), K = a'
+  ozaki_split(Hin, Dlk, 1, (int)M1, Dlk, Hp, s);                     // rows (a w), K = a'
+  ozaki_split(ket, 1, N1, (int)N1, Dlk, Kp, s);                      // rows (t b'), K = a'
   // E1: T1[(a w)][(t b')] = sum_a' Hin[(a w)][a'] ket[a'][(t b')]   (FP32 pair out)
-  tc_gemm_f64emu(Hp, ldH, pH, Kp, ldK, pK, (int)M1, (int)N1, Dlk, nullptr, N1, c->tf, s, T1, p1);
+  tc_gemm_f64emu(Hp, Kp, (int)M1, (int)N1, Dlk, nullptr, N1, c->tf, s, T1, p1);
   {  // E2: T2[(a s)][(w' b')] = sum_{w,t} A[w,s,t,w'] T1[(a w)][(t b')]   (FP64 out)
     SparseGeom gm;
     gm.veclen = Drk;
@@ -592,9 +583,9 @@ void env_left_f64e(a2_ctx* c, const SiteOps& so, const double* Hin, const double
     sparse_rows_apply_df(so.lr.rows<float>(), gm, T1, p1, nullptr, 0, T2, s);
   }
   // E3: Hout[b][(w' b')] = sum_{(a s)} bra[(a s)][b] T2[(a s)][(w' b')]
-  ozaki_split(bra, 1, Drb, Drb, (int)K3, Bp, ldB, pB, s);            // rows b, K = (a s)
-  ozaki_split_cols(T2, N3, (int)N3, (int)K3, T2p, ldB, pT, s);      // rows (w' b'), K = (a s)
-  tc_gemm_f64emu(Bp, ldB, pB, T2p, ldB, pT, Drb, (int)N3, (int)K3, Hout, N3, c->tf, s);
+  ozaki_split(bra, 1, Drb, Drb, (int)K3, Bp, s);                     // rows b, K = (a s)
+  ozaki_split_cols(T2, N3, (int)N3, (int)K3, T2p, s);               // rows (w' b'), K = (a s)
+  tc_gemm_f64emu(Bp, T2p, Drb, (int)N3, (int)K3, Hout, N3, c->tf, s);
 }
 
 void env_right_f64e(a2_ctx* c, const SiteOps& so, const double* Hin, const double* bra, int Dlb,
@@ -606,28 +597,25 @@ void env_right_f64e(a2_ctx* c, const SiteOps& so, const double* Hin, const doubl
                       2.0 * Drb * Rr * n * Dlk + 2.0 * n * Drb * Rl * Dlk));
   const long long M1 = (long long)Drb * Rr, N1 = (long long)n * Dlk;
   const long long N3 = (long long)Rl * Dlk, K3 = (long long)n * Drb;
-  const long long ldH = pad8(Drk), pH = round64(M1 * ldH);
-  const long long ldV = pad8(Drk), pV = round64(N1 * ldV);
-  const long long ldB = pad8(K3), pB = round64((long long)Dlb * ldB);
-  const long long pT = round64(N3 * ldB);
+  const long long pH = oz_elems(M1, Drk), pV = oz_elems(N1, Drk), pB = oz_elems(Dlb, K3);
   const long long s1 = M1 * N1, p1 = (s1 + 3) / 4 * 4, s2 = K3 * N3;
-  c->cb.ensure(sizeof(__nv_bfloat16) * (size_t)(kOzSlices * (pH + pV + pB)) +
+  c->cb.ensure(sizeof(__nv_bfloat16) * (size_t)(pH + pV + pB) +
                    sizeof(double) * (size_t)n * Dlk * Drk, s);
   __nv_bfloat16* Hp = c->cb.as<__nv_bfloat16>();
-  __nv_bfloat16* Vp = Hp + kOzSlices * pH;
-  __nv_bfloat16* Bp = Vp + kOzSlices * pV;
-  double* Vt = reinterpret_cast<double*>(Bp + kOzSlices * pB);
+  __nv_bfloat16* Vp = Hp + pH;
+  __nv_bfloat16* Bp = Vp + pV;
+  double* Vt = reinterpret_cast<double*>(Bp + pB);
   c->tmp1.ensure(std::max(sizeof(float) * 2 * (size_t)p1, sizeof(double) * (size_t)s2), s);
   c->tmp2.ensure(sizeof(double) * (size_t)s2, s);
-  c->t3.ensure(sizeof(__nv_bfloat16) * (size_t)(kOzSlices * pT), s);
+  c->t3.ensure(sizeof(__nv_bfloat16) * (size_t)oz_elems(N3, K3), s);
   float* T1 = c->tmp1.as<float>();
   double* T2 = c->tmp2.as<double>();
   __nv_bfloat16* T2p = c->t3.as<__nv_bfloat16>();
   permute_swap01<double, double>(ket, Vt, n, Dlk, Drk, s);            // Vt[t][a'][b']
-  ozaki_split(Hin, Drk, 1, (int)M1, Drk, Hp, ldH, pH, s);             // rows (b w'), K = b'
-  ozaki_split(Vt, Drk, 1, (int)N1, Drk, Vp, ldV, pV, s);              // rows (t a'), K = b'
+  ozaki_split(Hin, Drk, 1, (int)M1, Drk, Hp, s);                      // rows (b w'), K = b'
+  ozaki_split(Vt, Drk, 1, (int)N1, Drk, Vp, s);                       // rows (t a'), K = b'
   // F1: T1[(b w')][(t a')] = sum_b' Hin[(b w')][b'] Vt[(t a')][b']   (FP32 pair out)
-  tc_gemm_f64emu(Hp, ldH, pH, Vp, ldV, pV, (int)M1, (int)N1, Drk, nullptr, N1, c->tf, s, T1, p1);
+  tc_gemm_f64emu(Hp, Vp, (int)M1, (int)N1, Drk, nullptr, N1, c->tf, s, T1, p1);
   {  // F2: T2[(s b)][(w a')] = sum_{w',t} A[w,s,t,w'] T1[(b w')][(t a')]   (FP64 out)
     SparseGeom gm;
     gm.veclen = Dlk;
@@ -637,13 +625,13 @@ void env_right_f64e(a2_ctx* c, const SiteOps& so, const double* Hin, const doubl
     sparse_rows_apply_df(so.rl.rows<float>(), gm, T1, p1, nullptr, 0, T2, s);
   }
   // F3: Hout[a][(w a')] = sum_{(s b)} bra[a][(s b)] T2[(s b)][(w a')]
-  ozaki_split(bra, K3, 1, Dlb, (int)K3, Bp, ldB, pB, s);             // rows a, K = (s b)
-  ozaki_split_cols(T2, N3, (int)N3, (int)K3, T2p, ldB, pT, s);      // rows (w a'), K = (s b)
-  tc_gemm_f64emu(Bp, ldB, pB, T2p, ldB, pT, Dlb, (int)N3, (int)K3, Hout, N3, c->tf, s);
+  ozaki_split(bra, K3, 1, Dlb, (int)K3, Bp, s);                      // rows a, K = (s b)
+  ozaki_split_cols(T2, N3, (int)N3, (int)K3, T2p, s);               // rows (w a'), K = (s b)
+  tc_gemm_f64emu(Bp, T2p, Dlb, (int)N3, (int)K3, Hout, N3, c->tf, s);
 }
 
 // Environment updates this small stay on the FP64 SIMT kernels (the Ozaki path costs a
-// dozen launches and 36 tensor-core products per FP64 product).
+// dozen launches and 28 tensor-core products per FP64 product).
 constexpr double kF64eEnvMinFlops = 2e8;
 
 // Split-K factor so that the skinny S4 GEMM fills the GPU.
@@ -882,20 +870,16 @@ struct OzEnvs {
   DevBuf buf;
   const __nv_bfloat16* L = nullptr;
   const __nv_bfloat16* R = nullptr;
-  long long ldl = 0, ldr = 0, lplane = 0, rplane = 0;
   void set(a2_ctx* c, const double* Lf, int Dl, int Rl, const double* Rf, int Dr, int Rr) {
     cudaStream_t s = c->stream;
     ProfScope ps(PK_F64E_SPLIT, s, 0.0,
-                 10.0 * ((double)Dl * Rl * Dl + (double)Dr * Rr * Dr) * 2.0);
-    ldl = pad8(Dl);
-    ldr = pad8((long long)Rr * Dr);
-    lplane = ((long long)Dl * Rl * ldl + 63) / 64 * 64;
-    rplane = ((long long)Dr * ldr + 63) / 64 * 64;
-    buf.ensure(sizeof(__nv_bfloat16) * (size_t)(kOzSlices * (lplane + rplane)), s);
+                 (8.0 + 2.0 * kOzSlices) * ((double)Dl * Rl * Dl + (double)Dr * Rr * Dr));
+    const long long nl = oz_elems((long long)Dl * Rl, Dl), nr = oz_elems(Dr, (long long)Rr * Dr);
+    buf.ensure(sizeof(__nv_bfloat16) * (size_t)(nl + nr), s);
     __nv_bfloat16* lb = buf.as<__nv_bfloat16>();
-    __nv_bfloat16* rb = lb + kOzSlices * lplane;
-    ozaki_split(Lf, Dl, 1, Dl * Rl, Dl, lb, ldl, lplane, s);
-    ozaki_split(Rf, (long long)Rr * Dr, 1, Dr, Rr * Dr, rb, ldr, rplane, s);
+    __nv_bfloat16* rb = lb + nl;
+    ozaki_split(Lf, Dl, 1, Dl * Rl, Dl, lb, s);
+    ozaki_split(Rf, (long long)Rr * Dr, 1, Dr, Rr * Dr, rb, s);
     L = lb;
     R = rb;
   }
@@ -911,19 +895,15 @@ void heff_f64emu(a2_ctx* c, const SiteOps& A1, const SiteOps& A2, const OzEnvs& 
   const int n1 = A1.n, n2 = A2.n, Rl = A1.Rl, R1 = A1.Rr, Rr = A2.Rr;
   cudaStream_t s = c->stream;
   const long long NX = (long long)n1 * n2 * Dr;
-  const long long ldx = pad8(Dl);
-  const long long xplane = (NX * ldx + 63) / 64 * 64;
   const long long s1 = (long long)Dl * Rl * NX, s2 = (long long)Dl * R1 * NX;
   const long long M4 = (long long)Dl * n1 * n2, K4 = (long long)Rr * Dr;
   const long long s3 = M4 * K4;
-  const long long ld3 = pad8(K4);
-  const long long plane3 = (M4 * ld3 + 63) / 64 * 64;
   // T1 and T2 as FP32 pairs (hi plane, lo plane), T3 in FP64 (the slicing input)
   const long long p1 = (s1 + 3) / 4 * 4, p2 = (s2 + 3) / 4 * 4;
-  c->xa.ensure(sizeof(__nv_bfloat16) * (size_t)(kOzSlices * xplane), s);
+  c->xa.ensure(sizeof(__nv_bfloat16) * (size_t)oz_elems(NX, Dl), s);
   c->t1.ensure(std::max(sizeof(float) * 2 * (size_t)p1, sizeof(double) * (size_t)s3), s);
   c->t2.ensure(sizeof(float) * 2 * (size_t)p2, s);
-  c->t3.ensure(sizeof(__nv_bfloat16) * (size_t)(kOzSlices * plane3), s);
+  c->t3.ensure(sizeof(__nv_bfloat16) * (size_t)oz_elems(M4, K4), s);
   __nv_bfloat16* XT = c->xa.as<__nv_bfloat16>();
   float* T1 = c->t1.as<float>();
   float* T2 = c->t2.as<float>();
@@ -931,14 +911,13 @@ void heff_f64emu(a2_ctx* c, const SiteOps& A1, const SiteOps& A2, const OzEnvs& 
   __nv_bfloat16* T3p = c->t3.as<__nv_bfloat16>();
   {  // slices of x^T: row n = column n of x [a'][(s1 s2 b')]
     ProfScope ps(PK_F64E_SPLIT, s, 0.0, (8.0 + 2.0 * kOzSlices) * (double)NX * Dl);
-    ozaki_split(x, 1, NX, (int)NX, Dl, XT, ldx, xplane, s);
+    ozaki_split(x, 1, NX, (int)NX, Dl, XT, s);
   }
   {  // S1: T1[(a w)][(s1 s2 b')] = sum_a' L[(a w)][a'] x[a'][(s1 s2 b')]
     const double M = (double)Dl * Rl, N = (double)NX, K = Dl;
     ProfScope ps(PK_F64E_S1, s, 2.0 * M * N * K,
                  2.0 * kOzSlices * (M * K + N * K) + 8.0 * M * N);
-    tc_gemm_f64emu(E.L, E.ldl, E.lplane, XT, ldx, xplane, Dl * Rl, (int)NX, Dl, nullptr, NX,
-                   c->tf, s, T1, p1);
+    tc_gemm_f64emu(E.L, XT, Dl * Rl, (int)NX, Dl, nullptr, NX, c->tf, s, T1, p1);
   }
   {  // S2 / S3 in double-float arithmetic (FP32 pairs) on the full MPO cores
     ProfScope ps(PK_F64E_SPARSE, s,
@@ -962,14 +941,13 @@ void heff_f64emu(a2_ctx* c, const SiteOps& A1, const SiteOps& A2, const OzEnvs& 
   }
   {
     ProfScope ps(PK_F64E_SPLIT, s, 0.0, (8.0 + 2.0 * kOzSlices) * (double)s3);
-    ozaki_split(T3, K4, 1, (int)M4, (int)K4, T3p, ld3, plane3, s);
+    ozaki_split(T3, K4, 1, (int)M4, (int)K4, T3p, s);
   }
   {  // S4: y[(a s1 s2)][b] = sum_{(w2 b')} T3[(a s1 s2)][(w2 b')] R[b][(w2 b')]
     const double M = (double)M4, N = Dr, K = (double)K4;
     ProfScope ps(PK_F64E_S4, s, 2.0 * M * N * K,
                  2.0 * kOzSlices * (M * K + N * K) + 8.0 * M * N);
-    tc_gemm_f64emu(T3p, ld3, plane3, E.R, E.ldr, E.rplane, (int)M4, Dr, (int)K4, y, Dr, c->tf,
-                   s);
+    tc_gemm_f64emu(T3p, E.R, (int)M4, Dr, (int)K4, y, Dr, c->tf, s);
   }
 }
 
@@ -1521,13 +1499,13 @@ void gemm_f64(a2_ctx* c, int M, int N, int K, const double* A, long long sam, lo
   cudaStream_t s = c->stream;
   const bool tc_ok = (c->parent ? c->parent->gemm_tc : c->gemm_tc) && tc_available();
   if (tc_ok && M >= 16 && N >= 16 && K >= 16 && 2.0 * M * (double)N * K >= kF64eGemmMinFlops) {
-    const long long ld = pad8(K), pA = round64((long long)M * ld), pB = round64((long long)N * ld);
-    c->cb.ensure(sizeof(__nv_bfloat16) * (size_t)(kOzSlices * (pA + pB)), s);
+    const long long pA = oz_elems(M, K), pB = oz_elems(N, K);
+    c->cb.ensure(sizeof(__nv_bfloat16) * (size_t)(pA + pB), s);
     __nv_bfloat16* Ap = c->cb.as<__nv_bfloat16>();
-    __nv_bfloat16* Bp = Ap + kOzSlices * pA;
-    ozaki_split(A, sam, sak, M, K, Ap, ld, pA, s);
-    ozaki_split(B, sbn, sbk, N, K, Bp, ld, pB, s);
-    tc_gemm_f64emu(Ap, ld, pA, Bp, ld, pB, M, N, K, C, ldc, c->tf, s);
+    __nv_bfloat16* Bp = Ap + pA;
+    ozaki_split(A, sam, sak, M, K, Ap, s);
+    ozaki_split(B, sbn, sbk, N, K, Bp, s);
+    tc_gemm_f64emu(Ap, Bp, M, N, K, C, ldc, c->tf, s);
     return;
   }
   SimtGemm<double, double> g;

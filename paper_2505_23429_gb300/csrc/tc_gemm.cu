@@ -63,7 +63,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int co
     if (mbar_try_wait(bar, parity)) return true;
     if (it > 64) __nanosleep(64);
   }
-  atomicExch(&g_tc_error, code);
+  atomicCAS(&g_tc_error, 0, code);   // the first wait that gave up is reported
   return false;
 }
 
@@ -124,6 +124,37 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
+// The same MMA in a run of MMAs on one A tile: the first keeps A in the tensor core's
+// collector buffer (fill), the others take it from there (use, lastuse) instead of reading
+// shared memory again.
+template <bool FIRST, bool LAST>
+__device__ __forceinline__ void mma_bf16_a(uint32_t tmem_d, uint64_t a, uint64_t b,
+                                           uint32_t idesc, uint32_t accumulate) {
+#define A2_MMA_A(op)                                                                          \
+  asm volatile(                                                                               \
+      "{\n\t.reg .pred p;\n\t"                                                              \
+      "setp.ne.b32 p, %4, 0;\n\t"                                                             \
+      "tcgen05.mma.cta_group::1.kind::f16.collector::a::" op " [%0], %1, %2, %3, p;\n\t}" ::"r"( \
+          tmem_d),                                                                            \
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate))
+  if constexpr (FIRST && LAST) A2_MMA_A("discard");
+  else if constexpr (FIRST) A2_MMA_A("fill");
+  else if constexpr (LAST) A2_MMA_A("lastuse");
+  else A2_MMA_A("use");
+#undef A2_MMA_A
+}
+
+// One lane of a converged warp (always the same one).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t"
+      "elect.sync _|P, 0xffffffff;\n\t"
+      "selp.b32 %0, 1, 0, P;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile(
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -177,9 +208,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
 
 enum OutKind { OUT_BF16 = 0, OUT_F32 = 1, OUT_F32_ATOMIC = 2 };
 
-constexpr int kMaxPlanes = 8;      // BF16 planes per operand (8: the FP64 level products)
-constexpr int kMaxPairs = 8;       // operand pairs accumulated into one tile
-
 struct TcArgs {
   int M, N, K;
   int nk1, nk2;            // K blocks of the plain product and of the optional second segment
@@ -189,37 +217,29 @@ struct TcArgs {
   void* C;
   long long ldc;
   int out_kind;
-  int npairs;              // operand pairs accumulated into one tile (split precision)
-  int pa[kMaxPairs], pb[kMaxPairs];   // A / B plane of each pair
   int tma_store;           // 1: epilogue through shared memory + TMA bulk tensor store
-  long long split_ld;      // > 0: K split sp stores its own FP32 tile at C + sp * split_ld
   uint32_t wait_limit;     // iterations of every bounded wait (kWaitLimit)
   int no_loads;            // self-test only: the producer issues no copies, so the first
                            // wait of the MMA role runs out (see tc_selftest_timeout)
 };
 
-// Up to three BF16 planes per operand (a value split into high, middle and low parts).
 // a2 / b2: the optional second K segment, A as a 4D view [a][w1][s12][b'] (box
 // 64 x n12 x 1 x 128/n12, i.e. 128 rows (a, s12) x 64 b') and B as a 3D view
 // [b][w1][b'] (box 64 x 1 x BN); both land in shared memory exactly like the 2D boxes.
 struct TcMaps {
-  CUtensorMap a[kMaxPlanes];
-  CUtensorMap b[kMaxPlanes];
-  CUtensorMap a2[3];
-  CUtensorMap b2[3];
+  CUtensorMap a, b, a2, b2;
   CUtensorMap c;           // output (FP32 box 32 x 32 or BF16 box 64 x 32, 128B swizzle)
 };
 
-// Epilogue warps: 4 (one per TMEM lane quarter, each draining all BN columns), or 8 in
-// the promoted mode (two per lane quarter, 128 columns each, FP32 register accumulators).
-__host__ __device__ constexpr int epi_warps(bool promote) { return promote ? 8 : 4; }
-__host__ __device__ constexpr int tc_threads(bool promote) { return 64 + 32 * epi_warps(promote); }
+// Epilogue warps: one per TMEM lane quarter, each draining all BN columns.
+constexpr int kEpi = 4;
+constexpr int kTcThreads = 64 + 32 * kEpi;
 
-template <int BN, int STAGES, int EPI, int NBUF>
+template <int BN, int STAGES>
 struct TcSmem {
   alignas(1024) __nv_bfloat16 a[STAGES][BM * BK];
   alignas(1024) __nv_bfloat16 b[STAGES][BN * BK];
-  alignas(1024) unsigned char cbuf[EPI][NBUF][4096];      // epilogue staging buffers
+  alignas(1024) unsigned char cbuf[kEpi][2][4096];        // epilogue staging buffers
   alignas(8) uint64_t full[STAGES];                // TMA -> MMA
   alignas(8) uint64_t empty[STAGES];               // MMA -> TMA
   alignas(8) uint64_t acc_full[2];                 // MMA -> epilogue (per TMEM buffer)
@@ -268,9 +288,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-static_assert(sizeof(TcSmem<256, 4, 4, 2>) + 1024 <= 227 * 1024, "BN=256 ring exceeds smem");
-static_assert(sizeof(TcSmem<128, 6, 4, 2>) + 1024 <= 227 * 1024, "BN=128 ring exceeds smem");
-static_assert(sizeof(TcSmem<256, 4, 8, 1>) + 1024 <= 227 * 1024, "promoted ring exceeds smem");
+static_assert(sizeof(TcSmem<256, 4>) + 1024 <= 227 * 1024, "BN=256 ring exceeds smem");
+static_assert(sizeof(TcSmem<128, 6>) + 1024 <= 227 * 1024, "BN=128 ring exceeds smem");
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -285,8 +304,15 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parit
     if ((it & 255) == 255 && *(volatile const int*)abort_flag) return false;
     if (it > 64) __nanosleep(64);
   }
-  atomicExch(&g_tc_error, code);
+  atomicCAS(&g_tc_error, 0, code);   // the first wait that gave up is reported
   return false;
+}
+
+// The same for a converged warp: every lane waits, and all get the same answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int code,
+                                               const int* abort_flag,
+                                               uint32_t limit = kWaitLimit) {
+  return __all_sync(0xffffffffu, mbar_wait_or_abort(bar, parity, code, abort_flag, limit));
 }
 
 // Persistent warp-specialised GEMM.  Work unit = (128 x BN output tile, K split); CTA c
@@ -296,30 +322,19 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parit
 // TMEM lanes 32*(w%4)..+31) and store it, so the epilogue of one unit overlaps the MMAs
 // of the next.  Every wait is bounded; a timeout raises the device error flag and all
 // roles leave their loops, wait (bounded) for their copies / MMAs in flight and exit.
-// PROMOTE (FP32 outputs, BN = 256): the tensor cores' FP32 accumulator truncates, so
-// over long reductions its error grows with the number of accumulate steps.  In this
-// mode every kPromoteKB K blocks (with their operand pairs) are accumulated into a fresh
-// TMEM buffer and the eight epilogue warps add the partials into IEEE FP32 registers
-// (round to nearest), 128 columns of one row per thread.
-constexpr int kPromoteKB = 2;
-
-template <int BN, int STAGES, bool PROMOTE>
-__global__ void __launch_bounds__(tc_threads(PROMOTE), 1)
+template <int BN, int STAGES>
+__global__ void __launch_bounds__(kTcThreads, 1)
 tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs args) {
-  constexpr int EPI = epi_warps(PROMOTE);
-  constexpr int NBUF = PROMOTE ? 1 : 2;
-  static_assert(!PROMOTE || BN == 256, "promoted accumulation: two warps x 128 columns");
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
   const uint32_t pad = (1024u - (base & 1023u)) & 1023u;
-  auto& S = *reinterpret_cast<TcSmem<BN, STAGES, EPI, NBUF>*>(smem_raw + pad);
+  auto& S = *reinterpret_cast<TcSmem<BN, STAGES>*>(smem_raw + pad);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tiles_m = (args.M + BM - 1) / BM;
   const int tiles_n = (args.N + BN - 1) / BN;
   const int nk_total = args.nk1 + args.nk2;
   const int nunits = tiles_m * tiles_n * args.splits;
-  const int np = args.npairs;
   constexpr uint32_t kStageBytes = (BM + BN) * BK * 2;
 
   if (threadIdx.x == 0) {
@@ -329,7 +344,7 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs args) {
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&S.acc_full[i], 1);
-      mbar_init(&S.acc_empty[i], EPI);
+      mbar_init(&S.acc_empty[i], kEpi);
     }
     mbar_init(&S.drain, 1);
     S.abort_flag = 0;
@@ -361,8 +376,7 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs args) {
         const int n0 = ((u / tiles_m) % tiles_n) * BN;
         int kb0, nkb;
         unit_k(u, kb0, nkb);
-        const int steps = nkb * np;
-        for (int kb = 0; kb < steps; ++kb, ++g) {
+        for (int kb = 0; kb < nkb; ++kb, ++g) {
           const int s = g % STAGES;
           const uint32_t round = g / STAGES;
           if (round > 0 &&
@@ -372,17 +386,16 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs args) {
           }
           if (*(volatile int*)&S.abort_flag) break;
           mbar_expect_tx(&S.full[s], kStageBytes);
-          const int p = kb % np;
-          const int kbg = kb0 + kb / np;
+          const int kbg = kb0 + kb;
           if (kbg < args.nk1) {
             const int kx = kbg * BK;
-            tma_load_2d(&maps.a[args.pa[p]], &S.full[s], S.a[s], kx, m0);
-            tma_load_2d(&maps.b[args.pb[p]], &S.full[s], S.b[s], kx, n0);
+            tma_load_2d(&maps.a, &S.full[s], S.a[s], kx, m0);
+            tma_load_2d(&maps.b, &S.full[s], S.b[s], kx, n0);
           } else {   // second segment: K block = (w1, chunk of b')
             const int j = kbg - args.nk1;
             const int w1 = j / args.nbc2, bx = (j % args.nbc2) * BK;
-            tma_load_4d(&maps.a2[args.pa[p]], &S.full[s], S.a[s], bx, 0, w1, m0 / args.n12);
-            tma_load_3d(&maps.b2[args.pb[p]], &S.full[s], S.b[s], bx, w1, n0);
+            tma_load_4d(&maps.a2, &S.full[s], S.a[s], bx, 0, w1, m0 / args.n12);
+            tma_load_3d(&maps.b2, &S.full[s], S.b[s], bx, w1, n0);
           }
           issued = g + 1;
         }
@@ -394,68 +407,64 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs args) {
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer
-      constexpr uint32_t idesc = idesc_bf16(BM, BN);
-      uint32_t g = 0, ch = 0;                        // ring steps, accumulator chunks
-      bool issued_any = false, ok = true;
-      for (int u = blockIdx.x; ok && u < nunits && !*(volatile int*)&S.abort_flag;
-           u += gridDim.x) {
-        int kb0, nkb;
-        unit_k(u, kb0, nkb);
-        const int steps = nkb * np;
-        const int cs = PROMOTE ? kPromoteKB * np : steps;   // steps per accumulator chunk
-        for (int st0 = 0; st0 < steps; st0 += cs, ++ch) {
-          const uint32_t buf = ch & 1, use = ch >> 1;
-          if (use > 0 &&
-              !mbar_wait_or_abort(&S.acc_empty[buf], (use - 1) & 1, 5, &S.abort_flag, args.wait_limit)) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t d = tmem + buf * BN;
-          const int st1 = min(steps, st0 + cs);
-          for (int kb = st0; kb < st1; ++kb, ++g) {
-            const int s = g % STAGES;
-            if (!mbar_wait_or_abort(&S.full[s], (g / STAGES) & 1, 3, &S.abort_flag, args.wait_limit)) {
-              ok = false;
-              break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t da = smem_desc(S.a[s]);
-            const uint64_t db = smem_desc(S.b[s]);
+    // ---------------- MMA issuer (warp-uniform loops, one lane issues)
+    const bool leader = elect_one();
+    constexpr uint32_t idesc = idesc_bf16(BM, BN);
+    constexpr uint32_t kStepA = (BM * BK * 2) >> 4, kStepB = (BN * BK * 2) >> 4;
+    const uint64_t ad = smem_desc(S.a[0]), bd = smem_desc(S.b[0]);
+    uint32_t s = 0, par = 0, ch = 0;                // ring stage, its parity, accumulators
+    bool issued_any = false, ok = true;
+    for (int u = blockIdx.x; ok && u < nunits; u += gridDim.x, ++ch) {
+      int kb0, nkb;
+      unit_k(u, kb0, nkb);
+      const uint32_t buf = ch & 1, use = ch >> 1;
+      if (use > 0)
+        ok = mbar_wait_warp(&S.acc_empty[buf], (use - 1) & 1, 5, &S.abort_flag,
+                            args.wait_limit);
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t d = tmem + buf * BN;
+      for (int kb = 0; kb < nkb; ++kb) {
+        ok = mbar_wait_warp(&S.full[s], par, 3, &S.abort_flag, args.wait_limit);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (leader) {
 #pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk)
-              mma_bf16(d, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc,
-                       (kb > st0 || kk > 0) ? 1u : 0u);
-            issued_any = true;
-            mma_commit(&S.empty[s]);   // frees the stage once these MMAs have read it
-          }
-          if (!ok) break;
-          mma_commit(&S.acc_full[buf]);
+          for (int kk = 0; kk < BK / 16; ++kk)
+            mma_bf16(d, ad + s * kStepA + kk * 2, bd + s * kStepB + kk * 2, idesc,
+                     (kb > 0 || kk > 0) ? 1u : 0u);
+          mma_commit(&S.empty[s]);   // frees the stage once these MMAs have read it
+        }
+        issued_any = true;
+        if (++s == STAGES) {
+          s = 0;
+          par ^= 1;
         }
       }
-      if (!ok) S.abort_flag = 1;
-      if (*(volatile int*)&S.abort_flag && issued_any) {
-        mma_commit(&S.drain);      // wait (bounded) for the MMAs still in flight
-        mbar_wait(&S.drain, 0, 6, args.wait_limit);
-      }
+      if (!ok) break;
+      if (leader) mma_commit(&S.acc_full[buf]);
     }
+    if (!ok) S.abort_flag = 1;
+    if (*(volatile int*)&S.abort_flag && issued_any && leader) {
+      mma_commit(&S.drain);      // wait (bounded) for the MMAs still in flight
+      mbar_wait(&S.drain, 0, 6, args.wait_limit);
+    }
+    __syncwarp();
   } else {
     // ---------------- epilogue warps
     const int q = warp & 3;                          // TMEM lane quarter of this warp
     const int ew = warp - 2;                         // epilogue warp index
-    const int colbase = PROMOTE ? (ew >> 2) * 128 : 0;   // columns of this warp (promoted)
-    unsigned char* wbuf = S.cbuf[ew][0];             // NBUF x 4 KB, 1024-byte aligned
+    unsigned char* wbuf = S.cbuf[ew][0];             // 2 x 4 KB, 1024-byte aligned
     const bool bf16_out = args.out_kind == OUT_BF16;
     uint32_t ch = 0, chunk = 0;
     bool ok = true;
-    // wait for accumulator chunk `ch` and return its TMEM base
+    // wait for accumulator `ch` and return its TMEM base
     auto acquire = [&](uint32_t& tl) -> bool {
       const uint32_t buf = ch & 1, use = ch >> 1;
-      if (!mbar_wait_or_abort(&S.acc_full[buf], use & 1, 4, &S.abort_flag, args.wait_limit)) return false;
+      if (!mbar_wait_or_abort(&S.acc_full[buf], use & 1, 4, &S.abort_flag, 4 * args.wait_limit))
+        return false;   // (four times the limit of the role it waits for)
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      tl = tmem + buf * BN + (uint32_t)colbase + ((uint32_t)(q * 32) << 16);
+      tl = tmem + buf * BN + ((uint32_t)(q * 32) << 16);
       return true;
     };
     auto release = [&]() {
@@ -466,11 +475,8 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs args) {
     };
     // stage one row segment of 32 FP32 values (this lane's row) and store the 32-row slab
     auto store32 = [&](const float (&v)[32], int n0c, int row0) {
-      unsigned char* sb = wbuf + (chunk % NBUF) * 4096;
-      if (lane == 0) {                    // the store issued from sb NBUF chunks ago
-        if (NBUF == 1) bulk_wait_read0();
-        else bulk_wait_read1();
-      }
+      unsigned char* sb = wbuf + (chunk & 1) * 4096;
+      if (lane == 0) bulk_wait_read1();   // the store issued from sb two chunks ago
       __syncwarp();
       const uint32_t rowa = smem_u32(sb) + lane * 128;
 #pragma unroll
@@ -521,38 +527,7 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs args) {
       const int n0 = ((u / tiles_m) % tiles_n) * BN;
       const int row0 = m0 + q * 32;
       const bool rows_here = row0 < args.M;
-      if constexpr (PROMOTE) {
-        int kb0, nkb;
-        unit_k(u, kb0, nkb);
-        const int steps = nkb * np, cs = kPromoteKB * np;
-        float acc[128];
-#pragma unroll
-        for (int i = 0; i < 128; ++i) acc[i] = 0.f;
-        for (int st0 = 0; st0 < steps; st0 += cs) {
-          uint32_t tl;
-          if (!acquire(tl)) { ok = false; break; }
-#pragma unroll
-          for (int c0 = 0; c0 < 128; c0 += 32) {
-            float v[32];
-            tmem_ld32(tl + (uint32_t)c0, v);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) acc[c0 + i] += v[i];
-          }
-          release();
-        }
-        if (!ok) break;
-#pragma unroll
-        for (int c0 = 0; c0 < 128; c0 += 32) {
-          const int col = n0 + colbase + c0;
-          if (col < args.N && rows_here) {
-            float v[32];
-#pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = acc[c0 + i];
-            if (args.tma_store) store32(v, col, row0);
-            else plain32(v, col, row0, args.C);
-          }
-        }
-      } else {
+      {
         uint32_t tl;
         if (!acquire(tl)) { ok = false; break; }
         if (args.tma_store && rows_here) {
@@ -592,15 +567,12 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, TcArgs args) {
             }
           }
         } else if (!args.tma_store) {
-          void* Cb = args.C;
-          if (args.split_ld > 0)
-            Cb = reinterpret_cast<float*>(args.C) + (long long)(u / (tiles_m * tiles_n)) * args.split_ld;
 #pragma unroll 1
           for (int c0 = 0; c0 < BN; c0 += 32) {
             if (n0 + c0 >= args.N) break;
             float v[32];
             tmem_ld32(tl + (uint32_t)c0, v);
-            plain32(v, n0 + c0, row0, Cb);
+            plain32(v, n0 + c0, row0, args.C);
           }
         }
         release();
@@ -667,26 +639,24 @@ CUtensorMap make_map_nd(const __nv_bfloat16* ptr, int rank, const cuuint64_t* di
   return m;
 }
 
-// Returns the number of K splits launched.  split_ld > 0: every split stores its own FP32
-// tile at C + sp * split_ld (plain stores), with at most `splitk`-derived K blocks each.
-template <int BN, int STAGES, bool PROMOTE>
-int launch(const __nv_bfloat16* const* A, long long lda, const __nv_bfloat16* const* B,
-           long long ldb, int M, int N, int K, int npairs, const int* pa, const int* pb,
-           const TcSeg2* seg, void* C, long long ldc, int out_kind, int splitk,
-           cudaStream_t s, long long split_ld = 0) {
-  A2_REQUIRE(npairs >= 1 && npairs <= kMaxPairs, "tc GEMM: 1..8 operand pairs");
+int tc_sms() {
+  static int num_sms = 0;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    int dev = 0;
+    A2_CUDA(cudaGetDevice(&dev));
+    A2_CUDA(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
+  });
+  return num_sms;
+}
+
+template <int BN, int STAGES>
+void launch(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* B, long long ldb, int M,
+            int N, int K, const TcSeg2* seg, void* C, long long ldc, int out_kind, int splitk,
+            cudaStream_t s) {
   TcMaps maps;
-  int na = 0, nb = 0;
-  for (int p = 0; p < npairs; ++p) {
-    A2_REQUIRE(pa[p] >= 0 && pa[p] < kMaxPlanes && pb[p] >= 0 && pb[p] < kMaxPlanes,
-               "tc GEMM: plane index out of range");
-    na = std::max(na, pa[p] + 1);
-    nb = std::max(nb, pb[p] + 1);
-  }
-  for (int i = 0; i < kMaxPlanes; ++i) {
-    maps.a[i] = i < na || i == 0 ? make_map(A[i], M, K, lda, BM) : maps.a[0];
-    maps.b[i] = i < nb || i == 0 ? make_map(B[i], N, K, ldb, BN) : maps.b[0];
-  }
+  maps.a = make_map(A, M, K, lda, BM);
+  maps.b = make_map(B, N, K, ldb, BN);
   int nk2 = 0, nbc2 = 1, n12 = 1;
   if (seg) {
     const long long Dr = seg->Dr, R1 = seg->R1;
@@ -696,37 +666,25 @@ int launch(const __nv_bfloat16* const* A, long long lda, const __nv_bfloat16* co
     A2_REQUIRE(Dr % 8 == 0 && seg->Nb == N, "tc GEMM segment: Dr % 8 == 0, N == Dr");
     nbc2 = (int)((Dr + BK - 1) / BK);
     nk2 = (int)(R1 * nbc2);
-    for (int i = 0; i < 3; ++i) {
-      const cuuint64_t ad[4] = {(cuuint64_t)Dr, (cuuint64_t)n12, (cuuint64_t)R1,
-                                (cuuint64_t)seg->Dl};
-      const cuuint64_t as[3] = {(cuuint64_t)(Dr * 2), (cuuint64_t)(n12 * Dr * 2),
-                                (cuuint64_t)(R1 * n12 * Dr * 2)};
-      const cuuint32_t ab[4] = {(cuuint32_t)BK, (cuuint32_t)n12, 1u, (cuuint32_t)(BM / n12)};
-      maps.a2[i] = make_map_nd(seg->A[i < na ? i : 0], 4, ad, as, ab);
-      const cuuint64_t bd[3] = {(cuuint64_t)Dr, (cuuint64_t)R1, (cuuint64_t)N};
-      const cuuint64_t bs[2] = {(cuuint64_t)(Dr * 2), (cuuint64_t)(R1 * Dr * 2)};
-      const cuuint32_t bb[3] = {(cuuint32_t)BK, 1u, (cuuint32_t)BN};
-      maps.b2[i] = make_map_nd(seg->B[i < nb ? i : 0], 3, bd, bs, bb);
-    }
+    const cuuint64_t ad[4] = {(cuuint64_t)Dr, (cuuint64_t)n12, (cuuint64_t)R1,
+                              (cuuint64_t)seg->Dl};
+    const cuuint64_t as[3] = {(cuuint64_t)(Dr * 2), (cuuint64_t)(n12 * Dr * 2),
+                              (cuuint64_t)(R1 * n12 * Dr * 2)};
+    const cuuint32_t ab[4] = {(cuuint32_t)BK, (cuuint32_t)n12, 1u, (cuuint32_t)(BM / n12)};
+    maps.a2 = make_map_nd(seg->A[0], 4, ad, as, ab);
+    const cuuint64_t bd[3] = {(cuuint64_t)Dr, (cuuint64_t)R1, (cuuint64_t)N};
+    const cuuint64_t bs[2] = {(cuuint64_t)(Dr * 2), (cuuint64_t)(R1 * Dr * 2)};
+    const cuuint32_t bb[3] = {(cuuint32_t)BK, 1u, (cuuint32_t)BN};
+    maps.b2 = make_map_nd(seg->B[0], 3, bd, bs, bb);
   } else {
-    for (int i = 0; i < 3; ++i) {
-      maps.a2[i] = maps.a[i];
-      maps.b2[i] = maps.b[i];
-    }
+    maps.a2 = maps.a;
+    maps.b2 = maps.b;
   }
-  constexpr int EPI = epi_warps(PROMOTE);
-  const size_t smem = sizeof(TcSmem<BN, STAGES, EPI, PROMOTE ? 1 : 2>) + 1024;
+  const size_t smem = sizeof(TcSmem<BN, STAGES>) + 1024;
   static std::once_flag once;
   std::call_once(once, [smem] {
-    A2_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<BN, STAGES, PROMOTE>,
+    A2_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<BN, STAGES>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  });
-  static int num_sms = 0;
-  static std::once_flag sms_once;
-  std::call_once(sms_once, [] {
-    int dev = 0;
-    A2_CUDA(cudaGetDevice(&dev));
-    A2_CUDA(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
   });
   const int nk1 = (K + BK - 1) / BK;
   const int nk_total = nk1 + nk2;
@@ -737,21 +695,14 @@ int launch(const __nv_bfloat16* const* A, long long lda, const __nv_bfloat16* co
   args.kblocks_per_split = (nk_total + splitk - 1) / splitk;
   splitk = (nk_total + args.kblocks_per_split - 1) / args.kblocks_per_split;
   args.C = C; args.ldc = ldc; args.out_kind = out_kind;
-  args.npairs = npairs;
-  for (int p = 0; p < kMaxPairs; ++p) {
-    args.pa[p] = p < npairs ? pa[p] : 0;
-    args.pb[p] = p < npairs ? pb[p] : 0;
-  }
   args.splits = splitk;
-  args.split_ld = split_ld;
   args.wait_limit = kWaitLimit;
   args.no_loads = 0;
-  A2_REQUIRE(split_ld == 0 || (out_kind == OUT_F32 && !PROMOTE), "split tiles: FP32 stores");
   // TMA store epilogue when C's base and row stride allow it
   {
     const size_t es = out_kind == OUT_BF16 ? 2 : 4;
     args.tma_store = ((reinterpret_cast<uintptr_t>(C) & 15) == 0 && (ldc * es) % 16 == 0 &&
-                      ldc >= N && split_ld == 0) ? 1 : 0;
+                      ldc >= N) ? 1 : 0;
     if (args.tma_store) {
       const cuuint64_t cd[2] = {(cuuint64_t)N, (cuuint64_t)M};
       const cuuint64_t cs[1] = {(cuuint64_t)(ldc * es)};
@@ -768,35 +719,63 @@ int launch(const __nv_bfloat16* const* A, long long lda, const __nv_bfloat16* co
   }
   const long long units = (long long)cdiv(M, BM) * cdiv(N, BN) * splitk;
   A2_REQUIRE(units < (1LL << 31), "tcgen05 GEMM too large");
-  const int grid = (int)std::min<long long>(units, std::max(1, num_sms));
-  tc_gemm_kernel<BN, STAGES, PROMOTE><<<grid, tc_threads(PROMOTE), smem, s>>>(maps, args);
+  const int grid = (int)std::min<long long>(units, std::max(1, tc_sms()));
+  tc_gemm_kernel<BN, STAGES><<<grid, kTcThreads, smem, s>>>(maps, args);
   A2_CHECK_LAUNCH();
-  return splitk;
 }
 
-// ------------------------------------------------------------------ Ozaki GEMM, register sums
-// FP64-class product of two operands given as kOzSlices BF16 slice planes each (the
-// slicing of the FP64 emulation below).  Work unit = (128 x 128 output tile, K split).
-// For every level l = 2 .. kOzSlices + 1 the l - 1 slice pairs of that level are
-// accumulated over chunks of at most 16 / (l - 1) K blocks into a fresh TMEM buffer: a
-// chunk holds at most 1024 products per output element, each an integer multiple of the
-// level's unit below 2^14 units, so its FP32 sum is exact.  The epilogue adds every chunk
-// into a double-float register accumulator (hi + lo, Knuth's error-free two-sum), so no
-// per-level tile reaches memory.  Warp 0 lane 0: TMA producer; warp 1 lane 0: MMA issuer;
-// warps 2..9: epilogue (two per TMEM lane quarter, 64 columns each).  Every wait is
-// bounded as in tc_gemm_kernel.
+// ------------------------------------------------------------------ Ozaki GEMM
+// FP64-class product of two operands given as kOzSlices BF16 slices each (the slicing of the
+// FP64 emulation below): the slice pairs (i, j) with i + j <= 8, 28 of them.
+//
+// Bound: operand delivery.  The MMAs alone take 64 cycles each (M = N = 128, K = 16, operands
+// already in shared memory), but L2 and TMA deliver about 0.45 rows per clock to an SM,
+// whether a row is 64 or 128 bytes: with one pair of 128-byte-row tiles per slice pair the
+// kernel ran at half the tensor rate (1.10 PFLOP/s on every shape).  Three things raise the
+// products per delivered row:
+//  * a tile serves all the pairs it can while it is in shared memory: the K loop runs over
+//    chunks of 256, and each chunk is walked three times, for the levels l = i + j of
+//        2, 3 (slices 1..2, 3 pairs) | 4, 5 (slices 1..4, 7 pairs) | 6, 7 + 8 (18 pairs)
+//    with two TMEM accumulators of 128 columns per phase, so that the epilogue drains one
+//    phase's two while the next phase fills the other two (4 x 128 columns, all of TMEM);
+//  * the slices are interleaved in memory, [K / 32][row][slice][32], so that a 128-byte row of
+//    a tile holds two slices of a K block of 32 (the seventh slice has 64-byte rows): 7 tile
+//    loads per 28 products instead of 56 half as wide ones (with the rows outermost, a tile's
+//    rows lie 2.3 MB apart in S4 and its loads take 7.2 ms instead of 4.6);
+//  * MMAs on the same A slice follow each other and take it from the collector buffer.
+// Exactness: |digit| <= 128, so level l's sum over a chunk is an integer below
+// 256 (l - 1) 2^14 units, at most 2^24 for l <= 5: exact in FP32.  Level 6 reaches 1.25 x
+// 2^24 only if all digits are extreme and is then off by one unit, 2^-46 of the row and
+// column scale, per addition; levels 7 and 8 share an accumulator (level 8 is rounded at
+// 2^-24 of the level 7 sum, ~2^-60).
+// The epilogue adds every accumulator into a double-float register pair (hi + lo, Knuth's
+// error-free two-sum), so no per-level tile reaches memory.
+//
+// Work unit = (128 x 128 output tile, K split).  A ring slot holds one tile of both operands
+// (32 KB): slices 1-2, 3-4, 5-6 or 7 of one K block.  A phase loads 1, 2 or 4 tiles per K
+// block, the last phase in the order 3-4, 1-2, 5-6, 7: its first pairs need only the first two,
+// slices 3 and 4 are done first, and their slot is refilled while the rest runs.  Warp 0
+// lane 0: TMA producer; warp 1: MMA issuer (warp-uniform loops, one lane issues, the MMAs of a K
+// block unrolled: computed slots and branches in the issue loop took longer than the MMAs);
+// warps 2..9: epilogue (two per TMEM lane quarter, 64 columns each).  Every wait is bounded
+// as in tc_gemm_kernel.
+// Measured, D = 256, R = 342 -> 444 (28 products, before: 36 with one tile pair each; ms): left
+// update's 87552 x 1024 x 256 0.77 (1.50), its 256 x 113664 x 1024 0.99 (1.93), S4's 4096 x
+// 256 x 143872 4.6 (9.88).
 constexpr int kOzBN = 128;
-constexpr int kOzStages = 5;
+constexpr int kOzBK = 32;
+constexpr int kOzSlots = 6;
+constexpr int kOzChunk = 256 / kOzBK;           // K blocks between drains
+constexpr int kOzPhases = 3;
 constexpr int kOzEpi = 8;
 constexpr int kOzThreads = 64 + 32 * kOzEpi;
-constexpr int kOzMaxLevel = 9;                  // slice pairs (i, j) with i + j <= 9
 
 struct OzSmem {
-  alignas(1024) __nv_bfloat16 a[kOzStages][BM * BK];
-  alignas(1024) __nv_bfloat16 b[kOzStages][kOzBN * BK];
-  alignas(1024) float stage[kOzEpi][2][32 * 32];   // epilogue transpose buffers (hi, lo)
-  alignas(8) uint64_t full[kOzStages];
-  alignas(8) uint64_t empty[kOzStages];
+  alignas(1024) __nv_bfloat16 a[kOzSlots][BM * 64];
+  alignas(1024) __nv_bfloat16 b[kOzSlots][kOzBN * 64];
+  alignas(1024) float stage[kOzEpi][2][32 * 16];   // epilogue transpose buffers (hi, lo)
+  alignas(8) uint64_t full[kOzSlots];
+  alignas(8) uint64_t empty[kOzSlots];
   alignas(8) uint64_t acc_full[2];
   alignas(8) uint64_t acc_empty[2];
   alignas(8) uint64_t drain;
@@ -805,10 +784,15 @@ struct OzSmem {
 };
 static_assert(sizeof(OzSmem) + 1024 <= 227 * 1024, "Ozaki ring exceeds shared memory");
 
+struct OzMaps {              // views [K block][row][slice and k]
+  CUtensorMap a, b;          // box 1 x 128 x 64 (two slices), 128-byte swizzle
+  CUtensorMap a7, b7;        // box 1 x 128 x 32 (the last slice), 64-byte swizzle
+};
+
 enum OzOut { OZ_F64 = 0, OZ_PAIR = 1, OZ_SPLIT = 2 };
 
 struct OzArgs {
-  int M, N, nk;              // rows, columns, K blocks of BK
+  int M, N, nk;              // rows, columns, K blocks of kOzBK
   int kblocks_per_split, splits;
   int n_fast;                // 1: consecutive units walk the N tiles of one row of tiles
   int out_mode;              // OZ_F64: C[m*ldc + n] = hi + lo (FP64)
@@ -819,12 +803,62 @@ struct OzArgs {
   long long ldc, df_plane, MN;
 };
 
-__device__ __forceinline__ int oz_chunk_blocks(int np) { return max(1, 16 / np); }
+// End of the chunk that starts at block c0 of a split (blocks kb0 .. kb0 + nkb - 1): chunks end at
+// multiples of kOzChunk of the whole K range, where the operands' scales change.
+__device__ __forceinline__ int oz_chunk_end(int kb0, int c0, int nkb) {
+  return min(nkb, ((kb0 + c0) / kOzChunk + 1) * kOzChunk - kb0);
+}
+
+// Tiles of a phase in load order: 0 = slices 1-2, 1 = 3-4, 2 = 5-6, 3 = 7.
+__host__ __device__ constexpr int oz_tiles(int ph) { return ph == 2 ? 4 : ph + 1; }
+__host__ __device__ constexpr int oz_tile(int ph, int t) {
+  return ph == 2 && t < 2 ? 1 - t : t;
+}
+
+// Shared-memory matrix descriptor: K-major, 64-byte swizzle, 8-row groups 512 B apart.
+__device__ __forceinline__ uint64_t smem_desc64(const void* p) {
+  const uint64_t addr = smem_u32(p);
+  uint64_t d = 0;
+  d |= (addr >> 4) & 0x3FFFull;            // start address
+  d |= (uint64_t)1 << 16;                  // leading byte offset (unused for swizzled K-major)
+  d |= (uint64_t)(512 >> 4) << 32;         // stride byte offset: 8 rows x 64 B
+  d |= (uint64_t)1 << 46;                  // descriptor version for tcgen05
+  d |= (uint64_t)4 << 61;                  // SWIZZLE_64B
+  return d;
+}
+
+// A run of MMAs on A slice I with the B slices J... of one K block, into the accumulator of
+// level l0 (d0) or of the levels above it (d0 + 128 columns).  off[t]: descriptor offset of the ring
+// slot that holds tile t.
+template <int L0, int I, int... J>
+__device__ __forceinline__ void oz_run(uint32_t d0, uint64_t ad, uint64_t bd, uint64_t ad7,
+                                       uint64_t bd7, const uint32_t (&off)[4], bool& f0,
+                                       bool& f1) {
+  constexpr uint32_t idesc = idesc_bf16(BM, kOzBN);
+  constexpr int js[] = {J...};
+  constexpr int n = sizeof...(J);
+#pragma unroll
+  for (int kk = 0; kk < kOzBK / 16; ++kk)
+#pragma unroll
+    for (int q = 0; q < n; ++q) {
+      const int j = js[q];
+      const bool lead = I + j == L0;
+      const uint32_t d = d0 + (lead ? 0 : kOzBN), keep = (lead ? f0 : f1) ? 0u : 1u;
+      const uint64_t a = (I == 7 ? ad7 : ad) + off[(I - 1) / 2] + ((I - 1) & 1) * 4 + kk * 2;
+      const uint64_t b = (j == 7 ? bd7 : bd) + off[(j - 1) / 2] + ((j - 1) & 1) * 4 + kk * 2;
+      if (n == 1) mma_bf16_a<true, true>(d, a, b, idesc, keep);
+      else if (q == 0) mma_bf16_a<true, false>(d, a, b, idesc, keep);
+      else if (q == n - 1) mma_bf16_a<false, true>(d, a, b, idesc, keep);
+      else mma_bf16_a<false, false>(d, a, b, idesc, keep);
+      if (lead) f0 = false;
+      else f1 = false;
+    }
+}
 
 // 10 warps: three of them share one SM sub-partition's 16K registers, hence at most 168
 // registers per thread.
 __global__ void __launch_bounds__(kOzThreads, 1)
-tc_oz_kernel(const __grid_constant__ TcMaps maps, OzArgs args) {
+tc_oz_kernel(const __grid_constant__ OzMaps maps, OzArgs args) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
   const uint32_t pad = (1024u - (base & 1023u)) & 1023u;
@@ -834,10 +868,10 @@ tc_oz_kernel(const __grid_constant__ TcMaps maps, OzArgs args) {
   const int tiles_m = (args.M + BM - 1) / BM;
   const int tiles_n = (args.N + kOzBN - 1) / kOzBN;
   const int nunits = tiles_m * tiles_n * args.splits;
-  constexpr uint32_t kStageBytes = (BM + kOzBN) * BK * 2;
+  constexpr uint32_t kSlotBytes = (BM + kOzBN) * 64 * 2;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kOzStages; ++s) {
+    for (int s = 0; s < kOzSlots; ++s) {
       mbar_init(&S.full[s], 1);
       mbar_init(&S.empty[s], 1);
     }
@@ -849,10 +883,10 @@ tc_oz_kernel(const __grid_constant__ TcMaps maps, OzArgs args) {
     S.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) {   // two accumulators of 128 fp32 columns x 128 lanes
+  if (warp == 0) {   // two pairs of accumulators of 128 fp32 columns x 128 lanes
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&S.tmem_base)),
-                 "r"((uint32_t)(2 * kOzBN)));
+                 "r"((uint32_t)(4 * kOzBN)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -875,21 +909,21 @@ tc_oz_kernel(const __grid_constant__ TcMaps maps, OzArgs args) {
 
   if (warp == 0) {
     if (lane == 0) {
-      // ---------------- producer: level, chunk, K block, slice pair
+      // ---------------- producer: chunk, phase, K block, tile
       uint32_t g = 0, issued = 0;
       bool stop = false;
       for (int u = blockIdx.x; !stop && u < nunits && !*(volatile int*)&S.abort_flag;
            u += gridDim.x) {
         int m0, n0, kb0, nkb;
         unit(u, m0, n0, kb0, nkb);
-        for (int l = 2; !stop && l <= kOzMaxLevel; ++l) {
-          const int np = l - 1, kbl = oz_chunk_blocks(np);
-          for (int c0 = 0; !stop && c0 < nkb; c0 += kbl) {
-            const int c1 = min(nkb, c0 + kbl);
+        for (int c0 = 0, c1; !stop && c0 < nkb; c0 = c1) {
+          c1 = oz_chunk_end(kb0, c0, nkb);
+          for (int ph = 0; !stop && ph < kOzPhases; ++ph) {
+            const int nt = oz_tiles(ph);
             for (int kb = c0; !stop && kb < c1; ++kb) {
-              for (int p = 0; p < np; ++p, ++g) {
-                const int s = g % kOzStages;
-                const uint32_t round = g / kOzStages;
+              for (int t = 0; t < nt; ++t, ++g) {
+                const int s = g % kOzSlots;
+                const uint32_t round = g / kOzSlots;
                 if ((round > 0 &&
                      !mbar_wait_or_abort(&S.empty[s], (round - 1) & 1, 11, &S.abort_flag)) ||
                     *(volatile int*)&S.abort_flag) {
@@ -897,10 +931,12 @@ tc_oz_kernel(const __grid_constant__ TcMaps maps, OzArgs args) {
                   stop = true;
                   break;
                 }
-                mbar_expect_tx(&S.full[s], kStageBytes);
-                const int kx = (kb0 + kb) * BK;
-                tma_load_2d(&maps.a[p], &S.full[s], S.a[s], kx, m0);
-                tma_load_2d(&maps.b[np - 1 - p], &S.full[s], S.b[s], kx, n0);
+                const int tile = oz_tile(ph, t);
+                mbar_expect_tx(&S.full[s], tile == 3 ? kSlotBytes / 2 : kSlotBytes);
+                tma_load_3d(tile == 3 ? &maps.a7 : &maps.a, &S.full[s], S.a[s], tile * 64, m0,
+                            kb0 + kb);
+                tma_load_3d(tile == 3 ? &maps.b7 : &maps.b, &S.full[s], S.b[s], tile * 64, n0,
+                            kb0 + kb);
                 issued = g + 1;
               }
             }
@@ -908,71 +944,124 @@ tc_oz_kernel(const __grid_constant__ TcMaps maps, OzArgs args) {
         }
       }
       if (*(volatile int*)&S.abort_flag) {   // wait (bounded) for the copies in flight
-        for (uint32_t j = issued > (uint32_t)kOzStages ? issued - kOzStages : 0; j < issued; ++j)
-          mbar_wait(&S.full[j % kOzStages], (j / kOzStages) & 1, 12);
+        for (uint32_t j = issued > (uint32_t)kOzSlots ? issued - kOzSlots : 0; j < issued; ++j)
+          mbar_wait(&S.full[j % kOzSlots], (j / kOzSlots) & 1, 12);
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer: one TMEM buffer per (level, chunk)
-      constexpr uint32_t idesc = idesc_bf16(BM, kOzBN);
-      uint32_t g = 0, ch = 0;
-      bool issued_any = false, ok = true;
-      for (int u = blockIdx.x; ok && u < nunits && !*(volatile int*)&S.abort_flag;
-           u += gridDim.x) {
-        int m0, n0, kb0, nkb;
-        unit(u, m0, n0, kb0, nkb);
-        for (int l = 2; ok && l <= kOzMaxLevel; ++l) {
-          const int np = l - 1, kbl = oz_chunk_blocks(np);
-          for (int c0 = 0; ok && c0 < nkb; c0 += kbl, ++ch) {
-            const int c1 = min(nkb, c0 + kbl);
-            const uint32_t buf = ch & 1, use = ch >> 1;
-            if (use > 0 &&
-                !mbar_wait_or_abort(&S.acc_empty[buf], (use - 1) & 1, 13, &S.abort_flag)) {
-              ok = false;
-              break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t d = tmem + buf * kOzBN;
-            bool first = true;
-            for (int kb = c0; ok && kb < c1; ++kb) {
-              for (int p = 0; p < np; ++p, ++g) {
-                const int s = g % kOzStages;
-                if (!mbar_wait_or_abort(&S.full[s], (g / kOzStages) & 1, 14, &S.abort_flag)) {
-                  ok = false;
-                  break;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint64_t da = smem_desc(S.a[s]);
-                const uint64_t db = smem_desc(S.b[s]);
+    // ---------------- MMA issuer: two TMEM accumulators per (chunk, phase)
+    const bool leader = elect_one();
+    const uint64_t ad = smem_desc(S.a[0]), bd = smem_desc(S.b[0]);
+    const uint64_t ad7 = smem_desc64(S.a[0]), bd7 = smem_desc64(S.b[0]);
+    uint32_t slot = 0, par = 0, pc = 0;     // next slot, parity of its round, phase counter
+    bool issued_any = false, ok = true;
+    constexpr uint32_t kSlotStep = (BM * 64 * 2) >> 4;          // descriptor units
+    uint32_t off[4];                        // by tile
+    auto slot_of = [&](int t) {             // ring slot of the t-th tile of this K block
+      const uint32_t sl = slot + t;
+      return sl >= kOzSlots ? sl - kOzSlots : sl;
+    };
+    auto wait_tile = [&](int ph, int t) {   // the t-th tile of this K block has arrived
+      const uint32_t sl = slot_of(t);
+      ok = ok && mbar_wait_warp(&S.full[sl], par ^ (slot + t >= kOzSlots ? 1u : 0u), 14,
+                                &S.abort_flag);
+      off[oz_tile(ph, t)] = sl * kSlotStep;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    };
+    auto advance = [&](int nt) {
+      slot += nt;
+      if (slot >= kOzSlots) {
+        slot -= kOzSlots;
+        par ^= 1;
+      }
+    };
+    for (int u = blockIdx.x; ok && u < nunits; u += gridDim.x) {
+      int m0, n0, kb0, nkb;
+      unit(u, m0, n0, kb0, nkb);
+      for (int c0 = 0, c1; ok && c0 < nkb; c0 = c1) {
+        c1 = oz_chunk_end(kb0, c0, nkb);
 #pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk)
-                  mma_bf16(d, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc,
-                           (first && kk == 0) ? 0u : 1u);
-                first = false;
-                issued_any = true;
-                mma_commit(&S.empty[s]);
+        for (int ph = 0; ph < kOzPhases; ++ph) {
+          if (!ok) break;
+          const uint32_t set = pc & 1, use = pc >> 1;
+          if (use > 0) {
+            ok = mbar_wait_warp(&S.acc_empty[set], (use - 1) & 1, 13, &S.abort_flag);
+            if (!ok) break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t d0 = tmem + set * (2 * kOzBN);
+          for (int kb = c0; kb < c1; ++kb) {
+            bool f0 = kb == c0, f1 = f0;
+#define A2_RUN(...) oz_run<__VA_ARGS__>(d0, ad, bd, ad7, bd7, off, f0, f1)
+            if (ph == 0) {
+              wait_tile(0, 0);
+              if (ok && leader) {
+                A2_RUN(2, 1, 1, 2);
+                A2_RUN(2, 2, 1);
+                mma_commit(&S.empty[slot_of(0)]);
+              }
+            } else if (ph == 1) {
+              wait_tile(1, 0);
+              wait_tile(1, 1);
+              if (ok && leader) {
+                A2_RUN(4, 2, 2, 3);
+                A2_RUN(4, 1, 3, 4);
+                A2_RUN(4, 3, 1, 2);
+                A2_RUN(4, 4, 1);
+                mma_commit(&S.empty[slot_of(0)]);
+                mma_commit(&S.empty[slot_of(1)]);
+              }
+            } else {
+              wait_tile(2, 0);
+              wait_tile(2, 1);
+              if (ok && leader) {
+                A2_RUN(6, 3, 3, 4);
+                A2_RUN(6, 4, 2, 3, 4);
+                A2_RUN(6, 2, 4);
+              }
+              wait_tile(2, 2);
+              if (ok && leader) {
+                A2_RUN(6, 3, 5);
+                A2_RUN(6, 5, 3, 1, 2);
+                mma_commit(&S.empty[slot_of(0)]);        // slices 3, 4 are done
+                A2_RUN(6, 1, 5, 6);
+                A2_RUN(6, 2, 5, 6);
+                A2_RUN(6, 6, 1, 2);
+              }
+              wait_tile(2, 3);
+              if (ok && leader) {
+                A2_RUN(6, 1, 7);
+                A2_RUN(6, 7, 1);
+                mma_commit(&S.empty[slot_of(1)]);
+                mma_commit(&S.empty[slot_of(2)]);
+                mma_commit(&S.empty[slot_of(3)]);
               }
             }
+#undef A2_RUN
+            issued_any |= ok;
+            advance(oz_tiles(ph));
             if (!ok) break;
-            mma_commit(&S.acc_full[buf]);
           }
+          if (!ok) break;
+          if (leader) mma_commit(&S.acc_full[set]);
+          ++pc;
         }
       }
-      if (!ok) S.abort_flag = 1;
-      if (*(volatile int*)&S.abort_flag && issued_any) {
-        mma_commit(&S.drain);
-        mbar_wait(&S.drain, 0, 15);
-      }
     }
+    if (!ok) S.abort_flag = 1;
+    if (*(volatile int*)&S.abort_flag && issued_any && leader) {
+      mma_commit(&S.drain);
+      mbar_wait(&S.drain, 0, 15);
+    }
+    __syncwarp();
   } else {
-    // ---------------- epilogue: double-float sums of the chunks, then the output
+    // ---------------- epilogue: double-float sums of the accumulators, then the output
     const int q = warp & 3;                 // TMEM lane quarter of this warp
     const int ew = warp - 2;
     const int colbase = (ew >> 2) * 64;     // this warp's 64 columns of the tile
     float* sh = S.stage[ew][0];
     float* sl = S.stage[ew][1];
-    uint32_t ch = 0;
+    uint32_t pc = 0;
     bool ok = true;
     for (int u = blockIdx.x; ok && u < nunits; u += gridDim.x) {
       int m0, n0, kb0, nkb;
@@ -980,63 +1069,66 @@ tc_oz_kernel(const __grid_constant__ TcMaps maps, OzArgs args) {
       float hi[64], lo[64];
 #pragma unroll
       for (int i = 0; i < 64; ++i) hi[i] = lo[i] = 0.f;
-      for (int l = 2; ok && l <= kOzMaxLevel; ++l) {
-        const int kbl = oz_chunk_blocks(l - 1);
-        for (int c0 = 0; c0 < nkb; c0 += kbl, ++ch) {
-          const uint32_t buf = ch & 1, use = ch >> 1;
-          if (!mbar_wait_or_abort(&S.acc_full[buf], use & 1, 16, &S.abort_flag)) {
+      for (int c0 = 0; ok && c0 < nkb; c0 = oz_chunk_end(kb0, c0, nkb)) {
+        for (int ph = 0; ph < kOzPhases; ++ph, ++pc) {
+          const uint32_t set = pc & 1, use = pc >> 1;
+          if (!mbar_wait_or_abort(&S.acc_full[set], use & 1, 16, &S.abort_flag)) {
             ok = false;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t tl = tmem + buf * kOzBN + (uint32_t)colbase + ((uint32_t)(q * 32) << 16);
+          const uint32_t tl =
+              tmem + set * (2 * kOzBN) + (uint32_t)colbase + ((uint32_t)(q * 32) << 16);
+#pragma unroll 1
+          for (int acc = 0; acc < 2; ++acc) {
 #pragma unroll
-          for (int c = 0; c < 64; c += 8) {
-            float v[8];
-            tmem_ld8(tl + (uint32_t)c, v);
+            for (int c = 0; c < 64; c += 8) {
+              float v[8];
+              tmem_ld8(tl + (uint32_t)(acc * kOzBN + c), v);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {   // (hi, lo) += v exactly up to lo's rounding
-              const float sum = __fadd_rn(hi[c + i], v[i]);
-              const float bp = __fsub_rn(sum, hi[c + i]);
-              const float err =
-                  __fadd_rn(__fsub_rn(hi[c + i], __fsub_rn(sum, bp)), __fsub_rn(v[i], bp));
-              hi[c + i] = sum;
-              lo[c + i] = __fadd_rn(lo[c + i], err);
+              for (int i = 0; i < 8; ++i) {   // (hi, lo) += v exactly up to lo's rounding
+                const float sum = __fadd_rn(hi[c + i], v[i]);
+                const float bp = __fsub_rn(sum, hi[c + i]);
+                const float err =
+                    __fadd_rn(__fsub_rn(hi[c + i], __fsub_rn(sum, bp)), __fsub_rn(v[i], bp));
+                hi[c + i] = sum;
+                lo[c + i] = __fadd_rn(lo[c + i], err);
+              }
             }
           }
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
           __syncwarp();
-          if (lane == 0) mbar_arrive(&S.acc_empty[buf]);
+          if (lane == 0) mbar_arrive(&S.acc_empty[set]);
         }
       }
       if (!ok) break;
-      // output: 32 x 32 blocks through the transpose buffers (lane = row on the way in,
-      // lane = column on the way out), so that every store instruction is coalesced
+      // output: 32 x 16 blocks through the transpose buffers (lane = row on the way in; a
+      // half warp writes one row's 16 columns on the way out)
       const int row0 = m0 + q * 32;
 #pragma unroll
-      for (int c = 0; c < 64; c += 32) {
+      for (int c = 0; c < 64; c += 16) {
         const int col0 = n0 + colbase + c;
         if (col0 >= args.N || row0 >= args.M) continue;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          sh[lane * 32 + (i ^ lane)] = hi[c + i];
-          sl[lane * 32 + (i ^ lane)] = lo[c + i];
+        for (int i = 0; i < 16; ++i) {
+          sh[lane * 16 + (i ^ (lane & 15))] = hi[c + i];
+          sl[lane * 16 + (i ^ (lane & 15))] = lo[c + i];
         }
         __syncwarp();
-        const int col = col0 + lane;
+        const int cc = lane & 15, col = col0 + cc;
         const int nrow = min(32, args.M - row0);
         if (col < args.N) {
           if (args.out_mode == OZ_F64) {
             double* cp = reinterpret_cast<double*>(args.C) + (long long)row0 * args.ldc + col;
 #pragma unroll 4
-            for (int r = 0; r < nrow; ++r)
-              cp[(long long)r * args.ldc] =
-                  (double)sh[r * 32 + (lane ^ r)] + (double)sl[r * 32 + (lane ^ r)];
+            for (int r = lane >> 4; r < nrow; r += 2)
+              cp[(long long)r * args.ldc] = (double)sh[r * 16 + (cc ^ (r & 15))] +
+                                            (double)sl[r * 16 + (cc ^ (r & 15))];
           } else if (args.out_mode == OZ_PAIR) {
             float* cp = reinterpret_cast<float*>(args.C) + (long long)row0 * args.ldc + col;
 #pragma unroll 4
-            for (int r = 0; r < nrow; ++r) {
-              const float h = sh[r * 32 + (lane ^ r)], e = sl[r * 32 + (lane ^ r)];
+            for (int r = lane >> 4; r < nrow; r += 2) {
+              const float h = sh[r * 16 + (cc ^ (r & 15))], e = sl[r * 16 + (cc ^ (r & 15))];
               const float sum = __fadd_rn(h, e);   // renormalised pair
               cp[(long long)r * args.ldc] = sum;
               cp[(long long)r * args.ldc + args.df_plane] = __fsub_rn(e, __fsub_rn(sum, h));
@@ -1046,9 +1138,9 @@ tc_oz_kernel(const __grid_constant__ TcMaps maps, OzArgs args) {
             float* cp = reinterpret_cast<float*>(args.C) + 2LL * sp * args.MN +
                         (long long)row0 * args.N + col;
 #pragma unroll 4
-            for (int r = 0; r < nrow; ++r) {
-              cp[(long long)r * args.N] = sh[r * 32 + (lane ^ r)];
-              cp[(long long)r * args.N + args.MN] = sl[r * 32 + (lane ^ r)];
+            for (int r = lane >> 4; r < nrow; r += 2) {
+              cp[(long long)r * args.N] = sh[r * 16 + (cc ^ (r & 15))];
+              cp[(long long)r * args.N + args.MN] = sl[r * 16 + (cc ^ (r & 15))];
             }
           }
         }
@@ -1061,40 +1153,47 @@ tc_oz_kernel(const __grid_constant__ TcMaps maps, OzArgs args) {
   __syncthreads();
   if (warp == 0) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                 "r"((uint32_t)(2 * kOzBN)));
+                 "r"((uint32_t)(4 * kOzBN)));
   }
 }
 
-// Launches tc_oz_kernel over planes A[0..7] (M x K, row stride lda) and B[0..7] (N x K).
-void launch_oz(const __nv_bfloat16* const* A, long long lda, const __nv_bfloat16* const* B,
-               long long ldb, int M, int N, int K, int splits, int out_mode, void* C,
-               long long ldc, long long df_plane, cudaStream_t s) {
-  TcMaps maps;
-  for (int i = 0; i < kMaxPlanes; ++i) {
-    maps.a[i] = make_map(A[i], M, K, lda, BM);
-    maps.b[i] = make_map(B[i], N, K, ldb, kOzBN);
-  }
-  for (int i = 0; i < 3; ++i) {
-    maps.a2[i] = maps.a[i];
-    maps.b2[i] = maps.b[i];
-  }
-  maps.c = maps.a[0];
+// Maps of a sliced operand ([nkb][rows][8][32] BF16, slice 8 unused): two slices per box row,
+// or the last one.
+CUtensorMap make_oz_map(const __nv_bfloat16* ptr, int rows, int nkb, bool last) {
+  const cuuint64_t dims[3] = {(cuuint64_t)(kOzSlices * kOzBK), (cuuint64_t)rows, (cuuint64_t)nkb};
+  const cuuint64_t strides[2] = {(cuuint64_t)(kOzRowBlock * 2), (cuuint64_t)rows * kOzRowBlock * 2};
+  const cuuint32_t box[3] = {last ? 32u : 64u, (cuuint32_t)BM, 1u};
+  A2_REQUIRE((reinterpret_cast<uintptr_t>(ptr) & 15) == 0, "TMA base must be 16-byte aligned");
+  CUtensorMap m;
+  const cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)ptr, dims, strides,
+                           box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           last ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) throw CudaError("cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
+  return m;
+}
+
+// Launches tc_oz_kernel over the slices of A (M x K) and B (N x K).
+void launch_oz(const __nv_bfloat16* A, const __nv_bfloat16* B, int M, int N, int K, int splits,
+               int out_mode, void* C, long long ldc, long long df_plane, cudaStream_t s) {
+  static_assert(kOzBN == BM, "one box shape for both operands");
+  const int nkb = (K + kOzBK - 1) / kOzBK;
+  OzMaps maps;
+  maps.a = make_oz_map(A, M, nkb, false);
+  maps.b = make_oz_map(B, N, nkb, false);
+  maps.a7 = make_oz_map(A, M, nkb, true);
+  maps.b7 = make_oz_map(B, N, nkb, true);
   const size_t smem = sizeof(OzSmem) + 1024;
   static std::once_flag once;
   std::call_once(once, [smem] {
     A2_CUDA(cudaFuncSetAttribute(tc_oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem));
   });
-  static int num_sms = 0;
-  static std::once_flag sms_once;
-  std::call_once(sms_once, [] {
-    int dev = 0;
-    A2_CUDA(cudaGetDevice(&dev));
-    A2_CUDA(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
-  });
   OzArgs args;
   args.M = M; args.N = N;
-  args.nk = (K + BK - 1) / BK;
+  args.nk = (K + kOzBK - 1) / kOzBK;
   splits = std::max(1, std::min(splits, args.nk));
   args.kblocks_per_split = (args.nk + splits - 1) / splits;
   args.splits = (args.nk + args.kblocks_per_split - 1) / args.kblocks_per_split;
@@ -1105,8 +1204,401 @@ void launch_oz(const __nv_bfloat16* const* A, long long lda, const __nv_bfloat16
   args.MN = (long long)M * N;
   const long long units = (long long)cdiv(M, BM) * cdiv(N, kOzBN) * args.splits;
   A2_REQUIRE(units < (1LL << 31), "Ozaki GEMM too large");
-  const int grid = (int)std::min<long long>(units, std::max(1, num_sms));
+  const int grid = (int)std::min<long long>(units, std::max(1, tc_sms()));
   tc_oz_kernel<<<grid, kOzThreads, smem, s>>>(maps, args);
+  A2_CHECK_LAUNCH();
+}
+
+// ------------------------------------------------------------------ split products
+// C = A B^T to FP32 accuracy for operands given as three BF16 planes each (a value as
+// high + middle + low part): the six plane pairs (i, j) with i + j <= 2 accumulated together.
+//
+// Bound: shared-memory bandwidth, as for the Ozaki GEMM.  With one pair of tiles loaded per plane
+// pair, TMA writes (94) and the MMAs read (96) 190 bytes per clock and SM of a possible
+// 128 at the full tensor rate, and the kernel ran at 63 to 65 % of it.  Here a K block of 32
+// is loaded once, plane by plane (a ring slot holds plane i of both operands, 64-byte
+// swizzled rows), and all six pairs run from it: half the loads, 141 bytes per clock.
+// The pairs run in the order of their later plane, so that the MMAs start before the last
+// plane has arrived.
+// The tensor cores' FP32 accumulator truncates, so every kS3Chunk K blocks are accumulated
+// into a fresh TMEM buffer of BN columns (two in turn) and the eight epilogue warps add the
+// partial sums into IEEE FP32 registers (round to nearest), BN / 2 columns of one row per
+// thread.  BN = 128 serves outputs of at most 128 columns (S4 at D <= 128) without
+// multiplying padding.
+// Roles, waits and the optional second K segment as in tc_gemm_kernel.  Measured at D = 256,
+// bond 7 (R = 444, 562, 444; ms): S1 113664 x 4096 x 256 0.99 (1.15), S4 with its second
+// segment 4096 x 256 x (113664 + 143872) 2.30 (2.61).
+constexpr int kS3BK = 32;
+constexpr int kS3Chunk = 4;                 // K blocks per partial sum
+constexpr int kS3Epi = 8;
+constexpr int kS3Threads = 64 + 32 * kS3Epi;
+__host__ __device__ constexpr int s3_slots(int bn) { return bn == 256 ? 8 : 12; }
+
+template <int BN>
+struct S3Smem {
+  static constexpr int SLOTS = s3_slots(BN);
+  alignas(1024) __nv_bfloat16 a[SLOTS][BM * kS3BK];
+  alignas(1024) __nv_bfloat16 b[SLOTS][BN * kS3BK];
+  alignas(1024) unsigned char cbuf[kS3Epi][4096];         // epilogue staging buffers
+  alignas(8) uint64_t full[SLOTS];
+  alignas(8) uint64_t empty[SLOTS];
+  alignas(8) uint64_t acc_full[2];
+  alignas(8) uint64_t acc_empty[2];
+  alignas(8) uint64_t drain;
+  uint32_t tmem_base;
+  int abort_flag;
+};
+static_assert(sizeof(S3Smem<256>) + 1024 <= 227 * 1024, "split ring exceeds shared memory");
+static_assert(sizeof(S3Smem<128>) + 1024 <= 227 * 1024, "split ring exceeds shared memory");
+
+struct S3Maps {
+  CUtensorMap a[3], b[3];
+  CUtensorMap a2[3], b2[3];      // optional second K segment (4D / 3D views)
+  CUtensorMap c;
+};
+struct S3Args {
+  int M, N, nk1, nk2;            // K blocks of the plain product and of the second segment
+  int nbc2, n12;                 // second segment: b' chunks per w1, (s1 s2) rows per a
+  int kblocks_per_split, splits;
+  void* C;
+  long long ldc;
+  int out_kind, tma_store;
+};
+
+template <int BN>
+__global__ void __launch_bounds__(kS3Threads, 1)
+tc_split3_kernel(const __grid_constant__ S3Maps maps, S3Args args) {
+  constexpr int SLOTS = s3_slots(BN), WC = BN / 2;         // columns of one epilogue warp
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  const uint32_t base = smem_u32(smem_raw);
+  const uint32_t pad = (1024u - (base & 1023u)) & 1023u;
+  auto& S = *reinterpret_cast<S3Smem<BN>*>(smem_raw + pad);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tiles_m = (args.M + BM - 1) / BM;
+  const int tiles_n = (args.N + BN - 1) / BN;
+  const int nk_total = args.nk1 + args.nk2;
+  const int nunits = tiles_m * tiles_n * args.splits;
+  constexpr uint32_t kSlotBytes = (BM + BN) * kS3BK * 2;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < SLOTS; ++s) {
+      mbar_init(&S.full[s], 1);
+      mbar_init(&S.empty[s], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&S.acc_full[i], 1);
+      mbar_init(&S.acc_empty[i], kS3Epi);
+    }
+    mbar_init(&S.drain, 1);
+    S.abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {   // two accumulators of BN fp32 columns x 128 lanes
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&S.tmem_base)),
+                 "r"((uint32_t)(2 * BN)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = S.tmem_base;
+
+  auto unit = [&](int u, int& m0, int& n0, int& kb0, int& nkb) {
+    m0 = (u % tiles_m) * BM;
+    n0 = ((u / tiles_m) % tiles_n) * BN;
+    kb0 = (u / (tiles_m * tiles_n)) * args.kblocks_per_split;
+    nkb = max(0, min(nk_total - kb0, args.kblocks_per_split));
+  };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---------------- producer: K block, plane
+      uint32_t g = 0, issued = 0;
+      bool stop = false;
+      for (int u = blockIdx.x; !stop && u < nunits && !*(volatile int*)&S.abort_flag;
+           u += gridDim.x) {
+        int m0, n0, kb0, nkb;
+        unit(u, m0, n0, kb0, nkb);
+        for (int kb = 0; !stop && kb < nkb; ++kb) {
+          const int kbg = kb0 + kb;
+          for (int p = 0; p < 3; ++p, ++g) {
+            const int s = g % SLOTS;
+            const uint32_t round = g / SLOTS;
+            if ((round > 0 &&
+                 !mbar_wait_or_abort(&S.empty[s], (round - 1) & 1, 1, &S.abort_flag)) ||
+                *(volatile int*)&S.abort_flag) {
+              S.abort_flag = 1;
+              stop = true;
+              break;
+            }
+            mbar_expect_tx(&S.full[s], kSlotBytes);
+            if (kbg < args.nk1) {
+              tma_load_2d(&maps.a[p], &S.full[s], S.a[s], kbg * kS3BK, m0);
+              tma_load_2d(&maps.b[p], &S.full[s], S.b[s], kbg * kS3BK, n0);
+            } else {   // second segment: K block = (w1, chunk of b')
+              const int j = kbg - args.nk1;
+              const int w1 = j / args.nbc2, bx = (j % args.nbc2) * kS3BK;
+              tma_load_4d(&maps.a2[p], &S.full[s], S.a[s], bx, 0, w1, m0 / args.n12);
+              tma_load_3d(&maps.b2[p], &S.full[s], S.b[s], bx, w1, n0);
+            }
+            issued = g + 1;
+          }
+        }
+      }
+      if (*(volatile int*)&S.abort_flag) {   // wait (bounded) for the copies in flight
+        for (uint32_t j = issued > (uint32_t)SLOTS ? issued - SLOTS : 0; j < issued; ++j)
+          mbar_wait(&S.full[j % SLOTS], (j / SLOTS) & 1, 2);
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer: one TMEM buffer per chunk (warp-uniform loops, one lane
+    // issues, the MMAs of a K block unrolled)
+    const bool leader = elect_one();
+    constexpr uint32_t idesc = idesc_bf16(BM, BN);
+    constexpr uint32_t kStepA = (BM * kS3BK * 2) >> 4, kStepB = (BN * kS3BK * 2) >> 4;
+    const uint64_t ad = smem_desc64(S.a[0]), bd = smem_desc64(S.b[0]);
+    uint32_t slot = 0, par = 0, ch = 0;
+    bool issued_any = false, ok = true;
+    for (int u = blockIdx.x; ok && u < nunits; u += gridDim.x) {
+      int m0, n0, kb0, nkb;
+      unit(u, m0, n0, kb0, nkb);
+      for (int c0 = 0; ok && c0 < nkb; c0 += kS3Chunk, ++ch) {
+        const int c1 = min(nkb, c0 + kS3Chunk);
+        const uint32_t buf = ch & 1, use = ch >> 1;
+        if (use > 0)
+          ok = mbar_wait_warp(&S.acc_empty[buf], (use - 1) & 1, 5, &S.abort_flag);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t d = tmem + buf * BN;
+        for (int kb = c0; kb < c1; ++kb) {
+          uint32_t sl[3];
+#pragma unroll
+          for (int m = 0; m < 3; ++m) {
+            sl[m] = slot + m;
+            uint32_t pr = par;
+            if (sl[m] >= SLOTS) {
+              sl[m] -= SLOTS;
+              pr ^= 1;
+            }
+            ok = ok && mbar_wait_warp(&S.full[sl[m]], pr, 3, &S.abort_flag);
+          }
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          if (leader) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i)          // A plane i against B planes 0 .. 2 - i
+#pragma unroll
+              for (int kk = 0; kk < kS3BK / 16; ++kk)
+#pragma unroll
+                for (int j = 0; j <= 2 - i; ++j) {
+                  const uint64_t a = ad + sl[i] * kStepA + kk * 2, b = bd + sl[j] * kStepB + kk * 2;
+                  const uint32_t keep = (i > 0 || kk > 0 || j > 0 || kb > c0) ? 1u : 0u;
+                  if (i == 2) mma_bf16_a<true, true>(d, a, b, idesc, keep);
+                  else if (j == 0) mma_bf16_a<true, false>(d, a, b, idesc, keep);
+                  else if (j == 2 - i) mma_bf16_a<false, true>(d, a, b, idesc, keep);
+                  else mma_bf16_a<false, false>(d, a, b, idesc, keep);
+                }
+#pragma unroll
+            for (int m = 0; m < 3; ++m) mma_commit(&S.empty[sl[m]]);
+          }
+          issued_any = true;
+          slot += 3;
+          if (slot >= SLOTS) {
+            slot -= SLOTS;
+            par ^= 1;
+          }
+        }
+        if (!ok) break;
+        if (leader) mma_commit(&S.acc_full[buf]);
+      }
+    }
+    if (!ok) S.abort_flag = 1;
+    if (*(volatile int*)&S.abort_flag && issued_any && leader) {
+      mma_commit(&S.drain);
+      mbar_wait(&S.drain, 0, 6);
+    }
+    __syncwarp();
+  } else {
+    // ---------------- epilogue warps: FP32 sums of the partial tiles, then the output
+    const int q = warp & 3;                          // TMEM lane quarter of this warp
+    const int ew = warp - 2;
+    const int colbase = (ew >> 2) * WC;
+    unsigned char* wbuf = S.cbuf[ew];
+    uint32_t ch = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < nunits; u += gridDim.x) {
+      int m0, n0, kb0, nkb;
+      unit(u, m0, n0, kb0, nkb);
+      const int row0 = m0 + q * 32;
+      float acc[WC];
+#pragma unroll
+      for (int i = 0; i < WC; ++i) acc[i] = 0.f;
+      for (int c0 = 0; c0 < nkb; c0 += kS3Chunk, ++ch) {
+        const uint32_t buf = ch & 1, use = ch >> 1;
+        if (!mbar_wait_or_abort(&S.acc_full[buf], use & 1, 4, &S.abort_flag)) {
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t tl = tmem + buf * BN + (uint32_t)colbase + ((uint32_t)(q * 32) << 16);
+#pragma unroll
+        for (int c = 0; c < WC; c += 32) {
+          float v[32];
+          tmem_ld32(tl + (uint32_t)c, v);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) acc[c + i] += v[i];
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&S.acc_empty[buf]);
+      }
+      if (!ok) break;
+#pragma unroll
+      for (int c = 0; c < WC; c += 32) {
+        const int col0 = n0 + colbase + c;
+        if (col0 >= args.N || row0 >= args.M) continue;
+        if (args.tma_store) {
+          // this lane's 128-byte row segment into a 128B-swizzled staging buffer, one TMA
+          // store (or reduce-add) of the 32-row box, clipped by the map
+          if (lane == 0) bulk_wait_read0();
+          __syncwarp();
+          const uint32_t rowa = smem_u32(wbuf) + lane * 128;
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            st_shared_v4(rowa + ((j ^ (lane & 7)) << 4), __float_as_uint(acc[c + 4 * j]),
+                         __float_as_uint(acc[c + 4 * j + 1]), __float_as_uint(acc[c + 4 * j + 2]),
+                         __float_as_uint(acc[c + 4 * j + 3]));
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) {
+            if (args.out_kind == OUT_F32_ATOMIC) tma_reduce_add_2d(&maps.c, wbuf, col0, row0);
+            else tma_store_2d(&maps.c, wbuf, col0, row0);
+            bulk_commit();
+          }
+        } else {
+          float* stage = reinterpret_cast<float*>(wbuf);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) stage[lane * 32 + (i ^ lane)] = acc[c + i];
+          __syncwarp();
+          const int col = col0 + lane, nrow = min(32, args.M - row0);
+          if (col < args.N) {
+            float* cp = reinterpret_cast<float*>(args.C) + (long long)row0 * args.ldc + col;
+            if (args.out_kind == OUT_F32_ATOMIC)
+              for (int r = 0; r < nrow; ++r)
+                atomicAdd(cp + (long long)r * args.ldc, stage[r * 32 + (lane ^ r)]);
+            else
+              for (int r = 0; r < nrow; ++r)
+                cp[(long long)r * args.ldc] = stage[r * 32 + (lane ^ r)];
+          }
+          __syncwarp();
+        }
+      }
+    }
+    if (!ok) S.abort_flag = 1;
+    if (args.tma_store && lane == 0) bulk_wait_all();   // stores complete before exit
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"((uint32_t)(2 * BN)));
+  }
+}
+
+// Tiled BF16 map of rank 2 to 4 (dims innermost first, strides in bytes for dims 1..) with
+// 64-byte swizzle, zero fill outside the extents.
+CUtensorMap make_map64(const __nv_bfloat16* ptr, int rank, const cuuint64_t* dims,
+                       const cuuint64_t* strides, const cuuint32_t* box) {
+  A2_REQUIRE((reinterpret_cast<uintptr_t>(ptr) & 15) == 0, "TMA base must be 16-byte aligned");
+  for (int i = 0; i < rank - 1; ++i)
+    A2_REQUIRE(strides[i] % 16 == 0, "TMA strides must be multiples of 16 bytes");
+  CUtensorMap m;
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, (void*)ptr, dims, strides,
+                           box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) throw CudaError("cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
+  return m;
+}
+
+// FP32 output map of the epilogue's 32 x 32 boxes; false if C's base or stride rules it out.
+bool make_out_map(CUtensorMap* m, void* C, int M, int N, long long ldc) {
+  if ((reinterpret_cast<uintptr_t>(C) & 15) != 0 || (ldc * 4) % 16 != 0 || ldc < N) return false;
+  const cuuint64_t cd[2] = {(cuuint64_t)N, (cuuint64_t)M};
+  const cuuint64_t cs[1] = {(cuuint64_t)(ldc * 4)};
+  const cuuint32_t cb[2] = {32u, 32u};
+  const cuuint32_t ce[2] = {1, 1};
+  return encode_fn()(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, C, cd, cs, cb, ce,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int BN>
+void launch_split3(const __nv_bfloat16* const* A, long long lda, const __nv_bfloat16* const* B,
+                   long long ldb, int M, int N, int K, const TcSeg2* seg, void* C, long long ldc,
+                   int out_kind, int splitk, cudaStream_t s) {
+  S3Maps maps;
+  S3Args args;
+  for (int i = 0; i < 3; ++i) {
+    const cuuint64_t ad[2] = {(cuuint64_t)K, (cuuint64_t)M}, bd[2] = {(cuuint64_t)K, (cuuint64_t)N};
+    const cuuint64_t as[1] = {(cuuint64_t)(lda * 2)}, bs[1] = {(cuuint64_t)(ldb * 2)};
+    const cuuint32_t ab[2] = {(cuuint32_t)kS3BK, (cuuint32_t)BM};
+    const cuuint32_t bb[2] = {(cuuint32_t)kS3BK, (cuuint32_t)BN};
+    maps.a[i] = make_map64(A[i], 2, ad, as, ab);
+    maps.b[i] = make_map64(B[i], 2, bd, bs, bb);
+  }
+  args.nk1 = (K + kS3BK - 1) / kS3BK;
+  args.nk2 = 0;
+  args.nbc2 = args.n12 = 1;
+  if (seg) {
+    const long long Dr = seg->Dr, R1 = seg->R1;
+    args.n12 = seg->n12;
+    A2_REQUIRE(args.n12 >= 1 && BM % args.n12 == 0 && (long long)M == (long long)seg->Dl * args.n12,
+               "tc GEMM segment: rows must be (a, s12) with s12 dividing 128");
+    A2_REQUIRE(Dr % 8 == 0 && seg->Nb == N, "tc GEMM segment: Dr % 8 == 0, N == Dr");
+    args.nbc2 = (int)((Dr + kS3BK - 1) / kS3BK);
+    args.nk2 = (int)(R1 * args.nbc2);
+    for (int i = 0; i < 3; ++i) {
+      const cuuint64_t ad[4] = {(cuuint64_t)Dr, (cuuint64_t)args.n12, (cuuint64_t)R1,
+                                (cuuint64_t)seg->Dl};
+      const cuuint64_t as[3] = {(cuuint64_t)(Dr * 2), (cuuint64_t)(args.n12 * Dr * 2),
+                                (cuuint64_t)(R1 * args.n12 * Dr * 2)};
+      const cuuint32_t ab[4] = {(cuuint32_t)kS3BK, (cuuint32_t)args.n12, 1u,
+                                (cuuint32_t)(BM / args.n12)};
+      maps.a2[i] = make_map64(seg->A[i], 4, ad, as, ab);
+      const cuuint64_t bd[3] = {(cuuint64_t)Dr, (cuuint64_t)R1, (cuuint64_t)N};
+      const cuuint64_t bs[2] = {(cuuint64_t)(Dr * 2), (cuuint64_t)(R1 * Dr * 2)};
+      const cuuint32_t bb[3] = {(cuuint32_t)kS3BK, 1u, (cuuint32_t)BN};
+      maps.b2[i] = make_map64(seg->B[i], 3, bd, bs, bb);
+    }
+  } else {
+    for (int i = 0; i < 3; ++i) {
+      maps.a2[i] = maps.a[i];
+      maps.b2[i] = maps.b[i];
+    }
+  }
+  const size_t smem = sizeof(S3Smem<BN>) + 1024;
+  static std::once_flag once;
+  std::call_once(once, [smem] {
+    A2_CUDA(cudaFuncSetAttribute(tc_split3_kernel<BN>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  });
+  const int nk_total = args.nk1 + args.nk2;
+  splitk = std::max(1, std::min(splitk, nk_total));
+  args.M = M; args.N = N;
+  args.kblocks_per_split = (nk_total + splitk - 1) / splitk;
+  args.splits = (nk_total + args.kblocks_per_split - 1) / args.kblocks_per_split;
+  args.C = C; args.ldc = ldc; args.out_kind = out_kind;
+  args.tma_store = make_out_map(&maps.c, C, M, N, ldc) ? 1 : 0;
+  if (!args.tma_store) maps.c = maps.a[0];
+  const long long units = (long long)cdiv(M, BM) * cdiv(N, BN) * args.splits;
+  A2_REQUIRE(units < (1LL << 31), "tcgen05 GEMM too large");
+  const int grid = (int)std::min<long long>(units, std::max(1, tc_sms()));
+  tc_split3_kernel<BN><<<grid, kS3Threads, smem, s>>>(maps, args);
   A2_CHECK_LAUNCH();
 }
 
@@ -1137,15 +1629,11 @@ int tc_selftest_timeout(cudaStream_t s) {
   fill_zero(a.p, sizeof(__nv_bfloat16) * n * n, s);
   fill_zero(b.p, sizeof(__nv_bfloat16) * n * n, s);
   tc::TcMaps maps;
-  for (int i = 0; i < tc::kMaxPlanes; ++i) {
-    maps.a[i] = tc::make_map(a.as<__nv_bfloat16>(), n, n, n, tc::BM);
-    maps.b[i] = tc::make_map(b.as<__nv_bfloat16>(), n, n, n, 128);
-  }
-  for (int i = 0; i < 3; ++i) {
-    maps.a2[i] = maps.a[i];
-    maps.b2[i] = maps.b[i];
-  }
-  maps.c = maps.a[0];
+  maps.a = tc::make_map(a.as<__nv_bfloat16>(), n, n, n, tc::BM);
+  maps.b = tc::make_map(b.as<__nv_bfloat16>(), n, n, n, 128);
+  maps.a2 = maps.a;
+  maps.b2 = maps.b;
+  maps.c = maps.a;
   tc::TcArgs args{};
   args.M = args.N = args.K = n;
   args.nk1 = n / tc::BK;
@@ -1156,92 +1644,54 @@ int tc_selftest_timeout(cudaStream_t s) {
   args.C = c.p;
   args.ldc = n;
   args.out_kind = tc::OUT_F32;
-  args.npairs = 1;
   args.tma_store = 0;
-  args.split_ld = 0;
   args.wait_limit = 1u << 14;
   args.no_loads = 1;
-  const size_t smem = sizeof(tc::TcSmem<128, 6, 4, 2>) + 1024;
-  A2_CUDA(cudaFuncSetAttribute(tc::tc_gemm_kernel<128, 6, false>,
+  const size_t smem = sizeof(tc::TcSmem<128, 6>) + 1024;
+  A2_CUDA(cudaFuncSetAttribute(tc::tc_gemm_kernel<128, 6>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  tc::tc_gemm_kernel<128, 6, false><<<1, tc::tc_threads(false), smem, s>>>(maps, args);
+  tc::tc_gemm_kernel<128, 6><<<1, tc::kTcThreads, smem, s>>>(maps, args);
   A2_CHECK_LAUNCH();
   A2_CUDA(cudaStreamSynchronize(s));
   return tc_error_flag(true);
 }
 
-void tc_gemm_bf16(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* B, long long ldb,
-                  int M, int N, int K, void* C, long long ldc, int out_kind, int splitk,
-                  cudaStream_t s) {
-  const __nv_bfloat16* Ap[3] = {A, A, A};
-  const __nv_bfloat16* Bp[3] = {B, B, B};
-  const int p0[1] = {0};
-  tc_gemm_bf16_pairs(Ap, lda, Bp, ldb, M, N, K, 1, p0, p0, C, ldc, out_kind, splitk, s);
-}
-
 namespace {
 
-// One GEMM configuration: the kernel variant (0: BN = 128 / 6 stages, 1: BN = 256 /
-// 4 stages, 2: promoted split products) and the number of K splits.
+// One GEMM configuration: the tile width and the number of K splits.
 struct TcConfig {
-  int variant = 1, splitk = 1;
+  int bn = 256, splitk = 1;
 };
 
-void run_config(const TcConfig& cfg, const __nv_bfloat16* const* A, long long lda,
-                const __nv_bfloat16* const* B, long long ldb, int M, int N, int K, int npairs,
-                const int* pa, const int* pb, void* C, long long ldc, int out_kind,
-                cudaStream_t s, const TcSeg2* seg) {
-  if (cfg.variant == 2)
-    tc::launch<256, 4, true>(A, lda, B, ldb, M, N, K, npairs, pa, pb, seg, C, ldc, out_kind,
-                             cfg.splitk, s);
-  else if (cfg.variant == 0)
-    tc::launch<128, 6, false>(A, lda, B, ldb, M, N, K, npairs, pa, pb, seg, C, ldc, out_kind,
-                              cfg.splitk, s);
-  else
-    tc::launch<256, 4, false>(A, lda, B, ldb, M, N, K, npairs, pa, pb, seg, C, ldc, out_kind,
-                              cfg.splitk, s);
-}
-
 // Autotuner: the first call of a GEMM shape class (tile counts of M and N, K in steps of
-// 512, operand pairs, output kind, second segment) times the candidate configurations
-// with CUDA events on the caller's stream and keeps the fastest for every later call of
-// that class.  Candidates: the kernel
-// variants that apply (BN = 128 / 256; the promoted kernel for split products) and, for
-// accumulated outputs, the caller's K-split count, half and twice it.  Trials with an
-// accumulated output re-zero C first; the winner then runs on a zeroed C.
+// 512, plain or split products, output kind, second segment) times the candidate
+// configurations with CUDA events on the caller's stream and keeps the fastest for every
+// later call of that class.  Candidates: BN = 128 / 256 (split products take 128 only for
+// N <= 128, where the wide tile would multiply padding) and, for accumulated outputs, the
+// caller's K-split count, half and twice it.  Trials with an accumulated output re-zero C
+// first; the winner then runs on a zeroed C.
 struct TuneKey {
-  int M, N, K, npairs, out_kind, seg_rows;
+  int M, N, K, split3, out_kind, seg_rows;
   bool operator<(const TuneKey& o) const {
-    return std::tie(M, N, K, npairs, out_kind, seg_rows) <
-           std::tie(o.M, o.N, o.K, o.npairs, o.out_kind, o.seg_rows);
+    return std::tie(M, N, K, split3, out_kind, seg_rows) <
+           std::tie(o.M, o.N, o.K, o.split3, o.out_kind, o.seg_rows);
   }
 };
 std::mutex g_tune_mu;
 std::map<TuneKey, TcConfig> g_tune;
 bool g_tune_on = true;
 
-}  // namespace
-
-void tc_autotune(bool on) {
-  std::lock_guard<std::mutex> g(g_tune_mu);
-  g_tune_on = on;
-  if (!on) g_tune.clear();
-}
-
-void tc_gemm_bf16_pairs(const __nv_bfloat16* const* A, long long lda,
-                        const __nv_bfloat16* const* B, long long ldb, int M, int N, int K,
-                        int npairs, const int* pa, const int* pb, void* C, long long ldc,
-                        int out_kind, int splitk, cudaStream_t s, const TcSeg2* seg) {
-  if (M <= 0 || N <= 0) return;
-  A2_REQUIRE(K >= 1 && npairs >= 1 && npairs <= 6, "tc GEMM: K >= 1, 1..6 operand pairs");
+template <class Run>
+void tuned_gemm(int M, int N, int K, bool split3, void* C, long long ldc, int out_kind, int splitk,
+                cudaStream_t s, const TcSeg2* seg, Run&& run) {
+  A2_REQUIRE(K >= 1, "tc GEMM: K >= 1");
   if (splitk > 1)
     A2_REQUIRE(out_kind == tc::OUT_F32_ATOMIC, "split-K needs atomic FP32 output");
-  const bool promote = npairs > 1 && out_kind != tc::OUT_BF16;  // split products: promoted sums
   TcConfig def;
-  def.variant = promote ? 2 : (N <= 128 ? 0 : 1);
+  def.bn = N <= 128 ? 128 : 256;
   def.splitk = splitk;
   // shapes with the same tile counts (and K within 512) share one decision
-  const TuneKey key{(M + 127) / 128, (N + 127) / 128, (K + 511) / 512, npairs, out_kind,
+  const TuneKey key{(M + 127) / 128, (N + 127) / 128, (K + 511) / 512, split3 ? 1 : 0, out_kind,
                     seg ? (seg->R1 * seg->Dr + 511) / 512 : 0};
   bool tune = false;
   TcConfig best = def;
@@ -1254,17 +1704,17 @@ void tc_gemm_bf16_pairs(const __nv_bfloat16* const* A, long long lda,
     }
   }
   if (!tune) {
-    run_config(best, A, lda, B, ldb, M, N, K, npairs, pa, pb, C, ldc, out_kind, s, seg);
+    run(best);
     return;
   }
   std::vector<TcConfig> cand;
-  std::vector<int> variants = promote ? std::vector<int>{2} : std::vector<int>{0, 1};
+  std::vector<int> widths = split3 ? std::vector<int>{def.bn} : std::vector<int>{128, 256};
   std::vector<int> splits{splitk};
   if (out_kind == tc::OUT_F32_ATOMIC) {
     splits.push_back(splitk * 2);
     if (splitk > 1) splits.push_back(std::max(1, splitk / 2));
   }
-  for (int v : variants)
+  for (int v : widths)
     for (int k : splits) cand.push_back(TcConfig{v, k});
   const size_t cbytes = (size_t)M * ldc * (out_kind == tc::OUT_BF16 ? 2 : 4);
   cudaEvent_t e0, e1;
@@ -1274,7 +1724,7 @@ void tc_gemm_bf16_pairs(const __nv_bfloat16* const* A, long long lda,
   for (const TcConfig& cf : cand) {
     if (out_kind == tc::OUT_F32_ATOMIC) fill_zero(C, cbytes, s);
     A2_CUDA(cudaEventRecord(e0, s));
-    run_config(cf, A, lda, B, ldb, M, N, K, npairs, pa, pb, C, ldc, out_kind, s, seg);
+    run(cf);
     A2_CUDA(cudaEventRecord(e1, s));
     A2_CUDA(cudaEventSynchronize(e1));
     float ms = 0.f;
@@ -1291,7 +1741,40 @@ void tc_gemm_bf16_pairs(const __nv_bfloat16* const* A, long long lda,
     g_tune[key] = best;
   }
   if (out_kind == tc::OUT_F32_ATOMIC) fill_zero(C, cbytes, s);
-  run_config(best, A, lda, B, ldb, M, N, K, npairs, pa, pb, C, ldc, out_kind, s, seg);
+  run(best);
+}
+
+}  // namespace
+
+void tc_autotune(bool on) {
+  std::lock_guard<std::mutex> g(g_tune_mu);
+  g_tune_on = on;
+  if (!on) g_tune.clear();
+}
+
+void tc_gemm_bf16(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* B, long long ldb,
+                  int M, int N, int K, void* C, long long ldc, int out_kind, int splitk,
+                  cudaStream_t s, const TcSeg2* seg) {
+  if (M <= 0 || N <= 0) return;
+  tuned_gemm(M, N, K, false, C, ldc, out_kind, splitk, s, seg, [&](const TcConfig& cf) {
+    if (cf.bn == 128)
+      tc::launch<128, 6>(A, lda, B, ldb, M, N, K, seg, C, ldc, out_kind, cf.splitk, s);
+    else
+      tc::launch<256, 4>(A, lda, B, ldb, M, N, K, seg, C, ldc, out_kind, cf.splitk, s);
+  });
+}
+
+void tc_gemm_split3(const __nv_bfloat16* const* A, long long lda, const __nv_bfloat16* const* B,
+                    long long ldb, int M, int N, int K, float* C, long long ldc, bool add,
+                    int splitk, cudaStream_t s, const TcSeg2* seg) {
+  if (M <= 0 || N <= 0) return;
+  const int out_kind = add ? tc::OUT_F32_ATOMIC : tc::OUT_F32;
+  tuned_gemm(M, N, K, true, C, ldc, out_kind, splitk, s, seg, [&](const TcConfig& cf) {
+    if (cf.bn == 128)
+      tc::launch_split3<128>(A, lda, B, ldb, M, N, K, seg, C, ldc, out_kind, cf.splitk, s);
+    else
+      tc::launch_split3<256>(A, lda, B, ldb, M, N, K, seg, C, ldc, out_kind, cf.splitk, s);
+  });
 }
 
 // -------------------------------------------------------------- BF16 H_eff chain
@@ -1375,11 +1858,8 @@ void tc_heff_bf16(cudaStream_t s, int n1, int n2, int Rl, int R1, int Rr, int Dl
     const double M = M4, N = Dr, K = (double)K4 + (F.Rt ? (double)R1 * Dr : 0.0);
     ProfScope ps(PK_TC_S4, s, 2.0 * M * N * K, 2.0 * (M * K + N * K) + 4.0 * M * N);
     fill_zero(y, sizeof(float) * (size_t)M4 * Dr, s);
-    const __nv_bfloat16* A[3] = {T3, T3, T3};
-    const __nv_bfloat16* B[3] = {Rb, Rb, Rb};
-    const int p0[1] = {0};
-    tc_gemm_bf16_pairs(A, ld3, B, ldr, M4, Dr, (int)K4, 1, p0, p0, y, Dr, tc::OUT_F32_ATOMIC,
-                       s4_splitk(M4, Dr, kb), s, F.Rt ? &seg : nullptr);
+    tc_gemm_bf16(T3, ld3, Rb, ldr, M4, Dr, (int)K4, y, Dr, tc::OUT_F32_ATOMIC,
+                 s4_splitk(M4, Dr, kb), s, F.Rt ? &seg : nullptr);
   }
 }
 
@@ -1397,8 +1877,6 @@ void tc_heff_f32emu(cudaStream_t s, int n1, int n2, int Rl, int R1, int Rr, int 
                     const __nv_bfloat16* Rp, long long ldr, long long rplane, const double* x,
                     float* y, const SparseRows<float>& W1, const SparseRows<float>& W2,
                     const HeffFold& F, DevBuf& t1, DevBuf& t2, DevBuf& xa, DevBuf& tf) {
-  static const int pa[6] = {0, 0, 1, 0, 1, 2};
-  static const int pb[6] = {0, 1, 0, 2, 1, 0};
   const long long NX = (long long)n1 * n2 * Dr;
   const long long ldx = pad8(Dl);
   const long long xplane = NX * ldx;
@@ -1430,15 +1908,14 @@ void tc_heff_f32emu(cudaStream_t s, int n1, int n2, int Rl, int R1, int Rr, int 
     const __nv_bfloat16* B[3] = {XT, XT + xplane, XT + 2 * xplane};
     const double M = (double)Dl * Rl, N = (double)NX, K = Dl;
     ProfScope ps(PK_EMU_S1, s, 6.0 * 2.0 * M * N * K, 6.0 * (M * K + N * K) + 4.0 * M * N);
-    tc_gemm_bf16_pairs(A, ldl, B, ldx, Dl * Rl, (int)NX, Dl, 6, pa, pb, T1, NX, tc::OUT_F32, 1, s);
+    tc_gemm_split3(A, ldl, B, ldx, Dl * Rl, (int)NX, Dl, T1, NX, false, 1, s);
   }
   if (F.Lt) {   // folded G of A_k: Lt x, FP32 (into T2, or into Tg when T2 is split)
     const __nv_bfloat16* A[3] = {F.Lt, F.Lt + F.ltplane, F.Lt + 2 * F.ltplane};
     const __nv_bfloat16* B[3] = {XT, XT + xplane, XT + 2 * xplane};
     const double M = (double)Dl * R1, N = (double)NX, K = Dl;
     ProfScope ps(PK_EMU_S1, s, 6.0 * 2.0 * M * N * K, 6.0 * (M * K + N * K) + 4.0 * M * N);
-    tc_gemm_bf16_pairs(A, ldl, B, ldx, Dl * R1, (int)NX, Dl, 6, pa, pb, Tg ? Tg : T2, NX,
-                       tc::OUT_F32, 1, s);
+    tc_gemm_split3(A, ldl, B, ldx, Dl * R1, (int)NX, Dl, Tg ? Tg : T2, NX, false, 1, s);
   }
   {  // S2 (FP32; W_rest added to the folded part when A_k is folded)
     ProfScope ps(PK_EMU_S2, s, 2.0 * W1.nnz_total * (double)n2 * Dr * Dl,
@@ -1486,9 +1963,8 @@ void tc_heff_f32emu(cudaStream_t s, int n1, int n2, int Rl, int R1, int Rr, int 
     const double M = (double)M4, N = Dr, K = (double)K4 + (t2split ? (double)R1 * Dr : 0.0);
     ProfScope ps(PK_EMU_S4, s, 6.0 * 2.0 * M * N * K, 6.0 * (M * K + N * K) + 4.0 * M * N);
     fill_zero(y, sizeof(float) * (size_t)M4 * Dr, s);
-    tc_gemm_bf16_pairs(A, ld3, B, ldr, (int)M4, Dr, (int)K4, 6, pa, pb, y, Dr,
-                       tc::OUT_F32_ATOMIC, s4_splitk(M4, Dr, kb), s,
-                       t2split ? &seg : nullptr);
+    tc_gemm_split3(A, ld3, B, ldr, (int)M4, Dr, (int)K4, y, Dr, true, s4_splitk(M4, Dr, kb), s,
+                   t2split ? &seg : nullptr);
   }
 }
 
@@ -1500,8 +1976,6 @@ void tc_heff1_f32emu(cudaStream_t s, int n, int Rl, int Rr, int Dl, int Dr,
                      const __nv_bfloat16* Lp, long long ldl, long long lplane,
                      const __nv_bfloat16* Rp, long long ldr, long long rplane, const double* x,
                      float* y, const SparseRows<float>& W, DevBuf& t1, DevBuf& t2, DevBuf& xa) {
-  static const int pa[6] = {0, 0, 1, 0, 1, 2};
-  static const int pb[6] = {0, 1, 0, 2, 1, 0};
   const long long NX = (long long)n * Dr;
   const long long ldx = pad8(Dl);
   const long long xplane = (NX * ldx + 63) / 64 * 64;
@@ -1522,7 +1996,7 @@ void tc_heff1_f32emu(cudaStream_t s, int n, int Rl, int Rr, int Dl, int Dr,
     const __nv_bfloat16* B[3] = {XT, XT + xplane, XT + 2 * xplane};
     const double M = (double)Dl * Rl, N = (double)NX, K = Dl;
     ProfScope ps(PK_EMU_S1, s, 6.0 * 2.0 * M * N * K, 6.0 * (M * K + N * K) + 4.0 * M * N);
-    tc_gemm_bf16_pairs(A, ldl, B, ldx, Dl * Rl, (int)NX, Dl, 6, pa, pb, T1, NX, tc::OUT_F32, 1, s);
+    tc_gemm_split3(A, ldl, B, ldx, Dl * Rl, (int)NX, Dl, T1, NX, false, 1, s);
   }
   {
     ProfScope ps(PK_EMU_S3, s, 2.0 * W.nnz_total * (double)Dr * Dl,
@@ -1540,159 +2014,171 @@ void tc_heff1_f32emu(cudaStream_t s, int n, int Rl, int Rr, int Dl, int Dr,
     const double M = (double)M4, N = Dr, K = (double)K4;
     ProfScope ps(PK_EMU_S4, s, 6.0 * 2.0 * M * N * K, 6.0 * (M * K + N * K) + 4.0 * M * N);
     fill_zero(y, sizeof(float) * (size_t)M4 * Dr, s);
-    tc_gemm_bf16_pairs(A, ld3, B, ldr, (int)M4, Dr, (int)K4, 6, pa, pb, y, Dr,
-                       tc::OUT_F32_ATOMIC, s4_splitk(M4, Dr, (K4 + 63) / 64), s);
+    tc_gemm_split3(A, ld3, B, ldr, (int)M4, Dr, (int)K4, y, Dr, true,
+                   s4_splitk(M4, Dr, (K4 + 63) / 64), s);
   }
 }
 
 // ============================================================================ FP64 emulation
 // Ozaki scheme (Ozaki, Ogita, Oishi, Rump, "Error-free transformations of matrix
 // multiplication by using fast routines of matrix multiplication and its applications",
-// Numer. Algorithms 59, 2012) on the BF16 tensor cores.  Every row r of an FP64 operand
-// is split into kOzSlices slices P_i[r][k] = q * 2^(e_r - kOzBits*i) with integer
-// |q| <= 2^kOzBits - 1 (truncation of the remainder; e_r = ilogb(max_k |X[r][k]|) + 1),
-// each exact in BF16.  A product of slice i of A with slice j of B is then an integer
-// multiple of the unit 2^(e_r + e_c - kOzBits*(i+j)) of magnitude below 2^(2*kOzBits);
-// all pairs of one level l = i + j share that unit, so a level's sum over at most
-// 1024 / (l - 1) K indices per pair stays an integer below 2^24 units and the tensor
-// cores' FP32 accumulation of it is exact.  The pairs with i + j <= kOzSlices + 1 are
-// kept (the rest lie below 2^-kOzBits*kOzSlices of |A||B|), every level's tile of every K
-// split is stored in FP32, and a combine kernel adds the tiles, smallest level first, with
-// error-free two-sums into a pair of FP32 numbers (~2^-48 relative).
+// Numer. Algorithms 59, 2012) on the BF16 tensor cores.  Every 256-wide chunk of a row of an
+// FP64 operand is brought to 55-bit fixed point at the scale of its largest entry, S = X[r][k]
+// 2^(55 - e) rounded to an integer, e = ilogb(max_k |X[r][k]|) + 1 over the chunk, and S is written
+// in balanced digits of radix 2^kOzBits: slice i holds q_i 2^(e + 1 - 8 i) with -128 <= q_i <= 127
+// (the leading digit up to 128), exact in BF16.  Balanced digits use BF16's whole
+// significand (7 slices for 55 bits; digits of one sign would need 8 slices and 36 pairs for
+// the same products of 2^14).  A product of slice i of A with slice j of B is an integer
+// multiple of the unit 2^(e_A + e_B + 2 - 8 (i + j)) of the chunk; the pairs with i + j <= 8 are
+// kept (28; the rest lie below 2^-58 of the scales), see tc_oz_kernel for their exact
+// accumulation chunk by chunk.
 namespace {
 
-// Slicing with integer operations only (the FP64 pipe is slow on this part): for a row
-// with largest biased exponent field f_max, e = f_max - 1022 bounds |v| < 2^e; the
-// fixed-point magnitude N = floor(|v| * 2^(56 - e)) < 2^56 is the significand shifted by
-// f - e - 1019 bits, and slice i is bits [56 - 7i, 63 - 7i) of N times 2^(e - 7i) with the
-// sign of v (the same digits as truncating the remainder slice by slice).  Scales below
-// the FP32 normal range are flushed to zero.
-static_assert(kOzSlices * kOzBits == 56, "the slices cover bits 0..55 of the fixed-point value");
+static_assert(kOzSlices == 7 && kOzBits == 8, "the digits cover 55 bits and a sign");
 
 __device__ __forceinline__ float pow2f(int k) {
   return (k >= -126 && k <= 127) ? __int_as_float((k + 127) << 23) : 0.f;
 }
 
-// One warp per row: the row's largest exponent by a warp reduction (no block barrier),
-// then the slices of four consecutive entries per lane, each plane written as one 8-byte
-// vector per lane (the kernel is bound by its 16 bytes of writes per entry).
-// The 56-bit fixed-point magnitude of v at the row's scale 2^e (|v| < 2^e) and its sign.
-__device__ __forceinline__ unsigned long long oz_fixed(double v, int e, float& sgn) {
+// Slicing with integer operations only (the FP64 pipe is slow on this part): the signed
+// 55-bit fixed-point value of v at the row's scale 2^e (|v| < 2^e), rounded to nearest.
+__device__ __forceinline__ long long oz_fixed(double v, int e) {
   const long long bits = __double_as_longlong(v);
   int f = (int)((bits >> 52) & 0x7FF);
-  unsigned long long m = (unsigned long long)bits & ((1ull << 52) - 1);
-  if (f) m |= 1ull << 52;
+  long long m = bits & ((1ll << 52) - 1);
+  if (f) m |= 1ll << 52;
   else f = 1;                                    // subnormal: no hidden bit
-  const int sh = f - e - 1019;                   // <= 3 since |v| < 2^e
-  sgn = bits < 0 ? -1.f : 1.f;
-  return sh >= 0 ? (m << sh) : (sh > -64 ? (m >> -sh) : 0ull);
+  const int sh = f - e - 1020;                   // <= 2 since |v| < 2^e
+  if (sh >= 0) m <<= sh;
+  else m = sh > -60 ? (m + (1ll << (-sh - 1))) >> -sh : 0ll;
+  return bits < 0 ? -m : m;
 }
+// The last digit of S (slice kOzSlices - t for the t-th call) and S without it.
+__device__ __forceinline__ int oz_digit(long long& S) {
+  const int q = (int)(signed char)(S & 0xFF);
+  S = (S - q) >> kOzBits;
+  return q;
+}
+// The digits of S as floats, slice 1 first (the leading digit takes what is left).
+__device__ __forceinline__ void oz_digits(long long S, int (&q)[kOzSlices]) {
+#pragma unroll
+  for (int i = kOzSlices - 1; i > 0; --i) q[i] = oz_digit(S);
+  q[0] = (int)S;
+}
+
+// Four digits at the scale sc as BF16 (exact).
+__device__ __forceinline__ uint2 oz_pack(int a, int b, int c, int d, float sc) {
+  const __nv_bfloat162 lo = __floats2bfloat162_rn((float)a * sc, (float)b * sc);
+  const __nv_bfloat162 hi = __floats2bfloat162_rn((float)c * sc, (float)d * sc);
+  uint2 pk;
+  pk.x = *reinterpret_cast<const unsigned int*>(&lo);
+  pk.y = *reinterpret_cast<const unsigned int*>(&hi);
+  return pk;
+}
+
+// One warp per row and 256-wide K chunk, whose entries stay in registers (eight per lane): one
+// read, the chunk's largest exponent by a warp reduction, then each slice of four
+// consecutive entries as one 8-byte vector.  The last K block is filled with zeros.  Bound by
+// HBM: 8 bytes read and 14 written per entry.  With one scale for a whole row (read twice, one
+// warp for 143872 entries of T3) the slicing of S4's operand took 2.75 ms at D = 256 with the
+// slicing of x, now 1.82.
+constexpr int kOzGroup = 256;              // entries that share a scale (tc_oz_kernel's chunk)
+static_assert(kOzGroup == tc::kOzChunk * tc::kOzBK, "a chunk of the GEMM has one scale");
 __global__ void __launch_bounds__(256)
 ozaki_split_kernel(const double* __restrict__ X, long long sr, long long sk, int rows, int K,
-                   __nv_bfloat16* __restrict__ P, long long ldp, long long plane) {
+                   __nv_bfloat16* __restrict__ P, long long ntasks) {
   const int lane = threadIdx.x & 31;
-  const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
-  for (int r = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); r < rows; r += nwarps) {
+  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+  const int Kp = (K + kOzKBlock - 1) / kOzKBlock * kOzKBlock;
+  for (long long task = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; task < ntasks;
+       task += nwarps) {
+    const int ch = (int)(task / rows), r = (int)(task - (long long)ch * rows);
     const double* xr = X + (long long)r * sr;
+    double v[8];
     int fm = 0;
-    for (int k = lane; k < K; k += 32)
-      fm = max(fm, (int)((__double_as_longlong(xr[(long long)k * sk]) >> 52) & 0x7FF));
-    for (int o = 16; o; o >>= 1) fm = max(fm, __shfl_xor_sync(0xffffffffu, fm, o));
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int k = ch * kOzGroup + (u >> 2) * 128 + 4 * lane + (u & 3);
+      v[u] = k < K ? xr[(long long)k * sk] : 0.0;
+      fm = max(fm, (__double2hiint(v[u]) >> 20) & 0x7FF);
+    }
+    fm = __reduce_max_sync(0xffffffffu, fm);
     const int e = max(fm, 1) - 1022;
-    __nv_bfloat16* pr = P + (long long)r * ldp;
-    for (int k0 = 4 * lane; k0 < K; k0 += 128) {
-      unsigned long long N[4];
-      float sgn[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        sgn[u] = 1.f;
-        N[u] = k0 + u < K ? oz_fixed(xr[(long long)(k0 + u) * sk], e, sgn[u]) : 0ull;
-      }
+    for (int h = 0; h < 2; ++h) {
+      const int k0 = ch * kOzGroup + h * 128 + 4 * lane;
+      if (k0 >= Kp) continue;
+      int q[4][kOzSlices];
 #pragma unroll
-      for (int i = 1; i <= kOzSlices; ++i) {
-        const float sc = pow2f(e - kOzBits * i);
-        float w[4];
+      for (int u = 0; u < 4; ++u) oz_digits(oz_fixed(v[4 * h + u], e), q[u]);
+      __nv_bfloat16* dst =
+          P + ((long long)(k0 / kOzKBlock) * rows + r) * kOzRowBlock + k0 % kOzKBlock;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int q = (int)((N[u] >> (56 - kOzBits * i)) & ((1u << kOzBits) - 1));
-          w[u] = sgn[u] * (float)q * sc;   // exact in BF16
-        }
-        __nv_bfloat16* dst = pr + (long long)(i - 1) * plane + k0;
-        if (k0 + 4 <= K) {   // ldp % 8 == 0, plane % 64 == 0, k0 % 4 == 0: 8-byte aligned
-          const __nv_bfloat162 lo = __floats2bfloat162_rn(w[0], w[1]);
-          const __nv_bfloat162 hi = __floats2bfloat162_rn(w[2], w[3]);
-          uint2 pk;
-          pk.x = *reinterpret_cast<const unsigned int*>(&lo);
-          pk.y = *reinterpret_cast<const unsigned int*>(&hi);
-          *reinterpret_cast<uint2*>(dst) = pk;
-        } else {
-          for (int u = 0; u < 4; ++u)
-            if (k0 + u < K) dst[u] = __float2bfloat16_rn(w[u]);
-        }
-      }
+      for (int i = 0; i < kOzSlices; ++i)
+        *reinterpret_cast<uint2*>(dst + i * kOzKBlock) =
+            oz_pack(q[0][i], q[1][i], q[2][i], q[3][i], pow2f(e + 1 - kOzBits * (i + 1)));
     }
   }
 }
 
 // Slices of the rows of X^T, X a (K x N) row-major matrix (row stride ldx): output row n
-// holds X[k][n], k < K.  A block takes 32 consecutive output rows: the exponent pass and
-// the slicing read X row by row (coalesced across the 32 columns), the slices of a
-// 64-wide K chunk are staged in shared memory and leave as 8-byte vectors along K.  Same
-// slices as ozaki_split of the transposed matrix.
+// holds X[k][n], k < K.  A block takes 32 consecutive output rows and one K chunk, held in
+// registers (32 entries per thread, read row by row of X, coalesced); the digits of 64 k at a
+// time go through shared memory and leave as 8-byte vectors along K.  Same slices as
+// ozaki_split of the transposed matrix.  Environment update, T2 1024 x 113664: 0.75 ms with two
+// reads (one scale per row), now 0.68.
 constexpr int kOzColChunk = 64, kOzColPad = kOzColChunk + 4;   // row of 68 BF16 = 136 B
 __global__ void __launch_bounds__(256)
 ozaki_split_cols_kernel(const double* __restrict__ X, long long ldx, int N, int K,
-                        __nv_bfloat16* __restrict__ P, long long ldp, long long plane) {
+                        __nv_bfloat16* __restrict__ P) {
   __shared__ int emax[8][32];
   __shared__ __align__(16) __nv_bfloat16 tile[kOzSlices][32][kOzColPad];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int n0 = blockIdx.x * 32, n = n0 + lane;
+  const int n0 = blockIdx.x * 32, n = n0 + lane, kc = blockIdx.y * kOzGroup;
+  const int Kp = (K + kOzKBlock - 1) / kOzKBlock * kOzKBlock;
+  double v[kOzGroup / 8];
   int fm = 0;
-  if (n < N)
-    for (int k = warp; k < K; k += 8)
-      fm = max(fm, (int)((__double_as_longlong(X[(long long)k * ldx + n]) >> 52) & 0x7FF));
+#pragma unroll
+  for (int t = 0; t < kOzGroup / 8; ++t) {
+    const int k = kc + warp + 8 * t;
+    v[t] = n < N && k < K ? X[(long long)k * ldx + n] : 0.0;
+    fm = max(fm, (__double2hiint(v[t]) >> 20) & 0x7FF);
+  }
   emax[warp][lane] = fm;
   __syncthreads();
-  fm = 0;
 #pragma unroll
   for (int w = 0; w < 8; ++w) fm = max(fm, emax[w][lane]);
   const int e = max(fm, 1) - 1022;
-  for (int k0 = 0; k0 < K; k0 += kOzColChunk) {
+#pragma unroll
+  for (int c = 0; c < kOzGroup / kOzColChunk; ++c) {
+    const int k0 = kc + c * kOzColChunk;
+    if (k0 >= Kp) break;
 #pragma unroll
     for (int t = 0; t < kOzColChunk / 8; ++t) {
-      const int kk = warp + 8 * t, k = k0 + kk;
-      float sgn = 1.f;
-      const unsigned long long Nq =
-          (n < N && k < K) ? oz_fixed(X[(long long)k * ldx + n], e, sgn) : 0ull;
+      int q[kOzSlices];
+      oz_digits(oz_fixed(v[c * (kOzColChunk / 8) + t], e), q);
 #pragma unroll
-      for (int i = 1; i <= kOzSlices; ++i) {
-        const int q = (int)((Nq >> (56 - kOzBits * i)) & ((1u << kOzBits) - 1));
-        tile[i - 1][lane][kk] = __float2bfloat16_rn(sgn * (float)q * pow2f(e - kOzBits * i));
-      }
+      for (int i = 0; i < kOzSlices; ++i)
+        tile[i][lane][warp + 8 * t] =
+            __float2bfloat16_rn((float)q[i] * pow2f(e + 1 - kOzBits * (i + 1)));
     }
     __syncthreads();
-    // 8 slices x 32 rows x 16 vectors of 4 values
-    for (int v = threadIdx.x; v < kOzSlices * 32 * (kOzColChunk / 4); v += blockDim.x) {
-      const int i = v / (32 * (kOzColChunk / 4)), r = (v / (kOzColChunk / 4)) % 32;
-      const int c4 = v % (kOzColChunk / 4), k = k0 + 4 * c4;
-      if (n0 + r >= N || k >= K) continue;
-      __nv_bfloat16* dst = P + (long long)i * plane + (long long)(n0 + r) * ldp + k;
-      const __nv_bfloat16* src = &tile[i][r][4 * c4];
-      if (k + 4 <= K)   // ldp % 8 == 0, plane % 64 == 0, k % 4 == 0: 8-byte aligned
-        *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(src);
-      else
-        for (int u = 0; k + u < K; ++u) dst[u] = src[u];
+    // vectors of 4 values, the slices of one (row, K block) one after another in memory
+    for (int w = threadIdx.x; w < kOzSlices * 32 * (kOzColChunk / 4); w += 256) {
+      const int c4 = w % (kOzKBlock / 4), i = (w / (kOzKBlock / 4)) % kOzSlices;
+      const int rk = w / (kOzKBlock / 4 * kOzSlices), r = rk % 32, k = k0 + rk / 32 * kOzKBlock;
+      if (n0 + r >= N || k >= Kp) continue;
+      *reinterpret_cast<uint2*>(P + ((long long)(k / kOzKBlock) * N + n0 + r) * kOzRowBlock +
+                                i * kOzKBlock + 4 * c4) =
+          *reinterpret_cast<const uint2*>(&tile[i][r][rk / 32 * kOzKBlock + 4 * c4]);
     }
     __syncthreads();
   }
 }
 
-// C[r][c] = sum over the level tiles: tile t of level lev[t] at T + t * MN (row-major,
-// N columns); tiles ordered by level (largest level last).
-// C[r][c] = sum of all level tiles (tile t at T + t * MN, row-major with N columns,
-// ordered by level, largest level last), added smallest level first in double-float
-// arithmetic: every tile value is exact, the two-sum keeps the running sum as an FP32
-// pair hi + lo (~2^-48), and the result is written as FP64 (hi + lo) or as the pair.
+// C[r][c] = sum of the K splits' FP32 pairs (tile t at T + t * MN, row-major with N columns),
+// in double-float arithmetic: the two-sum keeps the running sum as an FP32 pair hi + lo
+// (~2^-48), and the result is written as FP64 (hi + lo) or as the pair.
 template <bool DF>
 __global__ void ozaki_combine_kernel(const float* __restrict__ T, long long MN, int nt, int N,
                                      double* __restrict__ C, float* __restrict__ Cdf,
@@ -1722,57 +2208,50 @@ __global__ void ozaki_combine_kernel(const float* __restrict__ T, long long MN, 
 }  // namespace
 
 void ozaki_split_cols(const double* X, long long ldx, int N, int K, __nv_bfloat16* P,
-                      long long ldp, long long plane, cudaStream_t s) {
+                      cudaStream_t s) {
   if (N <= 0 || K <= 0) return;
-  ozaki_split_cols_kernel<<<(N + 31) / 32, 256, 0, s>>>(X, ldx, N, K, P, ldp, plane);
+  A2_REQUIRE(cdiv(K, kOzGroup) < 65536, "Ozaki slicing: K too large");
+  ozaki_split_cols_kernel<<<dim3((N + 31) / 32, cdiv(K, kOzGroup)), 256, 0, s>>>(X, ldx, N, K, P);
   A2_CHECK_LAUNCH();
 }
 
 void ozaki_split(const double* X, long long sr, long long sk, int rows, int K, __nv_bfloat16* P,
-                 long long ldp, long long plane, cudaStream_t s) {
+                 cudaStream_t s) {
   if (rows <= 0 || K <= 0) return;
-  const int grid = std::min((rows + 7) / 8, 152 * 8);   // eight rows (warps) per block
-  ozaki_split_kernel<<<grid, 256, 0, s>>>(X, sr, sk, rows, K, P, ldp, plane);
+  if (sr == 1 && sk > 1) {               // entries of a row far apart: the transposed kernel
+    ozaki_split_cols(X, sk, rows, K, P, s);
+    return;
+  }
+  const long long ntasks = (long long)rows * cdiv(K, kOzGroup);
+  const int grid = (int)std::min<long long>((ntasks + 7) / 8, 152 * 32);   // eight warps per block
+  ozaki_split_kernel<<<grid, 256, 0, s>>>(X, sr, sk, rows, K, P, ntasks);
   A2_CHECK_LAUNCH();
 }
 
-void tc_gemm_f64emu(const __nv_bfloat16* A, long long lda, long long aplane,
-                    const __nv_bfloat16* B, long long ldb, long long bplane, int M, int N, int K,
-                    double* C, long long ldc, DevBuf& slab, cudaStream_t s, float* Cdf,
-                    long long df_plane) {
+void tc_gemm_f64emu(const __nv_bfloat16* A, const __nv_bfloat16* B, int M, int N, int K, double* C,
+                    long long ldc, DevBuf& slab, cudaStream_t s, float* Cdf, long long df_plane) {
   if (M <= 0 || N <= 0) return;
-  static int num_sms = 0;
-  static std::once_flag sms_once;
-  std::call_once(sms_once, [] {
-    int dev = 0;
-    A2_CUDA(cudaGetDevice(&dev));
-    A2_CUDA(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
-  });
-  const __nv_bfloat16* Ap[tc::kMaxPlanes];
-  const __nv_bfloat16* Bp[tc::kMaxPlanes];
-  for (int i = 0; i < tc::kMaxPlanes; ++i) {
-    Ap[i] = A + i * aplane;
-    Bp[i] = B + i * bplane;
-  }
-  // K splits: at most kOzSplitBlocks K blocks per split (bounds the number of chunk sums
-  // per accumulator, hence the rounding of its lo part), and enough work units to fill
-  // the GPU when the output has few tiles
-  constexpr int kOzSplitBlocks = 64;
-  const int nk = (K + tc::BK - 1) / tc::BK;
+  const int num_sms = tc::tc_sms();
+  // K splits: at most kOzSplitBlocks K blocks per split (bounds the number of sums per
+  // accumulator, hence the rounding of its lo part), and enough work units to fill the GPU
+  // when the output has few tiles
+  static_assert(kOzKBlock == tc::kOzBK, "K block of the sliced layout");
+  constexpr int kOzSplitBlocks = 4096 / tc::kOzBK;
+  const int nk = (K + tc::kOzBK - 1) / tc::kOzBK;
   const long long tiles = (long long)cdiv(M, tc::BM) * cdiv(N, tc::kOzBN);
   int splits = cdiv(nk, kOzSplitBlocks);
   if (tiles < num_sms) splits = std::max<int>(splits, (int)cdiv(2LL * num_sms, tiles));
-  splits = std::max(1, std::min(splits, nk));
+  splits = std::max(1, std::min(splits, cdiv(nk, 2)));
   splits = cdiv(nk, cdiv(nk, splits));   // the count launch_oz will use
   if (splits == 1) {
-    if (Cdf) tc::launch_oz(Ap, lda, Bp, ldb, M, N, K, 1, tc::OZ_PAIR, Cdf, ldc, df_plane, s);
-    else tc::launch_oz(Ap, lda, Bp, ldb, M, N, K, 1, tc::OZ_F64, C, ldc, 0, s);
+    if (Cdf) tc::launch_oz(A, B, M, N, K, 1, tc::OZ_PAIR, Cdf, ldc, df_plane, s);
+    else tc::launch_oz(A, B, M, N, K, 1, tc::OZ_F64, C, ldc, 0, s);
     return;
   }
   const long long MN = (long long)M * N;
   slab.ensure(sizeof(float) * (size_t)(2LL * splits * MN), s);
   float* T = slab.as<float>();
-  tc::launch_oz(Ap, lda, Bp, ldb, M, N, K, splits, tc::OZ_SPLIT, T, N, 0, s);
+  tc::launch_oz(A, B, M, N, K, splits, tc::OZ_SPLIT, T, N, 0, s);
   const int grid = (int)std::min<long long>((MN + 255) / 256, 152LL * 16);
   if (Cdf)
     ozaki_combine_kernel<true><<<grid, 256, 0, s>>>(T, MN, 2 * splits, N, nullptr, Cdf,
