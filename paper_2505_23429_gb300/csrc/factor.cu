@@ -277,6 +277,340 @@ hh_form_q_kernel(const double* V, const double* tau, int cols, int k, double* Q)
   }
 }
 
+// ------------------------------------------------------------------ shared helpers
+__device__ __forceinline__ double lq_warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+// Sums of four values over the warp; lane l returns that of value (l >> 3) & 3.
+__device__ __forceinline__ double lq_warp_sum4(const double (&v)[4], int lane) {
+  const bool h16 = lane & 16, h8 = lane & 8;
+  const double u0 = (h16 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, h16 ? v[0] : v[2], 16);
+  const double u1 = (h16 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, h16 ? v[1] : v[3], 16);
+  double r = (h8 ? u1 : u0) + __shfl_xor_sync(0xffffffffu, h8 ? u0 : u1, 8);
+#pragma unroll
+  for (int o = 4; o; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  return r;
+}
+// 1 / q to ~2^-58 (q normal): hardware seed, e = 1 - q r, r (1 + e + e^2).
+__device__ __forceinline__ double lq_rcp(double q) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(q));
+  const double e = fma(-q, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+// (beta, tau, scale) of the reflection that maps (al, x_1..), sum x_k^2 = s2, onto beta e_0:
+// beta = -sign(al) |x|, tau = (beta - al) / beta = 1 + |al| / |x|, scale = 1 / (al - beta); tau = 0
+// (and beta = al) when s2 = 0.  One reciprocal square root and one reciprocal instead of a
+// square root and two divisions (half the latency); the latter outside the normal range.
+__device__ __forceinline__ void lq_scalars(double al, double s2, double& beta, double& tau,
+                                           double& scale) {
+  beta = al;
+  tau = 0.0;
+  scale = 0.0;
+  if (!(s2 > 0.0)) return;
+  const double n2 = fma(al, al, s2), aa = fabs(al);
+  double nrm;
+  if (n2 > 1e-280 && n2 < 1e280) {
+    const double inv = rsqrt(n2);
+    nrm = n2 * inv;
+    tau = fma(aa, inv, 1.0);
+    scale = lq_rcp(aa + nrm);
+  } else {
+    nrm = sqrt(n2);
+    tau = (nrm + aa) / nrm;
+    scale = 1.0 / (aa + nrm);
+  }
+  beta = al >= 0.0 ? -nrm : nrm;
+  if (!(al >= 0.0)) scale = -scale;
+}
+
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned cluster_size() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// Value at shared-memory address p of CTA `rank` of the cluster.
+__device__ __forceinline__ double ld_cluster(const double* p, unsigned rank) {
+  unsigned a = (unsigned)__cvta_generic_to_shared(p), ra;
+  double v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(ra) : "memory");
+  return v;
+}
+
+// ------------------------------------------------------------------ LQ, panel by panel
+// Two kernels per panel of kLqPanel rows:
+//   * lq_panel_kernel factors the panel's rows inside one thread-block cluster, each CTA holding a
+//     range of their columns in shared memory.  A reflection needs one exchange: with x = row
+//     j, the sums s_r = sum_{c > j} x_c row_r[c] of all later rows and the pivot column p_r =
+//     row_r[j] give everything (|x|^2 = p_j^2 + s_j; v . row_r = p_r + scale s_r), so a step is
+//     partial sums, one cluster barrier, sums over the CTAs through distributed shared
+//     memory, the scalars in one warp, the update.
+//   * lq_rows_kernel applies the panel's reflections to the rows below, a few rows per block
+//     in shared memory, every reflection vector fetched ahead (cp.async) and used for all of
+//     the block's rows.  The same kernel forms Q from e_j.
+// Bound: the FP64 pipe in the rows (two multiply-adds per entry and reflection), latency in the
+// panel (~5000 cycles a reflection: chains of FP64 instructions at 64 cycles each, the cluster
+// exchange ~1000).  As one cooperative kernel, each reflection handed from the block that
+// owned a row to all others through device memory, a reflection took 13 us.
+// 597 x 2388: reflections 7.9 -> 5.6 ms (panels 2.8), Q 3.0 -> 2.6 ms; 256 x 1024: 2.63 -> 2.18
+// ms, the whole call.
+constexpr int kLqPanel = 32;
+constexpr int kLqCluster = 16;
+
+// Rows i0 .. i0 + b - 1 of A (columns from i0 on; b <= kLqPanel): reflections into V (row i from
+// column i0 on), tau, beta, and the panel's part of L into A (columns i0 .. i).  One cluster; CTA
+// q holds columns i0 + q chunk ...
+__global__ void __launch_bounds__(kFacThreads)
+lq_panel_kernel(double* A, int cols, int i0, int b, double* V, double* tau, double* beta) {
+  extern __shared__ double xs[];                       // [b][chunk]
+  __shared__ double part[2][2 * kLqPanel];             // sums and pivots, by step parity
+  __shared__ double tot[kLqPanel], piv[kLqPanel], fac[kLqPanel], sc[3];
+  const unsigned rank = cluster_rank(), cs = cluster_size();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ncol = cols - i0, chunk = (ncol + (int)cs - 1) / (int)cs;
+  const int lo = (int)rank * chunk, n = max(0, min(chunk, ncol - lo));
+  for (int e = tid; e < b * n; e += kFacThreads) {
+    const int r = e / n, c = e - r * n;
+    xs[r * chunk + c] = A[(size_t)(i0 + r) * cols + i0 + lo + c];
+  }
+  __syncthreads();
+  for (int j = 0; j < b; ++j) {
+    const double* x = xs + j * chunk;
+    double* pt = part[j & 1];
+    const int cb = max(0, j + 1 - lo);                 // first local column beyond the pivot
+    // ---- partial sums over this CTA's columns: warp w takes rows w, w + 8, w + 16, w + 24 (a
+    // branch per row: a predicated-off FP64 instruction costs as much as an active one)
+    {
+      double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = warp + 8 * u;
+        if (r < j || r >= b) continue;
+        const double* xr = xs + r * chunk;
+        double a0 = 0.0;
+        for (int c = cb + lane; c < n; c += 32) a0 = fma(xr[c], x[c], a0);
+        acc[u] = a0;
+      }
+      const double s = lq_warp_sum4(acc, lane);
+      const int r = warp + 8 * ((lane >> 3) & 3);
+      if ((lane & 7) == 0 && r >= j && r < b) pt[r] = s;
+      if (j >= lo && j < lo + n && tid >= j && tid < b) pt[kLqPanel + tid] = xs[tid * chunk + j - lo];
+    }
+    cluster_sync();
+    {
+      const int r = tid >> 3, q = tid & 7;
+      double s = 0.0;
+      if (r >= j && r < b)
+        for (unsigned k = q; k < cs; k += 8) s += ld_cluster(pt + r, k);
+#pragma unroll
+      for (int o = 4; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (q == 0 && r >= j && r < b) {
+        tot[r] = s;
+        piv[r] = ld_cluster(pt + kLqPanel + r, (unsigned)(j / chunk));
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {
+      double be, t, s;
+      lq_scalars(piv[j], tot[j], be, t, s);
+      // what row `lane` loses: t (p_r + scale s_r) at the pivot, that times scale x_c beyond
+      const double f = lane > j && lane < b ? t * fma(s, tot[lane], piv[lane]) : 0.0;
+      if (lane > j && lane < b) {
+        fac[lane] = f * s;
+        if (j >= lo && j < lo + n) xs[lane * chunk + j - lo] -= f;
+      }
+      if (lane == 0) {
+        sc[0] = t;
+        sc[1] = s;
+        sc[2] = be;
+        if (rank == 0) {
+          tau[i0 + j] = t;
+          beta[i0 + j] = be;
+        }
+      }
+    }
+    __syncthreads();
+    const double t = sc[0], scale = sc[1];
+    // ---- the vector, and row_r -= t (p_r + scale s_r) v for the rows below
+    double* vj = V + (size_t)(i0 + j) * cols + i0 + lo;
+    for (int c = tid; c < n; c += kFacThreads)
+      vj[c] = c < cb ? (lo + c == j ? 1.0 : 0.0) : x[c] * scale;
+    if (t != 0.0) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = warp + 8 * u;
+        if (r <= j || r >= b) continue;
+        double* xr = xs + r * chunk;
+        const double f = fac[r];
+        for (int c = cb + lane; c < n; c += 32) xr[c] = fma(-f, x[c], xr[c]);
+      }
+    }
+    if (tid == 0 && j >= lo && j < lo + n) xs[j * chunk + j - lo] = sc[2];
+    __syncthreads();
+  }
+  // the panel's rows of L: columns i0 .. i0 + r
+  for (int e = tid; e < b * min(b, n); e += kFacThreads) {
+    const int r = e / min(b, n), c = e - r * min(b, n);
+    if (lo + c <= r) A[(size_t)(i0 + r) * cols + i0 + lo + c] = xs[r * chunk + c];
+  }
+  cluster_sync();          // no CTA leaves while another may still read its sums
+}
+
+__device__ __forceinline__ void cp_async8(double* dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+
+// Rows multiplied from the right by reflections, rb (<= 8) rows per block in shared memory.
+struct RowsArgs {
+  double* X;               // element c of row r at X[r * sr + c * se], changed in place
+  long long sr, se;
+  int nrows, n;            // rows, columns
+  const double* V;         // vector of reflection i: V + i * ldv, zero before column i - cbase
+  long long ldv;
+  const double* tau;
+  int first, nref, step, cbase;   // reflections first, first + step, ... (nref of them)
+  const double* beta;      // set: form Q (X only written): row j = e_j^T H_j ... H_0, times the sign
+                           // that makes beta_j >= 0
+  int rb;
+};
+
+// One reflection on the first ACT rows of the block: sums over the row and the vector, one
+// block reduction, update.  (Inactive rows are left out at compile time: a predicated-off
+// FP64 instruction costs as much as an active one.)
+template <int ACT>
+__device__ void rows_reflect(double* sm, const double* v, int cb, int n, double t,
+                             double (*red)[8], double* dsh) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double acc[ACT <= 4 ? 4 : 8];
+#pragma unroll
+  for (int u = 0; u < (ACT <= 4 ? 4 : 8); ++u) acc[u] = 0.0;
+#pragma unroll 4
+  for (int c = cb + tid; c < n; c += kFacThreads) {
+    const double vc = v[c];
+#pragma unroll
+    for (int u = 0; u < ACT; ++u) acc[u] = fma(sm[(size_t)u * n + c], vc, acc[u]);
+  }
+  if constexpr (ACT == 1) {
+    const double s = lq_warp_sum(acc[0]);
+    if (lane == 0) red[0][warp] = s;
+  } else {
+    const double q4[4] = {acc[0], acc[1], acc[2], acc[3]};
+    const double s = lq_warp_sum4(q4, lane);
+    if ((lane & 7) == 0) red[lane >> 3][warp] = s;
+    if constexpr (ACT > 4) {
+      const double q5[4] = {acc[4], acc[5], acc[6], acc[7]};
+      const double s5 = lq_warp_sum4(q5, lane);
+      if ((lane & 7) == 0) red[4 + (lane >> 3)][warp] = s5;
+    }
+  }
+  __syncthreads();
+  if (warp < (ACT > 4 ? 2 : 1)) {
+    double s = red[tid >> 3][tid & 7];
+#pragma unroll
+    for (int o = 4; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((tid & 7) == 0) dsh[tid >> 3] = s * t;
+  }
+  __syncthreads();
+  double d[ACT];
+#pragma unroll
+  for (int u = 0; u < ACT; ++u) d[u] = dsh[u];
+#pragma unroll 4
+  for (int c = cb + tid; c < n; c += kFacThreads) {
+    const double vc = v[c];
+#pragma unroll
+    for (int u = 0; u < ACT; ++u)
+      sm[(size_t)u * n + c] = fma(-d[u], vc, sm[(size_t)u * n + c]);
+  }
+}
+
+__global__ void __launch_bounds__(kFacThreads) lq_rows_kernel(RowsArgs p) {
+  extern __shared__ double sm[];                       // rb rows, then two reflection vectors
+  __shared__ double red[8][8];
+  __shared__ double dsh[8];
+  const int tid = threadIdx.x, n = p.n;
+  double* vs = sm + (size_t)p.rb * n;
+  const bool form = p.beta != nullptr;
+  if (tid < 64) red[tid >> 3][tid & 7] = 0.0;
+  // row of slot u; when forming Q the last row first, so that the active ones are slots 0, 1, ...
+  auto row_of = [&](int u) {
+    return form ? (int)blockIdx.x + (int)gridDim.x * (p.rb - 1 - u) : (int)blockIdx.x * p.rb + u;
+  };
+  // slots with a row at all: when forming Q a suffix, else a prefix of 0 .. rb - 1
+  int u0 = 0, u1 = p.rb;
+  while (u0 < u1 && row_of(u0) >= p.nrows) ++u0;
+  while (u1 > u0 && row_of(u1 - 1) >= p.nrows) --u1;
+  if (u0 == u1) return;
+  for (int u = u0; u < u1; ++u) {
+    const int r = row_of(u);
+    for (int c = tid; c < n; c += kFacThreads)
+      sm[(size_t)u * n + c] =
+          form ? (c == r ? 1.0 : 0.0) : p.X[(long long)r * p.sr + (long long)c * p.se];
+  }
+  const int first = form ? row_of(u0) : p.first, count = form ? first + 1 : p.nref;
+  auto fetch = [&](int i, int q) {                     // vector i into buffer q
+    const double* v = p.V + (long long)i * p.ldv;
+    double* d = vs + (size_t)q * n;
+    for (int c = max(i - p.cbase, 0) + tid; c < n; c += kFacThreads) cp_async8(d + c, v + c);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  double tn = 0.0;                                     // tau of the next reflection
+  if (count > 0) {
+    fetch(first, 0);
+    tn = __ldg(p.tau + first);
+  }
+  for (int m = 0; m < count; ++m) {
+    const int i = first + p.step * m;
+    const double t = tn;
+    if (m + 1 < count) {
+      fetch(i + p.step, (m + 1) & 1);
+      tn = __ldg(p.tau + i + p.step);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    if (t != 0.0) {
+      int act = u1 - u0;                               // when forming Q the rows j >= i
+      if (form)
+        while (act > 1 && row_of(u0 + act - 1) < i) --act;
+      double* x = sm + (size_t)u0 * n;
+      const double* v = vs + (size_t)(m & 1) * n;
+      const int cb = max(i - p.cbase, 0);
+      switch (act) {
+        case 1: rows_reflect<1>(x, v, cb, n, t, red, dsh); break;
+        case 2: rows_reflect<2>(x, v, cb, n, t, red, dsh); break;
+        case 3: rows_reflect<3>(x, v, cb, n, t, red, dsh); break;
+        case 4: rows_reflect<4>(x, v, cb, n, t, red, dsh); break;
+        case 5: rows_reflect<5>(x, v, cb, n, t, red, dsh); break;
+        case 6: rows_reflect<6>(x, v, cb, n, t, red, dsh); break;
+        case 7: rows_reflect<7>(x, v, cb, n, t, red, dsh); break;
+        default: rows_reflect<8>(x, v, cb, n, t, red, dsh); break;
+      }
+    }
+    __syncthreads();       // the vector's buffer is refilled in the next round
+  }
+  for (int u = u0; u < u1; ++u) {
+    const int r = row_of(u);
+    const double sg = form && p.beta[r] < 0.0 ? -1.0 : 1.0;
+    for (int c = tid; c < n; c += kFacThreads)
+      p.X[(long long)r * p.sr + (long long)c * p.se] = sg * sm[(size_t)u * n + c];
+  }
+}
+
 // L[r][j] = A[r][j] for j <= r (j < k), 0 above; then diag(L) >= 0: where beta_j < 0 the
 // column j of L and the row j of Q change sign.
 __global__ void hh_extract_l_kernel(const double* A, int rows, int cols, int k,
@@ -1341,6 +1675,58 @@ void set_attributes() {
   });
 }
 
+namespace {
+
+constexpr size_t kLqSmem = 216 * 1024;
+
+// Cluster of CTAs for a panel of ncol columns: about 96 columns per CTA (a sum over 16 rows then
+// takes ~900 cycles, as long as the exchange), at most what the device can place.
+int lq_cluster(int ncol) {
+  static int most = 8;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    A2_CUDA(cudaFuncSetAttribute(lq_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kLqSmem));
+    A2_CUDA(cudaFuncSetAttribute(lq_panel_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kLqCluster);
+    cfg.blockDim = dim3(kFacThreads);
+    cfg.dynamicSmemBytes = kLqSmem;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kLqCluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int nclusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&nclusters, lq_panel_kernel, &cfg) == cudaSuccess &&
+        nclusters >= 1)
+      most = kLqCluster;
+    (void)cudaGetLastError();
+  });
+  int cs = 1;
+  while (cs < most && cs * 96 < ncol) cs *= 2;
+  return cs;
+}
+
+// Rows per block: as few as give every SM two blocks (one's reductions then overlap the other's
+// sums: 597 rows of Q in 2 x 152 blocks 2.56 ms, in 152 blocks 2.64 ms), as many as shared
+// memory holds.
+void lq_rows(RowsArgs p, cudaStream_t s) {
+  static std::once_flag once;
+  std::call_once(once, [] {
+    A2_CUDA(cudaFuncSetAttribute(lq_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kLqSmem));
+  });
+  const int fit = (int)(kLqSmem / (sizeof(double) * (size_t)p.n)) - 2;
+  p.rb = std::max(1, std::min({8, fit, cdiv(p.nrows, 2 * num_sms())}));
+  lq_rows_kernel<<<cdiv(p.nrows, p.rb), kFacThreads, sizeof(double) * (size_t)(p.rb + 2) * p.n, s>>>(
+      p);
+  A2_CHECK_LAUNCH();
+}
+
+}  // namespace
+
 int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double* P,
               double* discarded, std::vector<double>* sv_out, FactorWork& w, cudaStream_t s) {
   A2_REQUIRE(rows >= 1 && cols >= 1 && D_max >= 1, "SVD: bad sizes");
@@ -1527,36 +1913,64 @@ int hh_lq(const double* M, int rows, int cols, double* L, double* Q, FactorWork&
   ProfScope ps(PK_LQ, s, 4.0 * (double)rows * rows * cols, 8.0 * 3.0 * rows * (double)cols);
   w.a.ensure(sizeof(double) * (size_t)rows * cols, s);
   w.v.ensure(sizeof(double) * ((size_t)k * cols + 2 * (size_t)k), s);
-  w.bar.ensure(sizeof(GridBarrier) + sizeof(int) * (size_t)k, s);
   double* A = w.a.as<double>();
   double* V = w.v.as<double>();
   double* tau = V + (size_t)k * cols;
   double* beta = tau + k;
   A2_CUDA(cudaMemcpyAsync(A, M, sizeof(double) * (size_t)rows * cols, cudaMemcpyDeviceToDevice, s));
-  A2_CUDA(cudaMemsetAsync(w.bar.p, 0, sizeof(GridBarrier) + sizeof(int) * (size_t)k, s));
   set_attributes();
-  // cooperative launch: every block resident at once (the ready flags rely on it)
-  int per_sm = 0;
-  A2_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hh_lq_kernel, kFacThreads,
-                                                        vbytes));
-  A2_REQUIRE(per_sm >= 1, "LQ: kernel does not fit on an SM");
-  const int grid = std::max(1, std::min({rows, num_sms() * per_sm, num_sms()}));
-  GridBarrier* bar = w.bar.as<GridBarrier>();
-  int* ready = reinterpret_cast<int*>(bar + 1);
-  void* args[] = {&A, &rows, &cols, const_cast<int*>(&k), &V, &tau, &beta, &bar, &ready};
-  A2_CUDA(cudaLaunchCooperativeKernel((const void*)hh_lq_kernel, dim3(grid), dim3(kFacThreads),
-                                      args, vbytes, s));
-  count_launch();
-  hh_form_q_kernel<<<std::min(k, 4 * num_sms()), kFacThreads, vbytes, s>>>(V, tau, cols, k, Q);
-  A2_CHECK_LAUNCH();
+  if (3 * vbytes <= kLqSmem) {
+    for (int i0 = 0; i0 < k;) {
+      const int ncol = cols - i0, cs = lq_cluster(ncol), chunk = cdiv(ncol, cs);
+      const int b = std::min({kLqPanel, k - i0, (int)(kLqSmem / (sizeof(double) * chunk))});
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(cs);
+      cfg.blockDim = dim3(kFacThreads);
+      cfg.dynamicSmemBytes = sizeof(double) * (size_t)b * chunk;
+      cfg.stream = s;
+      cudaLaunchAttribute at;
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = cs;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      A2_CUDA(cudaLaunchKernelEx(&cfg, lq_panel_kernel, A, cols, i0, b, V, tau, beta));
+      A2_CHECK_LAUNCH();
+      if (i0 + b < rows)
+        lq_rows(RowsArgs{A + (size_t)(i0 + b) * cols + i0, cols, 1, rows - i0 - b, cols - i0, V + i0,
+                         cols, tau, i0, b, 1, i0, nullptr, 0},
+                s);
+      i0 += b;
+    }
+    lq_rows(RowsArgs{Q, cols, 1, k, cols, V, cols, tau, k - 1, k, -1, 0, beta, 0}, s);
+  } else {
+    // rows of more than 9200 entries (three do not fit in shared memory): the kernels that
+    // keep the rows in device memory
+    w.bar.ensure(sizeof(GridBarrier) + sizeof(int) * (size_t)k, s);
+    A2_CUDA(cudaMemsetAsync(w.bar.p, 0, sizeof(GridBarrier) + sizeof(int) * (size_t)k, s));
+    // cooperative launch: every block resident at once (the ready flags rely on it)
+    int per_sm = 0;
+    A2_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hh_lq_kernel, kFacThreads,
+                                                          vbytes));
+    A2_REQUIRE(per_sm >= 1, "LQ: kernel does not fit on an SM");
+    const int grid = std::max(1, std::min({rows, num_sms() * per_sm, num_sms()}));
+    GridBarrier* bar = w.bar.as<GridBarrier>();
+    int* ready = reinterpret_cast<int*>(bar + 1);
+    void* args[] = {&A, &rows, &cols, const_cast<int*>(&k), &V, &tau, &beta, &bar, &ready};
+    A2_CUDA(cudaLaunchCooperativeKernel((const void*)hh_lq_kernel, dim3(grid), dim3(kFacThreads),
+                                        args, vbytes, s));
+    count_launch();
+    hh_form_q_kernel<<<std::min(k, 4 * num_sms()), kFacThreads, vbytes, s>>>(V, tau, cols, k, Q);
+    A2_CHECK_LAUNCH();
+    hh_sign_rows_kernel<<<std::min(k, 1024), 128, 0, s>>>(Q, cols, k, beta);
+    A2_CHECK_LAUNCH();
+  }
   {
     const long long n = (long long)rows * k;
     const int g = (int)std::min<long long>((n + 255) / 256, 4096);
     hh_extract_l_kernel<<<std::max(g, 1), 256, 0, s>>>(A, rows, cols, k, beta, L);
     A2_CHECK_LAUNCH();
   }
-  hh_sign_rows_kernel<<<std::min(k, 1024), 128, 0, s>>>(Q, cols, k, beta);
-  A2_CHECK_LAUNCH();
   return k;
 }
 
