@@ -781,88 +781,146 @@ hh_bidiag_kernel(double* A, int m, int n, double* d, double* e, double* tau_u,
 // whole reduction (rows never change owner: row q of the block is global row b + nb * q,
 // held at rows[q * n]), in one grid barrier per step.  What crosses blocks goes through
 // global memory, published in step i - 1 for step i:
-//   the partial squared norms of column i below the diagonal (part, by step parity), the
-//   pivot A[i][i] (alpha) and row i itself (rowg, by step parity) from the owner of row i,
-//   and Z_i[c] = sum_{r > i} A[r][i] A[r][c], the unscaled products of the left reflection
+//   row i itself from its owner (rowg, by step parity; entry i is the pivot A[i][i]),
+//   and Z_i[c] = sum_{r > i} A[r][i] A[r][c] for c >= i, the unscaled products of the left
+//   reflection, Z_i[i] its squared norm.  The blocks of a thread-block cluster add up their parts
+//   through distributed shared memory and one of them adds the cluster's sum to global memory
 //   (FP64 atomics into one of three buffers, so Z may differ in its last bits from run to
 //   run).
 // Step i then runs in every block without further exchange: the left reflection
 // (beta, tau_u, scale) from the norm and the pivot, y = u^T A = row_i + scale Z_i (u_i = 1,
-// u_r = scale A[r][i]), the left update of its rows, the right reflection from row i after
-// the left update (x = row_i - tau_u y, formed by one warp while the others update the
-// rows; each row's left update also accumulates its dot product with x, so the right
-// update is one more pass over the row), the right update of its rows (one warp per row),
-// and the publications for step i + 1.  The scalar work of a reflection runs in one warp and
-// is broadcast through shared memory: an FP64 instruction holds a sub-partition's FP64
-// pipe for many cycles on this part, so the other warps must not repeat it.  At the end
-// the rows, holding the reflection vectors in place, are written back to A for the
-// back-transformation.  zbuf (3 n) must be zero on entry.
+// u_r = scale A[r][i]), the left update of its rows (one warp per row), the right reflection
+// from row i after the left update (x = row_i - tau_u y, formed by one warp while the others
+// update the rows; each row's left update also accumulates its dot product with x, so the right
+// update is one more pass over the row), the right update of its rows, and the publications
+// for step i + 1.  The scalar work of a reflection runs in one warp and is broadcast through
+// shared memory: an FP64 instruction holds a sub-partition's FP64 pipe for many cycles on this
+// part, so the other warps must not repeat it.  At the end the rows, holding the reflection
+// vectors in place, are written back to A for the back-transformation.  zbuf (3 n) must be
+// zero on entry.
+// Bound: the FP64 pipe (four multiply-adds per entry and step, 8.5 of the cycles below in
+// thousands) and the latency of a step.  Cycles per step at 1024 x 1024 with every block adding
+// its products itself: 27.7 thousand, of them 9.3 in the products and their 150000 atomics,
+// 6.1 in reading 148 partial norms and the reflection's scalars, 5.8 in the barrier of 148
+// arrivals; 13.4 ms in all.  With clusters of four a quarter of the atomics and arrivals
+// remain and the norm is one number: 10.5 ms (clusters of eight leave room for 120 blocks only:
+// 12.0); 796 x 597: 6.4 -> 5.1 ms.
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-// (beta, tau, scale) of the reflection mapping (al, x_1..) with sum x_k^2 = s2 onto
-// beta e_0: beta = -sign(al) sqrt(al^2 + s2), tau = (beta - al) / beta,
-// scale = 1 / (al - beta); tau = 0 (and beta = al) when s2 = 0.
-__device__ __forceinline__ void reflection_scalars(double al, double s2, double& beta,
-                                                   double& tau, double& scale) {
-  beta = al;
-  tau = 0.0;
-  scale = 0.0;
-  if (s2 > 0.0) {
-    const double nrm = sqrt(fma(al, al, s2));
-    beta = al >= 0.0 ? -nrm : nrm;
-    tau = (beta - al) / beta;
-    scale = 1.0 / (al - beta);
+// All blocks of the grid (clusters of cs) arrive before any leaves, as grid_sync, but one
+// arrival per cluster.  ok: this block's flag in shared memory, set to 0 by the cluster's first
+// block if the barrier gave up.
+__device__ bool grid_sync_clusters(GridBarrier* b, unsigned& epoch, unsigned rank, unsigned cs,
+                                   int* ok) {
+  ++epoch;
+  const unsigned target = epoch * (gridDim.x / cs);
+  cluster_sync();
+  if (rank == 0 && threadIdx.x == 0) {
+    bool good = true;
+    __threadfence();
+    atomicAdd(&b->count, 1u);
+    for (unsigned int it = 0;; ++it) {
+      if (*(volatile unsigned int*)&b->count >= target) break;
+      if (*(volatile int*)&b->abort) { good = false; break; }
+      if (it >= kBarrierLimit) {
+        atomicExch(&g_factor_error, 1);
+        atomicExch(&b->abort, 1);
+        good = false;
+        break;
+      }
+      if (it > 64) __nanosleep(32);
+    }
+    __threadfence();
+    if (!good)
+      for (unsigned q = 0; q < cs; ++q) {
+        const unsigned a = (unsigned)__cvta_generic_to_shared(ok);
+        unsigned ra;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(q));
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(ra), "r"(0) : "memory");
+      }
   }
+  cluster_sync();
+  return *(volatile int*)ok != 0;
 }
+
+constexpr int kBdCluster = 4;
+
 __global__ void __launch_bounds__(kFacThreads)
 hh_bidiag_smem_kernel(double* A, int m, int n, double* d, double* e, double* tau_u,
-                      double* tau_v, double* part, double* zbuf, double* alpha, double* rowg,
-                      GridBarrier* bar) {
+                      double* tau_v, double* zbuf, double* rowg, GridBarrier* bar) {
   unsigned epoch = 0;
   extern __shared__ double sm[];
   __shared__ double sc[4];                      // tau_u, scale_u, tau_v, scale_v
+  __shared__ double t2s[8];                     // partial norms of x beyond its pivot
+  __shared__ int ok;
+  const unsigned rank = cluster_rank(), cs = cluster_size();
   const int nb = gridDim.x, b = blockIdx.x, tid = threadIdx.x;
-  const int warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
-  const int R = (m - b + nb - 1) / nb;          // rows of this block
+  const int warp = tid >> 5, lane = tid & 31, nw = kFacThreads / 32;
+  const int R = b < m ? (m - b + nb - 1) / nb : 0;   // rows of this block
+  const int Rmax = (m + nb - 1) / nb;
   double* rows = sm;                            // R x n
-  double* yv = sm + (size_t)R * n;              // y of the current step (n)
+  double* yv = sm + (size_t)Rmax * n;           // y of the current step, the products at its end (n)
   double* wv = yv + n;                          // row i after the left update, x (n)
   double* zr = wv + n;                          // x . row_r beyond the superdiagonal (R)
+  if (tid == 0) ok = 1;
   for (int q = 0; q < R; ++q)
-    for (int c = tid; c < n; c += blockDim.x) rows[(size_t)q * n + c] = A[(size_t)(b + nb * q) * n + c];
+    for (int c = tid; c < n; c += kFacThreads) rows[(size_t)q * n + c] = A[(size_t)(b + nb * q) * n + c];
   __syncthreads();
   auto qof = [&](int r) { return (r - b) / nb; };            // r % nb == b assumed
   auto q_first = [&](int r0) { return r0 <= b ? 0 : (r0 - b + nb - 1) / nb; };   // first q with row >= r0
   // publications for step j (column j, row j) from this block's rows, which are final
-  // for step j: partial norm, unscaled products Z_j, and (owner of row j) row j and pivot
+  // for step j: the products Z_j and (owner of row j) row j
   auto publish = [&](int j) {
     const int qa = q_first(j + 1);
-    if (warp == 0) {
-      double p2 = 0.0;
-      for (int q = qa + lane; q < R; q += 32)
-        p2 = fma(rows[(size_t)q * n + j], rows[(size_t)q * n + j], p2);
-      p2 = warp_sum(p2);
-      if (lane == 0) part[(size_t)(j & 1) * nb + b] = p2;
-    }
-    if (qa < R) {
-      double* zj = zbuf + (size_t)(j % 3) * n;
-      for (int c = j + 1 + tid; c < n; c += blockDim.x) {
-        double acc = 0.0;
-        for (int q = qa; q < R; ++q) acc = fma(rows[(size_t)q * n + j], rows[(size_t)q * n + c], acc);
-        atomicAdd(zj + c, acc);
+    double* zj = zbuf + (size_t)(j % 3) * n;
+    for (int c = j + tid; c < n; c += 4 * kFacThreads) {   // four columns at a time
+      double acc[4] = {0.0, 0.0, 0.0, 0.0};
+      const int left = (n - c + kFacThreads - 1) / kFacThreads;
+      const double* rq = rows + (size_t)qa * n;
+      if (left >= 4) {
+#pragma unroll 2
+        for (int q = qa; q < R; ++q, rq += n) {
+          const double u = rq[j];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) acc[k] = fma(u, rq[c + k * kFacThreads], acc[k]);
+        }
+      } else {
+#pragma unroll 2
+        for (int q = qa; q < R; ++q, rq += n) {
+          const double u = rq[j];
+          acc[0] = fma(u, rq[c], acc[0]);
+          if (left > 1) acc[1] = fma(u, rq[c + kFacThreads], acc[1]);
+          if (left > 2) acc[2] = fma(u, rq[c + 2 * kFacThreads], acc[2]);
+        }
       }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (k < left) {
+          if (cs == 1) atomicAdd(zj + c + k * kFacThreads, acc[k]);
+          else yv[c + k * kFacThreads] = acc[k];
+        }
     }
     if (j % nb == b) {
       const double* rj = rows + (size_t)qof(j) * n;
       double* rn = rowg + (size_t)(j & 1) * n;
-      for (int c = j + 1 + tid; c < n; c += blockDim.x) rn[c] = rj[c];
-      if (tid == 0) alpha[j] = rj[j];
+      for (int c = j + tid; c < n; c += kFacThreads) rn[c] = rj[c];
+    }
+    if (cs > 1) {        // the cluster's sums, each block those of one range of columns
+      cluster_sync();
+      const int per = (n - j + (int)cs - 1) / (int)cs, c0 = j + (int)rank * per;
+      const int c1 = min(n, c0 + per);
+      for (int c = c0 + tid; c < c1; c += kFacThreads) {
+        double v[kBdCluster];
+#pragma unroll
+        for (int q = 0; q < kBdCluster; ++q) v[q] = ld_cluster(yv + c, q);
+        atomicAdd(zj + c, (v[0] + v[1]) + (v[2] + v[3]));
+      }
     }
   };
   publish(0);
-  if (!grid_sync(bar, epoch)) return;
+  if (!grid_sync_clusters(bar, epoch, rank, cs, &ok)) return;
   for (int i = 0; i < n; ++i) {
     const bool own_i = i % nb == b;
     const int q0 = q_first(i), q1 = q_first(i + 1);
@@ -870,12 +928,9 @@ hh_bidiag_smem_kernel(double* A, int m, int n, double* d, double* e, double* tau
     const double* rg = rowg + (size_t)(i & 1) * n;
     // ---- left reflection from column i (one warp per block forms it)
     if (warp == 0) {
-      const double al = __ldcg(alpha + i);
-      double s2 = 0.0;
-      for (int q = lane; q < nb; q += 32) s2 += __ldcg(part + (size_t)(i & 1) * nb + q);
-      s2 = warp_sum(s2);
+      const double al = __ldcg(rg + i), s2 = __ldcg(zi + i);
       double beta, tu, scale;
-      reflection_scalars(al, s2, beta, tu, scale);
+      lq_scalars(al, s2, beta, tu, scale);
       if (lane == 0) {
         sc[0] = tu;
         sc[1] = scale;
@@ -885,35 +940,54 @@ hh_bidiag_smem_kernel(double* A, int m, int n, double* d, double* e, double* tau
         }
       }
     }
-    // meanwhile: row i and Z_i into shared memory
-    for (int c = i + 1 + tid; c < n; c += blockDim.x) {
-      wv[c] = __ldcg(rg + c);
-      yv[c] = __ldcg(zi + c);
+    // meanwhile: row i and Z_i into shared memory (loads of a batch issued together)
+    for (int c = i + 1 + tid; c < n; c += 4 * kFacThreads) {
+      double w4[4], z4[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int cu = c + u * kFacThreads;
+        w4[u] = cu < n ? __ldcg(rg + cu) : 0.0;
+        z4[u] = cu < n ? __ldcg(zi + cu) : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int cu = c + u * kFacThreads;
+        if (cu < n) {
+          wv[cu] = w4[u];
+          yv[cu] = z4[u];
+        }
+      }
     }
     __syncthreads();
     const double tu = sc[0], scale = sc[1];
     // u below the diagonal (kept in place for the back-transformation)
     if (tu != 0.0)
-      for (int q = q1 + tid; q < R; q += blockDim.x) rows[(size_t)q * n + i] *= scale;
+      for (int q = q1 + tid; q < R; q += kFacThreads) rows[(size_t)q * n + i] *= scale;
     if (i + 1 >= n) break;
-    // y = row_i + scale Z_i; row i after the left update
-    for (int c = i + 1 + tid; c < n; c += blockDim.x) {
-      const double yc = fma(scale, yv[c], wv[c]);
-      yv[c] = yc;
-      wv[c] = fma(-tu, yc, wv[c]);
+    // y = row_i + scale Z_i; row i after the left update and its norm beyond the pivot
+    {
+      double t2 = 0.0;
+      for (int c = i + 1 + tid; c < n; c += kFacThreads) {
+        const double yc = fma(scale, yv[c], wv[c]);
+        const double xc = fma(-tu, yc, wv[c]);
+        yv[c] = yc;
+        wv[c] = xc;
+        if (c > i + 1) t2 = fma(xc, xc, t2);
+      }
+      t2 = warp_sum(t2);
+      if (lane == 0) t2s[warp] = t2;
     }
     __syncthreads();
-    // warp 0 forms the right reflection from x = row i after the left update (in wv)
-    // while warps 1.. apply the left update to the block's rows, one warp per row; a row
-    // r > i also accumulates its dot product with x beyond the superdiagonal, z_r, so that
+    // warp 0 forms the right reflection from x = row i after the left update (in wv) before it
+    // joins the others, which apply the left update to the block's rows, one warp per row; a
+    // row r > i also accumulates its dot product with x beyond the superdiagonal, z_r, so that
     // the right update needs no second pass over it: with w = (1, sv x_{i+2:}),
     // w . row_r = row_r[i+1] + sv z_r
     if (warp == 0) {
-      double t2 = 0.0;
-      for (int c = i + 2 + lane; c < n; c += 32) t2 = fma(wv[c], wv[c], t2);
-      t2 = warp_sum(t2);
+      double t2 = lane < nw ? t2s[lane] : 0.0;
+      for (int o = 4; o; o >>= 1) t2 += __shfl_xor_sync(0xffffffffu, t2, o);
       double be, tv, sv;
-      reflection_scalars(wv[i + 1], t2, be, tv, sv);
+      lq_scalars(wv[i + 1], t2, be, tv, sv);
       if (lane == 0) {
         sc[2] = tv;
         sc[3] = sv;
@@ -922,63 +996,73 @@ hh_bidiag_smem_kernel(double* A, int m, int n, double* d, double* e, double* tau
           tau_v[i] = tv;
         }
       }
-    } else {
-      const int cb = (i + 1) & ~31;
-      for (int q = q0 + warp - 1; q < R; q += nw - 1) {
-        const bool row_i = own_i && q == q0;
-        const double f = tu * (row_i ? 1.0 : rows[(size_t)q * n + i]);
-        double* rq = rows + (size_t)q * n;
-        double z0 = 0.0, z1 = 0.0;
-        for (int c = cb + lane; c < n; c += 64) {
-          if (c > i) {
-            const double v = tu != 0.0 ? fma(-f, yv[c], rq[c]) : rq[c];
-            rq[c] = v;
-            if (c > i + 1) z0 = fma(v, wv[c], z0);
-          }
-          if (c + 32 < n) {
-            const double v = tu != 0.0 ? fma(-f, yv[c + 32], rq[c + 32]) : rq[c + 32];
-            rq[c + 32] = v;
-            if (c + 32 > i + 1) z1 = fma(v, wv[c + 32], z1);
-          }
-        }
-        const double z = warp_sum(z0 + z1);
-        if (lane == 0) zr[q] = z;
+    }
+    const int cb = (i + 1) & ~31;
+    // rows from the last warp on, so that warp 0 has one row less where the count allows it
+    const int wr = nw - 1 - warp;
+    for (int q = q0 + wr; q < R; q += nw) {
+      const bool row_i = own_i && q == q0;
+      const double f = tu * (row_i ? 1.0 : rows[(size_t)q * n + i]);
+      double* rq = rows + (size_t)q * n;
+      double z0 = 0.0, z1 = 0.0;
+      int c = cb + lane;
+      if (c <= i + 1) {        // the pivot column i + 1 takes no part in z; columns <= i none at all
+        if (c == i + 1 && tu != 0.0) rq[c] = fma(-f, yv[c], rq[c]);
+        c += 32;
       }
+      if (tu != 0.0) {
+        for (; c + 32 < n; c += 64) {
+          const double v0 = fma(-f, yv[c], rq[c]), v1 = fma(-f, yv[c + 32], rq[c + 32]);
+          rq[c] = v0;
+          rq[c + 32] = v1;
+          z0 = fma(v0, wv[c], z0);
+          z1 = fma(v1, wv[c + 32], z1);
+        }
+        if (c < n) {
+          const double v0 = fma(-f, yv[c], rq[c]);
+          rq[c] = v0;
+          z0 = fma(v0, wv[c], z0);
+        }
+      } else {
+        for (; c < n; c += 32) z0 = fma(rq[c], wv[c], z0);
+      }
+      const double z = warp_sum(z0 + z1);
+      if (lane == 0) zr[q] = z;
     }
     __syncthreads();
     const double tv = sc[2], sv = sc[3];
     // right update of the own rows r > i: row_r -= tv (w . row_r) w, each warp on the rows
     // whose dot product it formed; the owner of row i stores w_i right of the superdiagonal
-    if (warp > 0) {
-      const int cb = (i + 1) & ~31;
-      for (int q = q0 + warp - 1; q < R; q += nw - 1) {
-        double* rq = rows + (size_t)q * n;
-        if (own_i && q == q0) {
-          for (int c = cb + lane; c < n; c += 32)
-            if (c > i + 1) rq[c] = sv * wv[c];
-          continue;
-        }
-        if (tv == 0.0) continue;
-        const double f = tv * fma(sv, zr[q], rq[i + 1]);
-        const double fs = f * sv;
-        __syncwarp();   // every lane has read rq[i + 1] before its owner changes it
-        for (int c = cb + lane; c < n; c += 32) {
-          if (c == i + 1) rq[c] -= f;
-          else if (c > i + 1) rq[c] = fma(-fs, wv[c], rq[c]);
-        }
+    for (int q = q0 + wr; q < R; q += nw) {
+      double* rq = rows + (size_t)q * n;
+      if (own_i && q == q0) {
+        for (int c = cb + lane; c < n; c += 32)
+          if (c > i + 1) rq[c] = sv * wv[c];
+        continue;
       }
+      if (tv == 0.0) continue;
+      const double f = tv * fma(sv, zr[q], rq[i + 1]);
+      const double fs = f * sv;
+      __syncwarp();   // every lane has read rq[i + 1] before its owner changes it
+      // (the pivot column apart: a branch inside the loop costs its FP64 instruction in every
+      // round)
+      if (lane == ((i + 1) & 31)) rq[i + 1] -= f;
+      int c = cb + lane;
+      if (c <= i + 1) c += 32;
+#pragma unroll 4
+      for (; c < n; c += 32) rq[c] = fma(-fs, wv[c], rq[c]);
     }
     __syncthreads();
     publish(i + 1);
     // the buffer read in step i - 1 is cleared for step i + 2
     double* zc = zbuf + (size_t)((i + 2) % 3) * n;
-    for (int c = b + nb * tid; c < n; c += nb * blockDim.x) zc[c] = 0.0;
-    if (!grid_sync(bar, epoch)) return;
+    for (int c = b + nb * tid; c < n; c += nb * kFacThreads) zc[c] = 0.0;
+    if (!grid_sync_clusters(bar, epoch, rank, cs, &ok)) return;
   }
   // rows back to A: u_i below the diagonals, w_i right of the superdiagonals
   __syncthreads();
   for (int q = 0; q < R; ++q)
-    for (int c = tid; c < n; c += blockDim.x) A[(size_t)(b + nb * q) * n + c] = rows[(size_t)q * n + c];
+    for (int c = tid; c < n; c += kFacThreads) A[(size_t)(b + nb * q) * n + c] = rows[(size_t)q * n + c];
 }
 
 // Golub-Kahan tridiagonal of B: zero diagonal, off-diagonal t = (d0, e0, d1, e1, ..., d_{n-1});
@@ -1021,8 +1105,10 @@ __device__ __forceinline__ double scale_exp(double v, int s) {
 __device__ __forceinline__ double flip_sign(double v) {
   return __longlong_as_double(__double_as_longlong(v) ^ (long long)0x8000000000000000ull);
 }
-template <typename R, int K>
-__device__ void tgk_count(const R* nt2, int N, const R (&xs)[K], int (&cnt)[K]) {
+// The last minor itself is pv[u] * 2^pe[u] where asked for.
+template <typename R, int K, bool VAL = false>
+__device__ void tgk_count(const R* nt2, int N, const R (&xs)[K], int (&cnt)[K],
+                          R* pv = nullptr, int* pe = nullptr) {
   constexpr int bias = sizeof(R) == 8 ? 1023 : 127;
   constexpr int E = sizeof(R) == 8 ? 256 : 32;
   constexpr int G = sizeof(R) == 8 ? 300 : 40;
@@ -1033,6 +1119,7 @@ __device__ void tgk_count(const R* nt2, int N, const R (&xs)[K], int (&cnt)[K]) 
     pm[u] = 1;
     p[u] = nxs[u];
     cnt[u] = xs[u] > 0;
+    if constexpr (VAL) pe[u] = 0;
   }
   for (int j = 1; j < N; ++j) {
     const R t = nt2[j];
@@ -1051,6 +1138,7 @@ __device__ void tgk_count(const R* nt2, int N, const R (&xs)[K], int (&cnt)[K]) 
       cnt[u] += sign_change(pn, p[u]);
       const int emax = max(expo(pn), expo(p[u]));
       if (emax > bias + E || emax < bias - E) {
+        if constexpr (VAL) pe[u] += emax - bias;
         if constexpr (sizeof(R) == 8) {
           pn = scale_exp(pn, bias - emax);
           p[u] = scale_exp(p[u], bias - emax);
@@ -1064,6 +1152,9 @@ __device__ void tgk_count(const R* nt2, int N, const R (&xs)[K], int (&cnt)[K]) 
       p[u] = pn;
     }
   }
+  if constexpr (VAL)
+#pragma unroll
+    for (int u = 0; u < K; ++u) pv[u] = p[u];
 }
 
 // Scale of the Golub-Kahan tridiagonal: 2^ex > max_j |t_j| + |t_{j+1}| (every warp forms
@@ -1147,7 +1238,9 @@ tgk_bisect32_kernel(const double* d, const double* e, int n, int nev, double* bl
 // checked with FP64 counts: half of the lanes test lower ends lo (1 - w_c), the other half
 // upper ends hi (1 + w_c), w_c from 2^-24 up to ~2^-9 (beyond the worst-case relative error
 // of the FP32 phase), and the tightest ends that hold are kept (0 or the bound when none
-// does); then L-lane multisection.  sigma[k] = midpoint, unscaled.
+// does); then two rounds with interpolation (below), then L-lane multisection where the
+// bracket is still wider.  sigma[k] = midpoint, unscaled.  Bound by the chain of a count (2 n
+// steps of two FP64 instructions): three rounds instead of six, 3.6 -> 1.1 ms for 1024 values.
 template <int L>
 __global__ void __launch_bounds__(128)
 tgk_refine64_kernel(const double* d, const double* e, int n, int nev, const double* blo,
@@ -1180,6 +1273,65 @@ tgk_refine64_kernel(const double* d, const double* e, int n, int nev, const doub
     if (!done) {
       if (lo_ok) lo = l0 * (1.0 - ldexp(1.0, -24 + step * (__ffs(lo_ok) - 1)));
       if (hi_ok) hi = fmin(h0 * (1.0 + ldexp(1.0, -24 + step * (__ffs(hi_ok) - 1))), 1.0);
+    }
+  }
+  for (int round = 0; round < 2; ++round) {
+    // L points from end to end with the value of the last minor, which changes sign at the
+    // eigenvalue; where the points around it isolate it (the counts differ by one), inverse
+    // quadratic interpolation through three of them, then counts at geometrically spaced
+    // distances from that point on both sides: whatever bracket they confirm is kept (the
+    // second round is for the few values that the first does not isolate)
+    double xs[1], pv[1] = {0.0};
+    int c[1] = {0}, pe[1] = {0};
+    if (!done && (hi - lo <= 0x1p-40 * hi || hi < 0x1p-600)) done = true;
+    if (__all_sync(0xffffffffu, done)) break;
+    const double step = (hi - lo) / (double)(L - 1);
+    xs[0] = sub == L - 1 ? hi : lo + step * (double)sub;
+    if (!done) tgk_count<double, 1, true>(nt2, N, xs, c, pv, pe);
+    const unsigned gmask = L == 32 ? 0xffffffffu : (1u << L) - 1u;
+    const int base = lane & (32 - L);
+    const unsigned up = (__ballot_sync(0xffffffffu, !done && c[0] > j) >> base) & gmask;
+    const int i1 = up ? __ffs(up) - 1 : L, i0 = i1 - 1;           // sign change between i0, i1
+    const int i2 = i1 + 1 < L ? i1 + 1 : i0 - 1;
+    auto at = [&](int i) { return base + min(max(i, 0), L - 1); };
+    const int c0 = __shfl_sync(0xffffffffu, c[0], at(i0)), c1 = __shfl_sync(0xffffffffu, c[0], at(i1));
+    const double f0 = __shfl_sync(0xffffffffu, pv[0], at(i0)), g1 = __shfl_sync(0xffffffffu, pv[0], at(i1)),
+                 g2 = __shfl_sync(0xffffffffu, pv[0], at(i2));
+    const int e0 = __shfl_sync(0xffffffffu, pe[0], at(i0)), e1 = __shfl_sync(0xffffffffu, pe[0], at(i1)),
+              e2 = __shfl_sync(0xffffffffu, pe[0], at(i2));
+    const double nlo = i1 == 0 ? lo : lo + step * (double)i0;
+    const double nhi = i1 >= L - 1 ? hi : lo + step * (double)i1;
+    bool isolated = !done && i1 > 0 && i1 < L && c0 == j && c1 == j + 1 && abs(e1 - e0) < 400 &&
+                    abs(e2 - e0) < 400;
+    double xst = 0.0;
+    if (isolated) {
+      const double f1 = ldexp(g1, e1 - e0), f2 = ldexp(g2, e2 - e0);
+      const double d2 = i2 > i1 ? 2.0 : -1.0;                     // abscissae 0, 1, d2 (in steps)
+      double t = f0 * f2 / ((f1 - f0) * (f1 - f2)) + d2 * f0 * f1 / ((f2 - f0) * (f2 - f1));
+      if (!(t >= 0.0 && t <= 1.0)) t = f0 / (f0 - f1);
+      xst = nlo + t * step;
+      isolated = t >= 0.0 && t <= 1.0;
+    }
+    if (!done) {
+      lo = nlo;
+      hi = nhi;
+    }
+    if (__any_sync(0xffffffffu, isolated)) {
+      constexpr int H = L / 2;
+      const int q = sub < H ? sub : sub - H;
+      const double w = xst * ldexp(1.0, -42 + q * (16 / H));
+      xs[0] = sub < H ? fmax(xst - w, lo) : fmin(xst + w, hi);
+      int cc[1] = {0};
+      if (isolated) tgk_count<double, 1>(nt2, N, xs, cc);
+      const bool good = isolated && (sub < H ? cc[0] <= j : cc[0] > j);
+      const unsigned grp = (__ballot_sync(0xffffffffu, good) >> base) & gmask;
+      const unsigned lo_ok = grp & ((1u << H) - 1u), hi_ok = grp >> H;
+      const int sl = lo_ok ? __ffs(lo_ok) - 1 : 0, sh = hi_ok ? H + __ffs(hi_ok) - 1 : 0;
+      const double xl = __shfl_sync(0xffffffffu, xs[0], base + sl), xh = __shfl_sync(0xffffffffu, xs[0], base + sh);
+      if (isolated) {
+        if (lo_ok) lo = xl;
+        if (hi_ok) hi = xh;
+      }
     }
   }
   for (int pass = 0; pass < 64; ++pass) {
@@ -1236,52 +1388,73 @@ __global__ void tgk_invit_kernel(const double* d, const double* e, int n, const 
     z[j] = (double)((h >> 11) & 0xFFFFF) / 1048576.0 - 0.5;
   }
   __syncwarp();
+  const bool normal = tmax > 1e-260 && tmax < 1e260;
+  auto rcp = [&](double q) { return normal ? lq_rcp(q) : 1.0 / q; };
+  // magnitudes compared as integers (an FP64 comparison costs a slot of the FP64 pipe)
+  auto mag = [](double q) { return __double_as_longlong(q) & 0x7fffffffffffffffll; };
+  const long long mtiny = mag(tiny);
   if (lane == 0) {
     // eliminate the subdiagonal entry T[j+1][j] = t(j + 1) column by column; the final
     // pivots are kept as their reciprocals for the substitutions
+    double dj = dg[0], s1j = s1[0];
     for (int j = 0; j + 1 < N; ++j) {
-      const double sub = t(j + 1);
-      if (fabs(dg[j]) >= fabs(sub)) {
-        if (fabs(dg[j]) < tiny) dg[j] = dg[j] < 0.0 ? -tiny : tiny;
-        const double inv = 1.0 / dg[j];
+      const double sub = t(j + 1), dn = dg[j + 1], r2 = j + 2 < N ? s1[j + 1] : 0.0;
+      if (mag(dj) >= mag(sub) || mag(sub) < mtiny) {
+        if (mag(dj) < mtiny) dj = __double_as_longlong(dj) < 0 ? -tiny : tiny;
+        const double inv = rcp(dj);
         const double f = sub * inv;
         ml[j] = f;
-        dg[j + 1] -= f * s1[j];
+        s1[j] = s1j;
         dg[j] = inv;
+        dj = fma(-f, s1j, dn);
+        s1j = r2;
       } else {                                // interchange rows j and j + 1
-        const double inv = 1.0 / sub;
-        const double f = dg[j] * inv;
-        const double r1 = dg[j + 1], r2 = j + 1 < N - 1 ? s1[j + 1] : 0.0;   // row j+1
-        dg[j] = inv;
-        const double old1 = s1[j];
-        s1[j] = r1;
-        s2[j] = r2;
-        dg[j + 1] = old1 - f * r1;
-        if (j + 1 < N - 1) s1[j + 1] = -f * r2;
+        const double inv = rcp(sub);
+        const double f = dj * inv;
         ml[j] = f;
         sw[j] = 1;
+        s1[j] = dn;
+        s2[j] = r2;
+        dg[j] = inv;
+        dj = fma(-f, dn, s1j);
+        s1j = -f * r2;
       }
     }
-    if (fabs(dg[N - 1]) < tiny) dg[N - 1] = dg[N - 1] < 0.0 ? -tiny : tiny;
-    dg[N - 1] = 1.0 / dg[N - 1];
+    if (mag(dj) < mtiny) dj = __double_as_longlong(dj) < 0 ? -tiny : tiny;
+    dg[N - 1] = rcp(dj);
+  }
+  __syncwarp();
+  // the superdiagonals times the reciprocal pivots: a step of the back substitution is then
+  // z_j = z_j / d_j - s1_j z_{j+1} - s2_j z_{j+2}, one dependent multiply-add
+  for (int j = lane; j < N; j += 32) {
+    s1[j] = j + 1 < N ? s1[j] * dg[j] : 0.0;
+    s2[j] = s2[j] * dg[j];
   }
   __syncwarp();
   for (int it = 0; it < 3; ++it) {
     if (lane == 0) {
-      for (int j = 0; j + 1 < N; ++j) {     // forward: row interchanges and multipliers
-        if (sw[j]) {
-          const double a = z[j];
-          z[j] = z[j + 1];
-          z[j + 1] = a - ml[j] * z[j];
-        } else {
-          z[j + 1] -= ml[j] * z[j];
-        }
+      double cur = z[0];
+#pragma unroll 4
+      for (int j = 0; j + 1 < N; ++j) {       // forward: row interchanges and multipliers
+        const double nx = z[j + 1];
+        const bool w = sw[j] != 0;
+        const double a = w ? nx : cur, c = w ? cur : nx;
+        z[j] = a;
+        cur = fma(-ml[j], a, c);
       }
-      for (int j = N - 1; j >= 0; --j) {    // backward: the banded upper factor
-        double v = z[j];
-        if (j + 1 < N) v -= s1[j] * z[j + 1];
-        if (j + 2 < N) v -= s2[j] * z[j + 2];
-        z[j] = v * dg[j];
+      z[N - 1] = cur;
+    }
+    __syncwarp();
+    for (int j = lane; j < N; j += 32) z[j] *= dg[j];
+    __syncwarp();
+    if (lane == 0) {
+      double z1 = 0.0, z2 = 0.0;
+#pragma unroll 4
+      for (int j = N - 1; j >= 0; --j) {      // backward: the banded upper factor
+        const double v = fma(-s1[j], z1, fma(-s2[j], z2, z[j]));
+        z[j] = v;
+        z2 = z1;
+        z1 = v;
       }
     }
     __syncwarp();
@@ -1388,6 +1561,28 @@ bidiag_apply_kernel(const double* A, int lda, int p, int q, const double* tau, i
         for (int v = 0; v < kApplyCols; ++v)
           if (k0 + v < r) X[(size_t)j * r + k0 + v] = x[v * p + j];
     __syncthreads();
+  }
+}
+
+// The bidiagonalisation's reflections as rows: V[i][j] (row length p) = 0 for j < i + off, 1 for
+// j = i + off, then A[j][i] (left, off = 0) or A[i][j] (right, off = 1).  32 x 32 tiles through
+// shared memory on the left side (a column of A per vector).
+__global__ void reflectors_kernel(const double* A, int lda, int p, int q, int left, double* V) {
+  __shared__ double tile[32][33];
+  const int j0 = blockIdx.x * 32, i0 = blockIdx.y * 32, off = left ? 0 : 1;
+  if (left) {
+    for (int t = threadIdx.y; t < 32; t += 8) {
+      const int j = j0 + t, i = i0 + threadIdx.x;
+      if (j < p && i < q && j > i) tile[t][threadIdx.x] = A[(size_t)j * lda + i];
+    }
+    __syncthreads();
+  }
+  for (int t = threadIdx.y; t < 32; t += 8) {
+    const int i = i0 + t, j = j0 + threadIdx.x;
+    if (i >= q || j >= p) continue;
+    double v = j == i + off ? 1.0 : 0.0;
+    if (j > i + off) v = left ? tile[threadIdx.x][t] : A[(size_t)i * lda + j];
+    V[(size_t)i * p + j] = v;
   }
 }
 
@@ -1671,7 +1866,7 @@ void set_attributes() {
     set_smem((const void*)tgk_refine64_kernel<16>, 200 * 1024);
     set_smem((const void*)tgk_refine64_kernel<32>, 200 * 1024);
     set_smem((const void*)tgk_invit_kernel, 200 * 1024);
-    set_smem((const void*)hh_bidiag_smem_kernel, 200 * 1024);
+    set_smem((const void*)hh_bidiag_smem_kernel, 224 * 1024);
   });
 }
 
@@ -1727,6 +1922,52 @@ void lq_rows(RowsArgs p, cudaStream_t s) {
 
 }  // namespace
 
+// Launch shape of the shared-memory bidiagonalisation: blocks (0: the rows do not fit), cluster
+// size and shared memory.  Clusters of kBdCluster where there are rows for two of them; the blocks
+// of all clusters that the device holds at once (about 144 of 152 SMs).
+struct BdShape {
+  int blocks = 0, cluster = 1;
+  size_t smem = 0;
+};
+BdShape bd_shape(int m, int n) {
+  constexpr size_t most = 224 * 1024;
+  auto bytes = [&](int nb) {
+    return sizeof(double) * (((size_t)cdiv(m, nb) + 2) * n + cdiv(m, nb));
+  };
+  BdShape sh;
+  // clusters that fit with one block per SM (asked once: the query takes milliseconds)
+  static int nclusters = 0;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(num_sms() / kBdCluster * kBdCluster);
+    cfg.blockDim = dim3(kFacThreads);
+    cfg.dynamicSmemBytes = most;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kBdCluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    A2_CUDA(cudaOccupancyMaxActiveClusters(&nclusters, hh_bidiag_smem_kernel, &cfg));
+  });
+  if (m >= 2 * kBdCluster) {
+    const int nb = std::min(m / kBdCluster, nclusters) * kBdCluster;
+    if (nb >= kBdCluster && bytes(nb) <= most) {
+      sh.blocks = nb;
+      sh.cluster = kBdCluster;
+      sh.smem = bytes(nb);
+      return sh;
+    }
+  }
+  const int nb = std::max(1, std::min(m, num_sms()));
+  if (bytes(nb) <= most) {
+    sh.blocks = nb;
+    sh.smem = bytes(nb);
+  }
+  return sh;
+}
+
 int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double* P,
               double* discarded, std::vector<double>* sv_out, FactorWork& w, cudaStream_t s) {
   A2_REQUIRE(rows >= 1 && cols >= 1 && D_max >= 1, "SVD: bad sizes");
@@ -1737,8 +1978,7 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
   const int m = left ? rows : cols, n = left ? cols : rows;
   const int nb = std::max(1, std::min(m, num_sms()));
   // scratch: A (m n); d, e, tau_u, tau_v (n each); sigma and its brackets (3n); y (n);
-  // Z by step modulo 3 (3n); pivots (n); published rows by step parity (2n); part by step
-  // parity (2 nb); ypart (nb n)
+  // Z by step modulo 3 (3n); published rows by step parity (2n); part (nb); ypart (nb n)
   const size_t nA = (size_t)m * n;
   w.a.ensure(sizeof(double) * nA, s);
   w.s.ensure(sizeof(double) * (14 * (size_t)n + 2 * nb + (size_t)nb * n), s);
@@ -1751,8 +1991,7 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
   double* sig = tv + n;
   double* y = sig + 3 * n;
   double* zbuf = y + n;
-  double* alpha = zbuf + 3 * n;
-  double* rowg = alpha + n;
+  double* rowg = zbuf + 3 * n;
   double* part = rowg + 2 * n;
   double* ypart = part + 2 * nb;
   if (left)
@@ -1764,12 +2003,24 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
   {
     GridBarrier* bar = w.bar.as<GridBarrier>();
     int mm = m, nn = n;
-    const size_t smem = sizeof(double) * (((size_t)cdiv(m, nb) + 2) * n + cdiv(m, nb));
-    if (smem <= 200 * 1024) {   // every block's rows resident in shared memory
+    const BdShape sh = bd_shape(m, n);
+    if (sh.blocks > 0) {   // every block's rows resident in shared memory
       A2_CUDA(cudaMemsetAsync(zbuf, 0, sizeof(double) * 3 * (size_t)n, s));
-      void* args[] = {&A, &mm, &nn, &d, &e, &tu, &tv, &part, &zbuf, &alpha, &rowg, &bar};
-      A2_CUDA(cudaLaunchCooperativeKernel((const void*)hh_bidiag_smem_kernel, dim3(nb),
-                                          dim3(kFacThreads), args, smem, s));
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(sh.blocks);
+      cfg.blockDim = dim3(kFacThreads);
+      cfg.dynamicSmemBytes = sh.smem;
+      cfg.stream = s;
+      cudaLaunchAttribute at[2];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = sh.cluster;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      at[1].id = cudaLaunchAttributeCooperative;
+      at[1].val.cooperative = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 2;
+      A2_CUDA(cudaLaunchKernelEx(&cfg, hh_bidiag_smem_kernel, A, mm, nn, d, e, tu, tv, zbuf, rowg,
+                                 bar));
     } else {
       void* args[] = {&A, &mm, &nn, &d, &e, &tu, &tv, &part, &ypart, &y, &bar};
       A2_CUDA(cudaLaunchCooperativeKernel((const void*)hh_bidiag_kernel, dim3(nb),
@@ -1787,14 +2038,14 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
     tgk_bisect32_kernel<32><<<cdiv(nev * 32, 128), 128, sizeof(float) * 2 * (size_t)n, s>>>(
         d, e, n, nev, blo, bhi);
     A2_CHECK_LAUNCH();
-    // lanes per value L of the FP64 phase: fewest passes (one to check the bracket, then
-    // ~21 bits / log2(2 L + 1)) times the warps that share a sub-partition's FP64 pipe
+    // lanes per value L of the FP64 phase: three passes (a few more values need a fourth when
+    // L is small) times the warps that share a sub-partition's FP64 pipe
     const size_t sm2 = sizeof(double) * 2 * (size_t)n;
     int best = 8;
     double best_cost = 1e300;
     for (int L : {8, 16, 32}) {
       const double share = std::ceil((double)cdiv(nev * L, 32) / (4.0 * num_sms()));
-      const double cost = (1.0 + std::ceil(21.0 / std::log2(2.0 * L + 1.0))) * std::max(1.0, share);
+      const double cost = (L == 32 ? 3.0 : L == 16 ? 3.2 : 3.6) * std::max(1.0, share);
       if (cost <= best_cost) { best_cost = cost; best = L; }
     }
     const int grid = cdiv(nev * best, 128);
@@ -1831,6 +2082,7 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
     return (int)std::max<long long>(32, (want + 31) / 32 * 32);
   };
   const size_t wmax = (size_t)cdiv(rows, 32) * r * W;      // partial sums of any Gram
+  w.x.ensure(sizeof(double) * (size_t)n * rows, s);
   w.v.ensure(sizeof(double) * ((size_t)r * n + (size_t)r * W + W * W + wmax) +
                  sizeof(int) * npan, s);
   double* vecs = w.v.as<double>();
@@ -1889,6 +2141,19 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
   // ones of M^T's (both act on R^rows)
   {
     const int q = left ? n : std::max(n - 1, 0);
+    if (3 * sizeof(double) * (size_t)rows <= kLqSmem) {
+      // the reflections as explicit rows, then a few columns of P per block in shared memory
+      // (lq_rows_kernel on P^T)
+      double* vx = w.x.as<double>();
+      reflectors_kernel<<<dim3(cdiv(rows, 32), cdiv(std::max(q, 1), 32)), dim3(32, 8), 0, s>>>(
+          A, n, rows, q, left ? 1 : 0, vx);
+      A2_CHECK_LAUNCH();
+      if (q > 0)
+        lq_rows(RowsArgs{P, 1, r, r, rows, vx, rows, left ? tu : tv, q - 1, q, -1, left ? 0 : -1,
+                         nullptr, 0},
+                s);
+      return r;
+    }
     // the block's columns in shared memory when they fit; reflections staged per pass: as
     // many as fit beside them (at most 16)
     const long long cap = 200LL * 1024 / 8;

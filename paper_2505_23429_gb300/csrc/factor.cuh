@@ -9,7 +9,7 @@ namespace a2 {
 
 // Scratch of the factorisations (grown on demand, owned by a context).
 struct FactorWork {
-  DevBuf a, v, s, bar;
+  DevBuf a, v, s, x, bar;
 };
 
 // LQ of a row-major (rows x cols) matrix M: M = L Q with Q (k x cols) orthonormal rows and

@@ -14,6 +14,7 @@ struct Solver {
     fw.a.release();
     fw.v.release();
     fw.s.release();
+    fw.x.release();
     fw.bar.release();
   }
   void set_stream(cudaStream_t s) { (void)s; }
