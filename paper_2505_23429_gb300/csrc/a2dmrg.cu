@@ -367,9 +367,10 @@ const T* as_compute(a2_ctx* c, const double* core, long long n, DevBuf& buf) {
 }
 
 // Left environment update (eq. env_L update): Hin [Dlb][Rl][Dlk] -> Hout [Drb][Rr][Drk].
+// Returns its first stage Hin . ket as [(a w)][(t b')], valid until the context's next update.
 template <typename T>
-void env_left(a2_ctx* c, const SiteOps& so, const T* Hin, const T* bra, int Dlb, int Drb,
-              const T* ket, int Dlk, int Drk, T* Hout) {
+const T* env_left(a2_ctx* c, const SiteOps& so, const T* Hin, const T* bra, int Dlb, int Drb,
+                  const T* ket, int Dlk, int Drk, T* Hout) {
   const int n = so.n, Rl = so.Rl, Rr = so.Rr;
   cudaStream_t s = c->stream;
   ProfScope ps(PK_ENV, s, env_flops(so, std::max(Dlb, Dlk), std::max(Drb, Drk)),
@@ -403,6 +404,7 @@ void env_left(a2_ctx* c, const SiteOps& so, const T* Hin, const T* bra, int Dlb,
     g.C = Hout; g.scm = (long long)Rr * Drk; g.scn = 1;
     simt_gemm(g, s);
   }
+  return T1;
 }
 
 // Right environment update (eq. env_R update): Hin [Drb][Rr][Drk] -> Hout [Dlb][Rl][Dlk].
@@ -2496,26 +2498,10 @@ struct Sweeper {
     tt->dims = xd;
   }
 };
-
-template <typename T>
-double energy_T(a2_ctx* c, const a2_tt* tt, const a2_mpo* mpo, double* norm_out,
-                a2_precision prec = A2_FP64) {
-  Engine<T> eng(c, mpo, prec);
+// <tt|tt> by transfer matrices in FP64.
+double norm2_transfer(a2_ctx* c, const a2_tt* tt) {
   cudaStream_t s = c->stream;
   const int L = tt->L;
-  DevBuf E, En;
-  eng.set_unit(E);
-  for (int j = 0; j < L; ++j) {
-    const int Dl = tt->dims[j], Dr = tt->dims[j + 1];
-    En.ensure(sizeof(T) * (size_t)Dr * mpo->R[j + 1] * Dr, s);
-    eng.left_update(E.as<T>(), j, tt->cores[j].as<double>(), Dl, Dr, tt->cores[j].as<double>(),
-                    Dl, Dr, En.as<T>());
-    std::swap(E, En);
-  }
-  T e;
-  A2_CUDA(cudaMemcpyAsync(&e, E.p, sizeof(T), cudaMemcpyDeviceToHost, s));
-  A2_CUDA(cudaStreamSynchronize(s));
-  // norm by transfer matrices in FP64
   DevBuf N, Nn, Tm;
   N.ensure(sizeof(double), s);
   const double one = 1.0;
@@ -2537,6 +2523,28 @@ double energy_T(a2_ctx* c, const a2_tt* tt, const a2_mpo* mpo, double* norm_out,
   A2_CUDA(cudaMemcpyAsync(&nn, N.p, sizeof(double), cudaMemcpyDeviceToHost, s));
   A2_CUDA(cudaStreamSynchronize(s));
   check_finite(nn, "norm");
+  return nn;
+}
+
+template <typename T>
+double energy_T(a2_ctx* c, const a2_tt* tt, const a2_mpo* mpo, double* norm_out,
+                a2_precision prec = A2_FP64) {
+  Engine<T> eng(c, mpo, prec);
+  cudaStream_t s = c->stream;
+  const int L = tt->L;
+  DevBuf E, En;
+  eng.set_unit(E);
+  for (int j = 0; j < L; ++j) {
+    const int Dl = tt->dims[j], Dr = tt->dims[j + 1];
+    En.ensure(sizeof(T) * (size_t)Dr * mpo->R[j + 1] * Dr, s);
+    eng.left_update(E.as<T>(), j, tt->cores[j].as<double>(), Dl, Dr, tt->cores[j].as<double>(),
+                    Dl, Dr, En.as<T>());
+    std::swap(E, En);
+  }
+  T e;
+  A2_CUDA(cudaMemcpyAsync(&e, E.p, sizeof(T), cudaMemcpyDeviceToHost, s));
+  A2_CUDA(cudaStreamSynchronize(s));
+  const double nn = norm2_transfer(c, tt);
   if (norm_out) *norm_out = std::sqrt(std::max(nn, 0.0));
   return (double)e / nn;
 }
@@ -2615,45 +2623,46 @@ uint64_t splitmix_next(uint64_t& state) {
 // Adjoint of the energy sandwich with respect to one MPO core (the Hellmann-Feynman
 // derivative at a fixed TT): G[w,s,t,w'] = sum HL[a,w,a'] U[a,s,b] U[a',t,b'] HR[b,w',b']
 // with HL the environment of the sites left of the core and HR of those right of it,
-// both built from the same TT (any gauge).  FP64 SIMT contractions:
-//   X[a,w,t,b'] = sum_a' HL U;  Z[(s b)][(w t b')] = sum_a U X;
-//   G[w,s,t,w'] = sum_{b,b'} Z HR   (batched over b, one launch per (s, t)).
-void core_gradient(a2_ctx* c, const double* HL, int Dl, int Rl, const double* U, int n, int Dr,
-                   const double* HR, int Rr, double* G, DevBuf& bx, DevBuf& bz) {
-  cudaStream_t s = c->stream;
-  bx.ensure(sizeof(double) * (size_t)Dl * Rl * n * Dr, s);
-  bz.ensure(sizeof(double) * (size_t)n * Dr * Rl * n * Dr, s);
-  double* X = bx.as<double>();
-  double* Z = bz.as<double>();
-  const long long nD = (long long)n * Dr, RnD = (long long)Rl * n * Dr;
-  {
-    SimtGemm<double, double> g;
-    g.M = Dl * Rl; g.N = (int)nD; g.K = Dl;
-    g.A = HL; g.sam = Dl; g.sak = 1;
-    g.B = U; g.sbn = 1; g.sbk = nD;
-    g.C = X; g.scm = nD; g.scn = 1;
-    simt_gemm(g, s);
-  }
-  {
-    SimtGemm<double, double> g;
-    g.M = (int)nD; g.N = (int)RnD; g.K = Dl;
-    g.A = U; g.sam = 1; g.sak = nD;
-    g.B = X; g.sbn = 1; g.sbk = RnD;
-    g.C = Z; g.scm = RnD; g.scn = 1;
-    simt_gemm(g, s);
-  }
-  fill_zero(G, sizeof(double) * (size_t)Rl * n * n * Rr, s);
-  for (int sx = 0; sx < n; ++sx)
-    for (int t = 0; t < n; ++t) {
-      SimtGemm<double, double> g;
-      g.M = Rl; g.N = Rr; g.K = Dr;
-      g.A = Z + (long long)sx * Dr * RnD + (long long)t * Dr; g.sam = nD; g.sak = 1;
-      g.B = HR; g.sbn = Dr; g.sbk = 1;
-      g.C = G + ((long long)sx * n + t) * Rr; g.scm = (long long)n * n * Rr; g.scn = 1;
-      g.batch = Dr; g.abs = RnD; g.bbs = (long long)Rr * Dr; g.cbs = 0;
-      g.mode = GEMM_ATOMIC;
-      simt_gemm(g, s);
+// both built from the same TT (any gauge).  A map names few of the n^2 Rl Rr elements (3 to
+// 4 % of a chemistry core), so G is not formed: with
+//   X[a,w,t,b'] = sum_a' HL U (the first stage of the left environment's update) and
+//   Y[a,s,w',b'] = sum_b U HR for the w' that the map names,
+// element (w,s,t,w') is the dot product over (a, b') of rows of X and Y.
+// L = 8 chemistry, D = 64, all 4160 integrals: 12.7 -> 3.4 ms a call, of them 2.3 in the FP64
+// products of the environments and of Y and 0.14 in the dot products; forming G took 7 and a
+// separate chain for the energy 1.3 (the left chain is now closed instead).
+// Elements that the map names on one core, each once, in the order of their first entry.
+struct GradElems {
+  std::vector<int4> el;               // (w, s, t, place of w' in wr)
+  std::vector<int> wr;                // the w' that occur, in rising order
+};
+// es: map entries of the site; place[e] becomes base + the element's number.
+GradElems grad_elems(const std::vector<long long>& es, const long long* index, int n, int Rr,
+                     long long base, std::vector<long long>& place, size_t at) {
+  GradElems g;
+  int bits = 4;
+  while ((1ull << bits) < 2 * es.size()) ++bits;
+  const size_t mask = (1ull << bits) - 1;
+  std::vector<std::pair<long long, int>> table(mask + 1, {-1, 0});   // open addressing
+  std::vector<int> wplace(Rr, -1);
+  for (long long e : es) wplace[index[e] % Rr] = 0;
+  for (int w = 0; w < Rr; ++w)
+    if (wplace[w] == 0) {
+      wplace[w] = (int)g.wr.size();
+      g.wr.push_back(w);
     }
+  for (size_t q = 0; q < es.size(); ++q) {
+    const long long u = index[es[q]];
+    size_t h = (size_t)((unsigned long long)u * 0x9E3779B97F4A7C15ull >> (64 - bits));
+    while (table[h].first >= 0 && table[h].first != u) h = (h + 1) & mask;
+    if (table[h].first < 0) {
+      const int wr = (int)(u % Rr), st = (int)(u / Rr % ((long long)n * n));
+      table[h] = {u, (int)g.el.size()};
+      g.el.push_back(int4{(int)(u / Rr / ((long long)n * n)), st / n, st % n, wplace[wr]});
+    }
+    place[at + q] = base + table[h].second;
+  }
+  return g;
 }
 
 }  // namespace
@@ -3182,59 +3191,86 @@ a2_status a2_energy_gradient(a2_ctx* c, const a2_tt* t, const a2_mpo* m, long lo
                  map_param[e] < nparam, "a2_energy_gradient: map entry out of range");
       by_site[j].push_back(e);
     }
-    double nrm = 0.0;
-    const double E = energy_T<double>(c, t, m, &nrm);
-    const double n2 = nrm * nrm;
+    const double n2 = norm2_transfer(c, t);
     A2_REQUIRE(n2 > 0.0, "a2_energy_gradient: zero TT");
     Engine<double> eng(c, m, A2_FP64);
     // right environments of every suffix
     std::vector<DevBuf> HR(L + 1);
     eng.set_unit(HR[L]);
+    DevBuf grad, HL, HLn, HRp, Y, el, wr, part, g, mp, mi, mf;
+    eng.set_unit(HL);
     for (int j = L - 1; j >= 1; --j) {
       const int Dl = t->dims[j], Dr = t->dims[j + 1];
       HR[j].ensure(sizeof(double) * (size_t)Dl * m->R[j] * Dl, s);
       eng.right_update(HR[j + 1].as<double>(), j, t->cores[j].as<double>(), Dl, Dr,
                        t->cores[j].as<double>(), Dl, Dr, HR[j].as<double>());
     }
-    DevBuf grad, HL, HLn, G, bx, bz, mp, mi, mf;
+    // while those run: the elements of every core, the map in terms of them
+    std::vector<GradElems> ge(L);
+    std::vector<size_t> el_at(L + 1, 0), wr_at(L + 1, 0);
+    std::vector<long long> hp(nmap), hi(nmap);
+    std::vector<double> hf(nmap);
+    std::vector<int4> hel;
+    std::vector<int> hwr;
+    for (size_t j = 0, q = 0; j < (size_t)L; q += by_site[j].size(), ++j) {
+      ge[j] = grad_elems(by_site[j], map_index, t->phys[j], m->R[j + 1], (long long)hel.size(),
+                         hi, q);
+      for (size_t k = 0; k < by_site[j].size(); ++k) {
+        hp[q + k] = map_param[by_site[j][k]];
+        hf[q + k] = map_factor[by_site[j][k]] / n2;
+      }
+      hel.insert(hel.end(), ge[j].el.begin(), ge[j].el.end());
+      hwr.insert(hwr.end(), ge[j].wr.begin(), ge[j].wr.end());
+      el_at[j + 1] = hel.size();
+      wr_at[j + 1] = hwr.size();
+    }
+    upload(mp, hp.data(), sizeof(long long) * hp.size(), s);
+    upload(mi, hi.data(), sizeof(long long) * hi.size(), s);
+    upload(mf, hf.data(), sizeof(double) * hf.size(), s);
+    upload(el, hel.data(), sizeof(int4) * hel.size(), s);
+    upload(wr, hwr.data(), sizeof(int) * hwr.size(), s);
+    g.ensure(sizeof(double) * hel.size(), s);
     grad.ensure(sizeof(double) * (size_t)nparam, s);
     fill_zero(grad.p, sizeof(double) * (size_t)nparam, s);
-    eng.set_unit(HL);
     for (int j = 0; j < L; ++j) {
       const int Dl = t->dims[j], n = t->phys[j], Dr = t->dims[j + 1];
       const int Rl = m->R[j], Rr = m->R[j + 1];
-      if (!by_site[j].empty()) {
-        G.ensure(sizeof(double) * (size_t)Rl * n * n * Rr, s);
-        core_gradient(c, HL.as<double>(), Dl, Rl, t->cores[j].as<double>(), n, Dr,
-                      HR[j + 1].as<double>(), Rr, G.as<double>(), bx, bz);
-        const auto& es = by_site[j];
-        const size_t ne = es.size();
-        std::vector<long long> hp(ne), hi(ne);
-        std::vector<double> hf(ne);
-        for (size_t q = 0; q < ne; ++q) {
-          hp[q] = map_param[es[q]];
-          hi[q] = map_index[es[q]];
-          hf[q] = map_factor[es[q]] / n2;
+      const double* U = t->cores[j].as<double>();
+      // the last update closes the sandwich
+      HLn.ensure(sizeof(double) * (size_t)Dr * Rr * Dr, s);
+      const double* X = env_left<double>(c, m->site[j], HL.as<double>(), U, Dl, Dr, U, Dl, Dr,
+                                         HLn.as<double>());
+      const int nel = (int)ge[j].el.size(), nw = (int)ge[j].wr.size();
+      if (nel) {
+        const double* H = HR[j + 1].as<double>();
+        if (nw < Rr) {
+          HRp.ensure(sizeof(double) * (size_t)Dr * nw * Dr, s);
+          gather_mid(H, Dr, Rr, Dr, wr.as<int>() + wr_at[j], nw, HRp.as<double>(), s);
+          H = HRp.as<double>();
         }
-        upload(mp, hp.data(), sizeof(long long) * ne, s);
-        upload(mi, hi.data(), sizeof(long long) * ne, s);
-        upload(mf, hf.data(), sizeof(double) * ne, s);
-        gather_axpy_atomic(G.as<double>(), mi.as<long long>(), mp.as<long long>(),
-                           mf.as<double>(), (long long)ne, grad.as<double>(), s);
-        A2_CUDA(cudaStreamSynchronize(s));     // the host staging vectors go out of scope
+        Y.ensure(sizeof(double) * (size_t)Dl * n * nw * Dr, s);
+        SimtGemm<double, double> gy;          // Y[(a s)][(q b')] = sum_b U[(a s)][b] H[b][(q b')]
+        gy.M = Dl * n; gy.N = nw * Dr; gy.K = Dr;
+        gy.A = U; gy.sam = Dr; gy.sak = 1;
+        gy.B = H; gy.sbn = 1; gy.sbk = (long long)nw * Dr;
+        gy.C = Y.as<double>(); gy.scm = (long long)nw * Dr; gy.scn = 1;
+        simt_gemm(gy, s);
+        const int parts = grad_dot_parts(Dl, Dr, Rl, nw, n, nel);
+        part.ensure(sizeof(double) * (size_t)parts * nel, s);
+        grad_dots(X, Y.as<double>(), el.as<int4>() + el_at[j], nel, Dl, Rl, n, nw, Dr, parts,
+                  part.as<double>(), g.as<double>() + el_at[j], s);
       }
-      if (j + 1 < L) {
-        HLn.ensure(sizeof(double) * (size_t)Dr * m->R[j + 1] * Dr, s);
-        eng.left_update(HL.as<double>(), j, t->cores[j].as<double>(), Dl, Dr,
-                        t->cores[j].as<double>(), Dl, Dr, HLn.as<double>());
-        std::swap(HL, HLn);
-        HR[j + 1].release();
-      }
+      std::swap(HL, HLn);
+      HR[j + 1].release();
     }
+    double E = 0.0;
+    A2_CUDA(cudaMemcpyAsync(&E, HL.p, sizeof(double), cudaMemcpyDeviceToHost, s));
+    gather_axpy_atomic(g.as<double>(), mi.as<long long>(), mp.as<long long>(), mf.as<double>(),
+                       nmap, grad.as<double>(), s);
     A2_CUDA(cudaMemcpyAsync(grad_out, grad.p, sizeof(double) * (size_t)nparam,
                             cudaMemcpyDeviceToHost, s));
     A2_CUDA(cudaStreamSynchronize(s));
-    if (E_out) *E_out = E;
+    if (E_out) *E_out = E / n2;
   });
 }
 

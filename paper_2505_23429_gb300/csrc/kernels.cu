@@ -1438,6 +1438,95 @@ void gather_axpy_atomic(const double* G, const long long* index, const long long
   A2_CHECK_LAUNCH();
 }
 
+// out[a][q][b] = in[a][list[q]][b], in [A][R][B], out [A][nq][B].
+__global__ void gather_mid_kernel(const double* __restrict__ in, int R, int B,
+                                  const int* __restrict__ list, int nq, double* out) {
+  const double* src = in + ((long long)blockIdx.y * R + list[blockIdx.x]) * B;
+  double* dst = out + ((long long)blockIdx.y * nq + blockIdx.x) * B;
+  for (int b = threadIdx.x; b < B; b += blockDim.x) dst[b] = src[b];
+}
+void gather_mid(const double* in, int A, int R, int B, const int* list, int nq, double* out,
+                cudaStream_t s) {
+  for (int a0 = 0; a0 < A; a0 += 32768)
+    gather_mid_kernel<<<dim3(nq, std::min(A - a0, 32768)), 128, 0, s>>>(
+        in + (long long)a0 * R * B, R, B, list, nq, out + (long long)a0 * nq * B);
+  A2_CHECK_LAUNCH();
+}
+
+// Elements of the energy's derivative with respect to an MPO core, el = (w, s, t, q): the dot
+// product of X[.][w][t][.] and Y[.][s][q][.] over (a, b'), X [Dl][Rl][n][Dr], Y [Dl][n][nw][Dr].
+// One warp per element and part of the a range; the parts are outermost, so that the warps
+// that run at one time share the slices of X and Y that they read (through L2; the FP64 pipe
+// is the bound: 64 cycles a warp instruction against 512 bytes).  Parts are added in order.
+__global__ void __launch_bounds__(256)
+grad_dots_kernel(const double* __restrict__ X, const double* __restrict__ Y,
+                 const int4* __restrict__ el, int nel, int Dl, int Rl, int n, int nw, int Dr,
+                 int parts, double* __restrict__ out) {
+  const long long id = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (id >= (long long)nel * parts) return;
+  const int p = (int)(id / nel);
+  const int4 e = __ldg(el + id % nel);
+  const int a0 = (int)((long long)Dl * p / parts), a1 = (int)((long long)Dl * (p + 1) / parts);
+  const long long sx = (long long)Rl * n * Dr, sy = (long long)n * nw * Dr;
+  const double* x = X + a0 * sx + ((long long)e.x * n + e.z) * Dr;
+  const double* y = Y + a0 * sy + ((long long)e.y * nw + e.w) * Dr;
+  const long long total = (long long)(a1 - a0) * Dr;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  long long i = lane;
+  int a = lane / Dr, b = lane % Dr;                    // i = a Dr + b
+  const int da = 32 / Dr, db = 32 % Dr;
+  auto next = [&] {
+    a += da;
+    b += db;
+    if (b >= Dr) { b -= Dr; ++a; }
+  };
+  for (; i + 96 < total; i += 128) {                   // four loads of each in flight
+    double xv[4], yv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      xv[u] = __ldg(x + a * sx + b);
+      yv[u] = __ldg(y + a * sy + b);
+      next();
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[u] = fma(xv[u], yv[u], acc[u]);
+  }
+  for (; i < total; i += 32) {
+    acc[0] = fma(__ldg(x + a * sx + b), __ldg(y + a * sy + b), acc[0]);
+    next();
+  }
+  double v = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) out[id] = v;
+}
+__global__ void sum_parts_kernel(const double* __restrict__ in, int n, int parts,
+                                 double* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double v = 0.0;
+  for (int p = 0; p < parts; ++p) v += in[(long long)p * n + i];
+  out[i] = v;
+}
+// Parts of the a range: four warps for every sub-partition's share of the chip, and slices of
+// X and Y of at most 64 MB (half of L2).
+int grad_dot_parts(int Dl, int Dr, int Rl, int nw, int n, int nel) {
+  const long long bytes = 8LL * Dl * n * Dr * ((long long)Rl + nw);
+  const long long want = std::max<long long>(cdiv(16 * simt_sms(), nel), (bytes >> 26) + 1);
+  return (int)std::min<long long>(want, Dl);
+}
+void grad_dots(const double* X, const double* Y, const int4* el, int nel, int Dl, int Rl, int n,
+               int nw, int Dr, int parts, double* part, double* out, cudaStream_t s) {
+  const long long warps = (long long)nel * parts;
+  grad_dots_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(X, Y, el, nel, Dl, Rl, n, nw, Dr,
+                                                               parts, parts > 1 ? part : out);
+  A2_CHECK_LAUNCH();
+  if (parts > 1) {
+    sum_parts_kernel<<<cdiv(nel, 256), 256, 0, s>>>(part, nel, parts, out);
+    A2_CHECK_LAUNCH();
+  }
+}
+
 void fill_zero(void* p, size_t bytes, cudaStream_t s) {
   if (bytes) A2_CUDA(cudaMemsetAsync(p, 0, bytes, s));
 }

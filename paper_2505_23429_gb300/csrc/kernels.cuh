@@ -162,6 +162,12 @@ void sparse_rows_apply_df(const SparseRows<float>& sp, const SparseGeom& g, cons
 // grad[param[e]] += factor[e] * G[index[e]] for e < n (FP64 atomics)
 void gather_axpy_atomic(const double* G, const long long* index, const long long* param,
                         const double* factor, long long n, double* grad, cudaStream_t s);
+void gather_mid(const double* in, int A, int R, int B, const int* list, int nq, double* out,
+                cudaStream_t s);
+int grad_dot_parts(int Dl, int Dr, int Rl, int nw, int n, int nel);
+// out[i]: element el[i]; part: parts * nel values of scratch.
+void grad_dots(const double* X, const double* Y, const int4* el, int nel, int Dl, int Rl, int n,
+               int nw, int Dr, int parts, double* part, double* out, cudaStream_t s);
 void sign_fix_qr(double* Q, int ldq, int rows, double* R, int ldr, int k, cudaStream_t s);
 void scale_rows(double* M, int rows, int cols, const double* svals, cudaStream_t s); // M[r,:]*=s[r]
 // TT-sum block copy: dst[(o0 + i)*dst_s0 + j*dst_s1 + o2 + k] = alpha * src[i][j][k]
