@@ -363,10 +363,13 @@ __device__ __forceinline__ double ld_cluster(const double* p, unsigned rank) {
 // panel (~5000 cycles a reflection: chains of FP64 instructions at 64 cycles each, the cluster
 // exchange ~1000).  As one cooperative kernel, each reflection handed from the block that
 // owned a row to all others through device memory, a reflection took 13 us.
-// 597 x 2388: reflections 7.9 -> 5.6 ms (panels 2.8), Q 3.0 -> 2.6 ms; 256 x 1024: 2.63 -> 2.18
-// ms, the whole call.
+// 597 x 2388: reflections 7.9 -> 5.6 ms (panels 2.8), Q 3.0 -> 2.6 ms; with the next panel beside
+// the update of the rows below it 5.1 (forming Q beside the panels as well gains nothing: it
+// takes the FP64 pipe from them).  The whole call at 256 x 1024 2.63 -> 2.15 ms, 1024 x 256 1.78 ->
+// 1.77 (1.90 one after the other).
 constexpr int kLqPanel = 32;
 constexpr int kLqCluster = 16;
+constexpr int kLqAhead = 64;       // rows below the next panel that are worth a second stream
 
 // Rows i0 .. i0 + b - 1 of A (columns from i0 on; b <= kLqPanel): reflections into V (row i from
 // column i0 on), tau, beta, and the panel's part of L into A (columns i0 .. i).  One cluster; CTA
@@ -1906,15 +1909,16 @@ int lq_cluster(int ncol) {
 
 // Rows per block: as few as give every SM two blocks (one's reductions then overlap the other's
 // sums: 597 rows of Q in 2 x 152 blocks 2.56 ms, in 152 blocks 2.64 ms), as many as shared
-// memory holds.
-void lq_rows(RowsArgs p, cudaStream_t s) {
+// memory holds.  Beside a panel (per_sm 1) one block per SM, so that the panel's cluster finds
+// room.
+void lq_rows(RowsArgs p, cudaStream_t s, int per_sm = 2) {
   static std::once_flag once;
   std::call_once(once, [] {
     A2_CUDA(cudaFuncSetAttribute(lq_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kLqSmem));
   });
   const int fit = (int)(kLqSmem / (sizeof(double) * (size_t)p.n)) - 2;
-  p.rb = std::max(1, std::min({8, fit, cdiv(p.nrows, 2 * num_sms())}));
+  p.rb = std::max(1, std::min({8, fit, cdiv(p.nrows, per_sm * num_sms())}));
   lq_rows_kernel<<<cdiv(p.nrows, p.rb), kFacThreads, sizeof(double) * (size_t)(p.rb + 2) * p.n, s>>>(
       p);
   A2_CHECK_LAUNCH();
@@ -2185,6 +2189,22 @@ int hh_lq(const double* M, int rows, int cols, double* L, double* Q, FactorWork&
   A2_CUDA(cudaMemcpyAsync(A, M, sizeof(double) * (size_t)rows * cols, cudaMemcpyDeviceToDevice, s));
   set_attributes();
   if (3 * vbytes <= kLqSmem) {
+    // A panel's reflections go to the rows of the next panel first; the next panel then runs
+    // beside the update of the other rows, on the second stream (a panel is bound by latency and
+    // takes at most 16 SMs).
+    SideStream& side = w.side;
+    bool pending = false;                    // the second stream has work that s did not wait for
+    struct Join {                            // also when a launch throws
+      SideStream& side;
+      bool& pending;
+      ~Join() {
+        if (pending) cudaStreamSynchronize(side.s);
+      }
+    } join{side, pending};
+    auto wait_side = [&] {
+      if (pending) A2_CUDA(cudaStreamWaitEvent(s, side.done, 0));
+      pending = false;
+    };
     for (int i0 = 0; i0 < k;) {
       const int ncol = cols - i0, cs = lq_cluster(ncol), chunk = cdiv(ncol, cs);
       const int b = std::min({kLqPanel, k - i0, (int)(kLqSmem / (sizeof(double) * chunk))});
@@ -2201,12 +2221,29 @@ int hh_lq(const double* M, int rows, int cols, double* L, double* Q, FactorWork&
       cfg.numAttrs = 1;
       A2_CUDA(cudaLaunchKernelEx(&cfg, lq_panel_kernel, A, cols, i0, b, V, tau, beta));
       A2_CHECK_LAUNCH();
-      if (i0 + b < rows)
-        lq_rows(RowsArgs{A + (size_t)(i0 + b) * cols + i0, cols, 1, rows - i0 - b, cols - i0, V + i0,
-                         cols, tau, i0, b, 1, i0, nullptr, 0},
-                s);
+      const int first = i0 + b, below = rows - first;
+      auto update = [&](int row, int nrows, cudaStream_t st, int per_sm) {
+        lq_rows(RowsArgs{A + (size_t)row * cols + i0, cols, 1, nrows, cols - i0, V + i0, cols, tau, i0,
+                         b, 1, i0, nullptr, 0},
+                st, per_sm);
+      };
+      const int next = std::min(below, kLqPanel);
+      if (first < k && below - next >= kLqAhead) {
+        side.ensure();
+        A2_CUDA(cudaEventRecord(side.start, s));
+        wait_side();
+        update(first, next, s, 2);
+        A2_CUDA(cudaStreamWaitEvent(side.s, side.start, 0));
+        pending = true;
+        update(first + next, below - next, side.s, 1);
+        A2_CUDA(cudaEventRecord(side.done, side.s));
+      } else {
+        wait_side();
+        if (below > 0) update(first, below, s, 2);
+      }
       i0 += b;
     }
+    wait_side();
     lq_rows(RowsArgs{Q, cols, 1, k, cols, V, cols, tau, k - 1, k, -1, 0, beta, 0}, s);
   } else {
     // rows of more than 9200 entries (three do not fit in shared memory): the kernels that

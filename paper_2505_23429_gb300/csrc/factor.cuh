@@ -7,9 +7,29 @@
 
 namespace a2 {
 
+// A second stream beside the caller's, with the events that fork and join it (created at the
+// first use; never left with work that the caller's stream has not waited for).
+struct SideStream {
+  cudaStream_t s = nullptr;
+  cudaEvent_t start = nullptr, done = nullptr;
+  void ensure() {
+    if (!s) A2_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    if (!start) A2_CUDA(cudaEventCreateWithFlags(&start, cudaEventDisableTiming));
+    if (!done) A2_CUDA(cudaEventCreateWithFlags(&done, cudaEventDisableTiming));
+  }
+  void release() {
+    if (start) cudaEventDestroy(start);
+    if (done) cudaEventDestroy(done);
+    if (s) cudaStreamDestroy(s);
+    s = nullptr;
+    start = done = nullptr;
+  }
+};
+
 // Scratch of the factorisations (grown on demand, owned by a context).
 struct FactorWork {
   DevBuf a, v, s, x, bar;
+  SideStream side;
 };
 
 // LQ of a row-major (rows x cols) matrix M: M = L Q with Q (k x cols) orthonormal rows and

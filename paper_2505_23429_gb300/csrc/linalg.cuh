@@ -16,6 +16,7 @@ struct Solver {
     fw.s.release();
     fw.x.release();
     fw.bar.release();
+    fw.side.release();
   }
   void set_stream(cudaStream_t s) { (void)s; }
   // LQ of a row-major (rows x cols) matrix M: M = L Q, Q (k x cols) orthonormal rows,
