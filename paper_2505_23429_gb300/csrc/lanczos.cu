@@ -161,19 +161,68 @@ __device__ void lz_dots(const double* V, long long ld, const double* x, int n, i
   }
 }
 
-// tot[q] = sum over the workers of part[q * stride + i], q < kk, in a fixed order: four
-// threads per value, combined by one.
+// One warp's share of lz_totals: M values (warp, warp + 8, ...), U rounds of 32 workers of each
+// loaded at a time.
+template <int M, int U>
+__device__ __forceinline__ void lz_total_loop(const double* part, int workers, int stride, int warp,
+                                              int lane, int mine, double (&acc)[8]) {
+  for (int i = 0; i < workers; i += 32 * U) {
+    double v[M][U];
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        v[m][u] = m < mine && i + 32 * u + lane < workers
+                      ? __ldcg(part + (long long)(warp + 8 * m) * stride + i + 32 * u + lane)
+                      : 0.0;
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+      if (m < mine)
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (i + 32 * u < workers) acc[m] += v[m][u];   // (uniform: no add that does nothing)
+  }
+}
+
+// tot[q] = sum over the workers of part[q * stride + i], q < kk, in a fixed order.  WIDE (above 64
+// workers): a warp takes every eighth value and its lanes the workers; four threads per value,
+// each adding a quarter of the partial sums one after the other, wait for 38 loads and adds at
+// 150 workers (chemistry L = 8, D = 64, mean of a sweep's steps: 28.3 -> 26.3 us).  With fewer the
+// four threads are the faster form, as they need no sums over a warp (Heisenberg, D = 32, 32
+// workers: 24.5 us, by warps 25.7).
+template <bool WIDE>
 __device__ void lz_totals(const double* part, int workers, int stride, int kk, double* tot,
                           double (*red)[64]) {
-  const int q = threadIdx.x & 63, sl = threadIdx.x >> 6;
-  double t = 0.0;
-  if (q < kk)
-    for (int i = sl; i < workers; i += 4) t += __ldcg(part + (long long)q * stride + i);
-  red[sl][q] = t;
-  __syncthreads();
-  if (threadIdx.x < kk)
-    tot[threadIdx.x] = (red[0][threadIdx.x] + red[1][threadIdx.x]) +
-                       (red[2][threadIdx.x] + red[3][threadIdx.x]);
+  if constexpr (!WIDE) {
+    const int q = threadIdx.x & 63, sl = threadIdx.x >> 6;
+    double t = 0.0;
+    if (q < kk)
+      for (int i = sl; i < workers; i += 4) t += __ldcg(part + (long long)q * stride + i);
+    red[sl][q] = t;
+    __syncthreads();
+    if (threadIdx.x < kk)
+      tot[threadIdx.x] = (red[0][threadIdx.x] + red[1][threadIdx.x]) +
+                         (red[2][threadIdx.x] + red[3][threadIdx.x]);
+    __syncthreads();
+    return;
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int mine = (kk - warp + 7) / 8;
+  double acc[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) acc[u] = 0.0;
+  if (mine > 4) lz_total_loop<8, 2>(part, workers, stride, warp, lane, mine, acc);
+  else if (mine > 2) lz_total_loop<4, 5>(part, workers, stride, warp, lane, mine, acc);
+  else if (mine > 1) lz_total_loop<2, 5>(part, workers, stride, warp, lane, mine, acc);
+  else if (mine > 0) lz_total_loop<1, 5>(part, workers, stride, warp, lane, mine, acc);
+  if (mine > 1) {
+    const double s = warp_sum8(acc, lane);
+    const int m = warp_sum8_index(lane);
+    if ((lane & 3) == 0 && m < mine) tot[warp + 8 * m] = s;
+  } else if (mine > 0) {
+    const double s = warp_sum_d(acc[0]);
+    if (lane == 0) tot[warp] = s;
+  }
   __syncthreads();
 }
 
@@ -508,6 +557,7 @@ __device__ void tri_lowest(TriShared& S, int k) {
   }
 }
 
+template <bool WIDE>
 __global__ void __launch_bounds__(kLzThreads) lanczos_step_kernel(LzArgs p) {
   extern __shared__ __align__(16) double lz_smem[];
   const int tid = threadIdx.x, b = blockIdx.x, G = p.workers;
@@ -529,7 +579,7 @@ __global__ void __launch_bounds__(kLzThreads) lanczos_step_kernel(LzArgs p) {
       if (tid == 0) p.out[4] = 1.0;
       return;
     }
-    lz_totals(part_a, G, G, 1, tot, red);
+    lz_totals<WIDE>(part_a, G, G, 1, tot, red);
     if (tid == 0) {
       S.a[k - 1] = tot[0];
       p.tri[k - 1] = tot[0];
@@ -565,7 +615,7 @@ __global__ void __launch_bounds__(kLzThreads) lanczos_step_kernel(LzArgs p) {
     if (tid == 0) p.out[4] = 1.0;
     return;
   }
-  lz_totals(part_a, G, G, 1, tot, red);
+  lz_totals<WIDE>(part_a, G, G, 1, tot, red);
   const double alpha = tot[0];
   // ---- w -= alpha v_j + beta v_{j-1}
   {
@@ -587,7 +637,7 @@ __global__ void __launch_bounds__(kLzThreads) lanczos_step_kernel(LzArgs p) {
       if (tid == 0) p.out[4] = 1.0;
       return;
     }
-    lz_totals(part_h, G, G, k + 1, tot, red);
+    lz_totals<WIDE>(part_h, G, G, k + 1, tot, red);
     if (tid < k) h[tid] = tot[tid];
     const double n1 = tot[k];
     __syncthreads();
@@ -629,7 +679,7 @@ __global__ void __launch_bounds__(kLzThreads) lanczos_step_kernel(LzArgs p) {
       if (tid == 0) p.out[4] = 1.0;
       return;
     }
-    lz_totals(part_n, G, G, 1, tot, red);
+    lz_totals<WIDE>(part_n, G, G, 1, tot, red);
     n2 = tot[0];
     __syncthreads();
     if (!(n2 < 0.5 * n1)) break;
@@ -695,8 +745,9 @@ void lanczos_step(double* V, double* w, long long N, int j, double beta_prev, bo
     int dev = 0;
     A2_CUDA(cudaGetDevice(&dev));
     A2_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    A2_CUDA(cudaFuncSetAttribute(lanczos_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kSliceMax));
+    for (const void* f : {(const void*)lanczos_step_kernel<false>,
+                          (const void*)lanczos_step_kernel<true>})
+      A2_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSliceMax));
   });
   const int most = std::max(1, std::min(sms - 1, kReduceBlocks / 2));
   LzArgs p;
@@ -720,8 +771,9 @@ void lanczos_step(double* V, double* w, long long N, int j, double beta_prev, bo
   const size_t smem = std::max(sizeof(TriShared),
                                p.in_smem ? sizeof(double) * (size_t)chunk : (size_t)0);
   void* args[] = {&p};
-  A2_CUDA(cudaLaunchCooperativeKernel((const void*)lanczos_step_kernel, dim3(p.workers + 1),
-                                      dim3(kLzThreads), args, smem, s));
+  const void* kernel = p.workers > 64 ? (const void*)lanczos_step_kernel<true>
+                                      : (const void*)lanczos_step_kernel<false>;
+  A2_CUDA(cudaLaunchCooperativeKernel(kernel, dim3(p.workers + 1), dim3(kLzThreads), args, smem, s));
   A2_CHECK_LAUNCH();
 }
 
