@@ -384,14 +384,14 @@ def class_roofline(name, d, peaks, prec):
         return "tensor", "TFLOP/s", peaks["bf16_sus"], rate_f
     if name in ("sparse_s2", "sparse_s3", "emu_s2", "emu_s3", "lanczos", "f64e_split"):
         return "hbm", "GB/s", peaks["hbm"], rate_b
-    if name in ("f64e_s1", "f64e_s4"):   # 36 BF16 products per FP64-equivalent flop
-        return "tensor", "TFLOP/s", peaks["bf16_sus"], 36.0 * rate_f
+    if name in ("f64e_s1", "f64e_s4"):   # 28 BF16 products per FP64-equivalent flop
+        return "tensor", "TFLOP/s", peaks["bf16_sus"], 28.0 * rate_f
     if name == "f64e_sparse":
         return "alu", "TFLOP/s", FP32_SIMT_PEAK_TFLOPS, rate_f
     if name == "env" and prec in ("bf16", "f32emu", "f64emu"):
-        # FP64-class environments: the two GEMMs of an update Ozaki-emulated (36 BF16
+        # FP64-class environments: the two GEMMs of an update Ozaki-emulated (28 BF16
         # products per FP64-equivalent flop), small updates on the FP64 SIMT kernels
-        return "tensor", "TFLOP/s", peaks["bf16_sus"], 36.0 * rate_f
+        return "tensor", "TFLOP/s", peaks["bf16_sus"], 28.0 * rate_f
     if name in ("heff_simt", "env") and prec != "fp64":
         return "alu", "TFLOP/s", FP32_SIMT_PEAK_TFLOPS, rate_f
     return "alu", "TFLOP/s", FP64_PEAK_TFLOPS, rate_f        # FP64 factorisations / SIMT

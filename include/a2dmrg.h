@@ -61,9 +61,10 @@ typedef enum {
                    three BF16 slices, six slice pairs accumulated in FP32; environments,
                    refinement and coarse problem as in A2_BF16 */
   A2_F64EMU = 5  /* H_eff to FP64-class accuracy (~2^-48) on tcgen05 (Ozaki scheme): FP64
-                   operands split row-wise into eight 7-bit BF16 slices, the 36 slice
-                   pairs of level <= 9 accumulated exactly in FP32 per level and K chunk,
-                   the partial tiles summed by error-free two-sums into FP32 pairs; the
+                   operands split row by row and 256 entries at a time into seven slices
+                   of balanced 8-bit digits (BF16), the 28 slice pairs of level <= 8
+                   accumulated in FP32 per 256 entries (exact up to the two highest levels'
+                   units of 2^-46) and summed by error-free two-sums into FP32 pairs; the
                    sparse MPO stages in double-float (FP32 pairs); environments FP64,
                    their updates emulated the same way (two Ozaki GEMMs and a double-float
                    sparse stage) above a small size, plain FP64 below; vectors, SVD and
