@@ -603,6 +603,13 @@ __global__ void __launch_bounds__(kFacThreads) lq_rows_kernel(RowsArgs p) {
         case 7: rows_reflect<7>(x, v, cb, n, t, red, dsh); break;
         default: rows_reflect<8>(x, v, cb, n, t, red, dsh); break;
       }
+    } else if (form) {
+      // no reflection (zero vector): the row's own 0 v is kept, so that a NaN in the matrix
+      // reaches Q
+      for (int u = u0; u < u1; ++u)
+        if (row_of(u) == i)
+          for (int c = max(i - p.cbase, 0) + tid; c < n; c += kFacThreads)
+            sm[(size_t)u * n + c] -= t * vs[(size_t)(m & 1) * n + c];
     }
     __syncthreads();       // the vector's buffer is refilled in the next round
   }

@@ -32,3 +32,17 @@ def test_lq(rows, cols):
     assert np.abs(Q @ Q.T - np.eye(k)).max() < tol
     assert np.all(np.diag(L) >= 0.0) and np.abs(np.triu(L, 1)).max() == 0.0
     ctx.close()
+
+
+# a NaN in a row reaches that row of Q, in the first panel and in a later one
+@pytest.mark.parametrize("cols", [64, 9300])
+@pytest.mark.parametrize("row", [5, 37])
+def test_lq_nan_is_visible(row, cols):
+    ctx = a2.Context(0)
+    M = np.random.default_rng(1).standard_normal((40, cols))
+    M[row, 50] = np.nan
+    L = torch.zeros((40, 40), dtype=torch.float64, device="cuda")
+    Q = torch.zeros((40, cols), dtype=torch.float64, device="cuda")
+    a2.lq(ctx, dev(M), L, Q)
+    assert np.isnan(host(Q, ctx)[row]).any()
+    ctx.close()
