@@ -299,7 +299,11 @@ void st_launch_vec(const StArgs& a, bool vec, dim3 grid, size_t smem, cudaStream
 // they are bound by arithmetic and want the second block (bond 7, D = 128: S2 + S3 5.35 ms
 // against 5.78 with one).  FP32 inputs stay with the general kernels, which gather them at 10 TB/s and
 // were as fast or faster (bond 5: S2 1.10 ms both, S3 1.53 against 1.71; bond 7: S2 1.92
-// against 2.33).
+// against 2.33).  BF16 rows that are not whole 16-byte vectors are copied element by element,
+// which pays with long rows only (16 nonzeros or more on average; S3 at Dl, Dr = 40, 98: 0.100 ms
+// against 0.152; short ones 107, 234: 0.254 against 0.196; 41, 44: 0.054 against 0.029); under 128
+// blocks the general kernels, with one warp a row, spread better (S2 at 45, 26, 90 blocks: 13.6 us
+// against 10.1).
 bool sparse_staged(const SparseRows<float>& sp, const SparseGeom& g, int in_kind, const void* in,
                    long long in_plane, int out_kind, void* out, long long out_plane,
                    cudaStream_t s) {
@@ -330,6 +334,8 @@ bool sparse_staged(const SparseRows<float>& sp, const SparseGeom& g, int in_kind
                    al(g.out_b2) && al(out_plane) &&
                    reinterpret_cast<uintptr_t>(in) % (isz * nv) == 0 &&
                    reinterpret_cast<uintptr_t>(out) % std::min(16, osz * nv) == 0;
+  if (in_kind == ST_BF16 && (blocks < 128 || (!vec && sp.nnz_total < 16LL * sp.nrows)))
+    return false;
   StArgs a;
   a.sp = sp;
   a.g = g;
