@@ -157,11 +157,10 @@ simt_gemm_kernel(SimtGemm<T, OutT> g) {
   const int kg = tid / NG, tg = tid % NG;
   const int tx = tg % GX, ty = tg / GX;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const int z = blockIdx.z;
-  const int b = z / g.splitk, sk = z % g.splitk;
-  const T* A = g.A + (long long)b * g.abs;
-  const T* B = g.B + (long long)b * g.bbs;
-  OutT* C = g.C + (long long)b * g.cbs;
+  const int sk = blockIdx.z;
+  const T* A = g.A;
+  const T* B = g.B;
+  OutT* C = g.C;
   const int kchunk = ((g.K + g.splitk - 1) / g.splitk + BK - 1) / BK * BK;
   const int kbeg = sk * kchunk;
   const int kend = min(g.K, kbeg + kchunk);
@@ -287,7 +286,7 @@ static int simt_sms() {
 
 template <typename T, typename OutT, int BM, int BN, int BK, int TM, int TN, int KG>
 static void simt_launch(const SimtGemm<T, OutT>& g, cudaStream_t s) {
-  dim3 grid(cdiv(g.N, BN), cdiv(g.M, BM), g.batch * g.splitk);
+  dim3 grid(cdiv(g.N, BN), cdiv(g.M, BM), g.splitk);
   A2_REQUIRE(grid.y < 65536 && grid.z < 65536, "GEMM grid too large");
   simt_gemm_kernel<T, OutT, BM, BN, BK, TM, TN, KG>
       <<<grid, (BM / TM) * (BN / TN) * KG, 0, s>>>(g);
@@ -296,12 +295,12 @@ static void simt_launch(const SimtGemm<T, OutT>& g, cudaStream_t s) {
 // Index of the tile edge (of `edges`, descending) with the least work on the busiest SM:
 // rounds of blocks over the SMs times the tile's area, divided by the tile's relative
 // efficiency.  A smaller tile also has to gain something (its loads per product are more).
-static int pick_tile(int M, int N, long long batch, const int* edges, const double* eff, int n) {
+static int pick_tile(int M, int N, int splitk, const int* edges, const double* eff, int n) {
   const int sms = simt_sms();
   int best = 0;
   double best_cost = 0.0;
   for (int i = 0; i < n; ++i) {
-    const long long ty = cdiv(M, edges[i]), tiles = ty * cdiv(N, edges[i]) * batch;
+    const long long ty = cdiv(M, edges[i]), tiles = ty * cdiv(N, edges[i]) * splitk;
     if (i > 0 && ty >= 65536) break;
     const double cost =
         (double)((tiles + sms - 1) / sms) * edges[i] * edges[i] / eff[i];
@@ -321,13 +320,12 @@ static int pick_tile(int M, int N, long long batch, const int* edges, const doub
 // more, which is what bounds them, hence the large ones.
 template <typename T, typename OutT>
 void simt_gemm(const SimtGemm<T, OutT>& g, cudaStream_t s) {
-  if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
+  if (g.M <= 0 || g.N <= 0) return;
   A2_REQUIRE(g.splitk == 1 || g.mode == GEMM_ATOMIC, "split-K needs atomic mode");
-  const long long nz = (long long)g.batch * g.splitk;
   if constexpr (sizeof(T) == 8) {
     static const int edges[4] = {64, 32, 16, 8};
     static const double eff[4] = {1.0, 0.97, 0.9, 0.8};
-    switch (pick_tile(g.M, g.N, nz, edges, eff, 4)) {
+    switch (pick_tile(g.M, g.N, g.splitk, edges, eff, 4)) {
       case 0: simt_launch<T, OutT, 64, 64, 16, 4, 4, 1>(g, s); break;
       case 1: simt_launch<T, OutT, 32, 32, 16, 2, 2, 1>(g, s); break;
       case 2: simt_launch<T, OutT, 16, 16, 32, 2, 2, 4>(g, s); break;
@@ -336,7 +334,7 @@ void simt_gemm(const SimtGemm<T, OutT>& g, cudaStream_t s) {
   } else {
     static const int edges[3] = {128, 64, 32};
     static const double eff[3] = {1.0, 0.6, 0.3};
-    switch (pick_tile(g.M, g.N, nz, edges, eff, 3)) {
+    switch (pick_tile(g.M, g.N, g.splitk, edges, eff, 3)) {
       case 0: simt_launch<T, OutT, 128, 128, 8, 8, 8, 1>(g, s); break;
       case 1: simt_launch<T, OutT, 64, 64, 16, 4, 4, 1>(g, s); break;
       default: simt_launch<T, OutT, 32, 32, 32, 2, 2, 1>(g, s); break;

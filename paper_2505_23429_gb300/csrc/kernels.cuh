@@ -6,8 +6,7 @@ namespace a2 {
 
 // C(m,n) {=, +=, atomic +=} alpha * sum_k A(m,k) B(n,k), general strides:
 //   A(m,k) = A[m*sam + k*sak], B(n,k) = B[n*sbn + k*sbk], C(m,n) = C[m*scm + n*scn]
-// batched over `batch` with element strides abs/bbs/cbs, optional split-K
-// (splitk > 1 requires mode == GEMM_ATOMIC and a zeroed C).
+// with optional split-K (splitk > 1 requires mode == GEMM_ATOMIC and a zeroed C).
 enum GemmMode { GEMM_STORE = 0, GEMM_ADD = 1, GEMM_ATOMIC = 2 };
 
 template <typename T, typename OutT>
@@ -16,7 +15,6 @@ struct SimtGemm {
   const T* A = nullptr; long long sam = 0, sak = 1;
   const T* B = nullptr; long long sbn = 0, sbk = 1;
   OutT* C = nullptr; long long scm = 0, scn = 1;
-  int batch = 1; long long abs = 0, bbs = 0, cbs = 0;
   int splitk = 1;
   T alpha = T(1);
   int mode = GEMM_STORE;
