@@ -2032,12 +2032,21 @@ void tc_heff1_f32emu(cudaStream_t s, int n, int Rl, int Rr, int Dl, int Dr,
 // multiple of the unit 2^(e_A + e_B + 2 - 8 (i + j)) of the chunk; the pairs with i + j <= 8 are
 // kept (28; the rest lie below 2^-58 of the scales), see tc_oz_kernel for their exact
 // accumulation chunk by chunk.
+// Range: slices are BF16 values, so a chunk that holds a NaN, an infinity or an entry of 2^128 or
+// more has no slices.  Its first slice is written as NaN, which reaches every product of
+// the row.  At the other end, slices whose scale lies below 2^-126 are zero: chunks whose largest
+// entry is below 2^-72 keep an absolute accuracy of about 2^-126 instead of their 55 bits.
 namespace {
 
 static_assert(kOzSlices == 7 && kOzBits == 8, "the digits cover 55 bits and a sign");
 
 __device__ __forceinline__ float pow2f(int k) {
   return (k >= -126 && k <= 127) ? __int_as_float((k + 127) << 23) : 0.f;
+}
+
+// Scale of slice i (1 ... kOzSlices) of a chunk whose entries are below 2^e.
+__device__ __forceinline__ float oz_scale(int e, int i) {
+  return i == 1 && e > 128 ? __int_as_float(0x7fffffff) : pow2f(e + 1 - kOzBits * i);
 }
 
 // Slicing with integer operations only (the FP64 pipe is slow on this part): the signed
@@ -2116,7 +2125,7 @@ ozaki_split_kernel(const double* __restrict__ X, long long sr, long long sk, int
 #pragma unroll
       for (int i = 0; i < kOzSlices; ++i)
         *reinterpret_cast<uint2*>(dst + i * kOzKBlock) =
-            oz_pack(q[0][i], q[1][i], q[2][i], q[3][i], pow2f(e + 1 - kOzBits * (i + 1)));
+            oz_pack(q[0][i], q[1][i], q[2][i], q[3][i], oz_scale(e, i + 1));
     }
   }
 }
@@ -2160,7 +2169,7 @@ ozaki_split_cols_kernel(const double* __restrict__ X, long long ldx, int N, int 
 #pragma unroll
       for (int i = 0; i < kOzSlices; ++i)
         tile[i][lane][warp + 8 * t] =
-            __float2bfloat16_rn((float)q[i] * pow2f(e + 1 - kOzBits * (i + 1)));
+            __float2bfloat16_rn((float)q[i] * oz_scale(e, i + 1));
     }
     __syncthreads();
     // vectors of 4 values, the slices of one (row, K block) one after another in memory
