@@ -293,17 +293,10 @@ __device__ __forceinline__ double lq_warp_sum4(const double (&v)[4], int lane) {
   for (int o = 4; o; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
   return r;
 }
-// 1 / q to ~2^-58 (q normal): hardware seed, e = 1 - q r, r (1 + e + e^2).
-__device__ __forceinline__ double lq_rcp(double q) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(q));
-  const double e = fma(-q, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
 // (beta, tau, scale) of the reflection that maps (al, x_1..), sum x_k^2 = s2, onto beta e_0:
 // beta = -sign(al) |x|, tau = (beta - al) / beta = 1 + |al| / |x|, scale = 1 / (al - beta); tau = 0
-// (and beta = al) when s2 = 0.  One reciprocal square root and one reciprocal instead of a
-// square root and two divisions (half the latency); the latter outside the normal range.
+// (and beta = al) when s2 = 0.  One reciprocal square root and one division instead of a
+// square root and two divisions; the latter outside the normal range.
 __device__ __forceinline__ void lq_scalars(double al, double s2, double& beta, double& tau,
                                            double& scale) {
   beta = al;
@@ -316,12 +309,11 @@ __device__ __forceinline__ void lq_scalars(double al, double s2, double& beta, d
     const double inv = rsqrt(n2);
     nrm = n2 * inv;
     tau = fma(aa, inv, 1.0);
-    scale = lq_rcp(aa + nrm);
   } else {
     nrm = sqrt(n2);
     tau = (nrm + aa) / nrm;
-    scale = 1.0 / (aa + nrm);
   }
+  scale = 1.0 / (aa + nrm);
   beta = al >= 0.0 ? -nrm : nrm;
   if (!(al >= 0.0)) scale = -scale;
 }
@@ -1398,8 +1390,6 @@ __global__ void tgk_invit_kernel(const double* d, const double* e, int n, const 
     z[j] = (double)((h >> 11) & 0xFFFFF) / 1048576.0 - 0.5;
   }
   __syncwarp();
-  const bool normal = tmax > 1e-260 && tmax < 1e260;
-  auto rcp = [&](double q) { return normal ? lq_rcp(q) : 1.0 / q; };
   // magnitudes compared as integers (an FP64 comparison costs a slot of the FP64 pipe)
   auto mag = [](double q) { return __double_as_longlong(q) & 0x7fffffffffffffffll; };
   const long long mtiny = mag(tiny);
@@ -1411,7 +1401,7 @@ __global__ void tgk_invit_kernel(const double* d, const double* e, int n, const 
       const double sub = t(j + 1), dn = dg[j + 1], r2 = j + 2 < N ? s1[j + 1] : 0.0;
       if (mag(dj) >= mag(sub) || mag(sub) < mtiny) {
         if (mag(dj) < mtiny) dj = __double_as_longlong(dj) < 0 ? -tiny : tiny;
-        const double inv = rcp(dj);
+        const double inv = 1.0 / dj;
         const double f = sub * inv;
         ml[j] = f;
         s1[j] = s1j;
@@ -1419,7 +1409,7 @@ __global__ void tgk_invit_kernel(const double* d, const double* e, int n, const 
         dj = fma(-f, s1j, dn);
         s1j = r2;
       } else {                                // interchange rows j and j + 1
-        const double inv = rcp(sub);
+        const double inv = 1.0 / sub;
         const double f = dj * inv;
         ml[j] = f;
         sw[j] = 1;
@@ -1431,7 +1421,7 @@ __global__ void tgk_invit_kernel(const double* d, const double* e, int n, const 
       }
     }
     if (mag(dj) < mtiny) dj = __double_as_longlong(dj) < 0 ? -tiny : tiny;
-    dg[N - 1] = rcp(dj);
+    dg[N - 1] = 1.0 / dj;
   }
   __syncwarp();
   // the superdiagonals times the reciprocal pivots: a step of the back substitution is then

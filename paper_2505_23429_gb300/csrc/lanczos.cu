@@ -238,14 +238,6 @@ struct TriShared {
   double y[64], v[64], dl[64], d[64], du[64], du2[64], rhs[64];   // fallback
 };
 
-// 1 / q to ~2^-58 from the hardware's FP64 reciprocal seed: e = 1 - q r, r (1 + e + e^2).
-__device__ __forceinline__ double fast_rcp(double q) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(q));
-  const double e = fma(-q, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-
 // Lowest eigenpair by 32-way multisection of the Sturm count and inverse iteration with a
 // partially pivoted elimination, one warp: the general method, for spectra that the fast
 // one below does not settle (two eigenvalues closer than its sample points).
@@ -339,7 +331,7 @@ __device__ int tri_count(const TriShared& S, int k, double x) {
   c += !(q > 0.0);
   for (int i = 1; i < k; ++i) {
     if (q == 0.0) q = 1e-300;
-    q = fma(-S.b2[i - 1], fast_rcp(q), S.a[i] - x);
+    q = fma(-S.b2[i - 1], 1.0 / q, S.a[i] - x);
     c += !(q > 0.0);
   }
   return c;
@@ -468,7 +460,7 @@ __device__ void tri_lowest(TriShared& S, int k) {
           if (q == 0.0) q = 1e-300;
           S.Dp[i] = q;
           if (i == k - 1) break;
-          const double r = fast_rcp(q);
+          const double r = 1.0 / q;
           S.Rp[i] = r;
           q = fma(-S.b2[i], r, S.a[i + 1] - x);
         }
@@ -480,7 +472,7 @@ __device__ void tri_lowest(TriShared& S, int k) {
           if (q == 0.0) q = 1e-300;
           S.Dm[i] = q;
           if (i == 0) break;
-          const double r = fast_rcp(q);
+          const double r = 1.0 / q;
           S.Rm[i] = r;
           q = fma(-S.b2[i - 1], r, S.a[i - 1] - x);
         }
