@@ -7,6 +7,8 @@
 #include <string>
 #include <stdexcept>
 
+#include "per_device.h"
+
 namespace a2 {
 
 struct CudaError : std::runtime_error {
@@ -42,6 +44,13 @@ void set_capturing(bool on);          // this thread is capturing a CUDA graph
   do {                                                                             \
     if (!(cond)) throw ::a2::ArgError(std::string(msg));                           \
   } while (0)
+
+inline int current_device() {
+  int dev = 0;
+  A2_CUDA(cudaGetDevice(&dev));
+  return dev;
+}
+int device_sms();        // multiprocessors of the current device
 
 inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
 

@@ -14,7 +14,6 @@
 // so every row is independent.
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 #include <vector>
 
 #include "factor.cuh"
@@ -1827,17 +1826,6 @@ __global__ void rows_to_cols_kernel(const double* in, int r, int n, int p, doubl
   }
 }
 
-int num_sms() {
-  static int n = 0;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    int dev = 0;
-    A2_CUDA(cudaGetDevice(&dev));
-    A2_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
-  });
-  return n;
-}
-
 void set_smem(const void* fn, size_t bytes) {
   if (bytes > 48 * 1024)
     A2_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
@@ -1856,8 +1844,8 @@ int factor_error_flag(bool reset) {
 }
 
 void set_attributes() {
-  static std::once_flag attr;
-  std::call_once(attr, [] {
+  static PerDevice<bool> set;
+  set.at(current_device(), [] {
     set_smem((const void*)hh_lq_kernel, 200 * 1024);
     set_smem((const void*)hh_form_q_kernel, 200 * 1024);
     set_smem((const void*)bidiag_apply_kernel, 200 * 1024);
@@ -1867,6 +1855,7 @@ void set_attributes() {
     set_smem((const void*)tgk_refine64_kernel<32>, 200 * 1024);
     set_smem((const void*)tgk_invit_kernel, 200 * 1024);
     set_smem((const void*)hh_bidiag_smem_kernel, 224 * 1024);
+    return true;
   });
 }
 
@@ -1877,9 +1866,8 @@ constexpr size_t kLqSmem = 216 * 1024;
 // Cluster of CTAs for a panel of ncol columns: about 96 columns per CTA (a sum over 16 rows then
 // takes ~900 cycles, as long as the exchange), at most what the device can place.
 int lq_cluster(int ncol) {
-  static int most = 8;
-  static std::once_flag once;
-  std::call_once(once, [] {
+  static PerDevice<int> clusters;
+  const int most = clusters.at(current_device(), [] {
     A2_CUDA(cudaFuncSetAttribute(lq_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kLqSmem));
     A2_CUDA(cudaFuncSetAttribute(lq_panel_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
@@ -1894,10 +1882,11 @@ int lq_cluster(int ncol) {
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, lq_panel_kernel, &cfg) == cudaSuccess &&
-        nclusters >= 1)
-      most = kLqCluster;
+    const bool fits =
+        cudaOccupancyMaxActiveClusters(&nclusters, lq_panel_kernel, &cfg) == cudaSuccess &&
+        nclusters >= 1;
     (void)cudaGetLastError();
+    return fits ? kLqCluster : 8;
   });
   int cs = 1;
   while (cs < most && cs * 96 < ncol) cs *= 2;
@@ -1909,13 +1898,14 @@ int lq_cluster(int ncol) {
 // memory holds.  Beside a panel (per_sm 1) one block per SM, so that the panel's cluster finds
 // room.
 void lq_rows(RowsArgs p, cudaStream_t s, int per_sm = 2) {
-  static std::once_flag once;
-  std::call_once(once, [] {
+  static PerDevice<bool> set;
+  set.at(current_device(), [] {
     A2_CUDA(cudaFuncSetAttribute(lq_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kLqSmem));
+    return true;
   });
   const int fit = (int)(kLqSmem / (sizeof(double) * (size_t)p.n)) - 2;
-  p.rb = std::max(1, std::min({8, fit, cdiv(p.nrows, per_sm * num_sms())}));
+  p.rb = std::max(1, std::min({8, fit, cdiv(p.nrows, per_sm * device_sms())}));
   lq_rows_kernel<<<cdiv(p.nrows, p.rb), kFacThreads, sizeof(double) * (size_t)(p.rb + 2) * p.n, s>>>(
       p);
   A2_CHECK_LAUNCH();
@@ -1937,11 +1927,10 @@ BdShape bd_shape(int m, int n) {
   };
   BdShape sh;
   // clusters that fit with one block per SM (asked once: the query takes milliseconds)
-  static int nclusters = 0;
-  static std::once_flag once;
-  std::call_once(once, [] {
+  static PerDevice<int> asked;
+  const int nclusters = asked.at(current_device(), [] {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(num_sms() / kBdCluster * kBdCluster);
+    cfg.gridDim = dim3(device_sms() / kBdCluster * kBdCluster);
     cfg.blockDim = dim3(kFacThreads);
     cfg.dynamicSmemBytes = most;
     cudaLaunchAttribute at;
@@ -1950,7 +1939,9 @@ BdShape bd_shape(int m, int n) {
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    A2_CUDA(cudaOccupancyMaxActiveClusters(&nclusters, hh_bidiag_smem_kernel, &cfg));
+    int n = 0;
+    A2_CUDA(cudaOccupancyMaxActiveClusters(&n, hh_bidiag_smem_kernel, &cfg));
+    return n;
   });
   if (m >= 2 * kBdCluster) {
     const int nb = std::min(m / kBdCluster, nclusters) * kBdCluster;
@@ -1961,7 +1952,7 @@ BdShape bd_shape(int m, int n) {
       return sh;
     }
   }
-  const int nb = std::max(1, std::min(m, num_sms()));
+  const int nb = std::max(1, std::min(m, device_sms()));
   if (bytes(nb) <= most) {
     sh.blocks = nb;
     sh.smem = bytes(nb);
@@ -1977,7 +1968,7 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
   set_attributes();
   const bool left = rows >= cols;                 // bidiagonalise M (left) or M^T (right)
   const int m = left ? rows : cols, n = left ? cols : rows;
-  const int nb = std::max(1, std::min(m, num_sms()));
+  const int nb = std::max(1, std::min(m, device_sms()));
   // scratch: A (m n); d, e, tau_u, tau_v (n each); sigma and its brackets (3n); y (n);
   // Z by step modulo 3 (3n); published rows by step parity (2n); part (nb); ypart (nb n)
   const size_t nA = (size_t)m * n;
@@ -2045,7 +2036,7 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
     int best = 8;
     double best_cost = 1e300;
     for (int L : {8, 16, 32}) {
-      const double share = std::ceil((double)cdiv(nev * L, 32) / (4.0 * num_sms()));
+      const double share = std::ceil((double)cdiv(nev * L, 32) / (4.0 * device_sms()));
       const double cost = (L == 32 ? 3.0 : L == 16 ? 3.2 : 3.6) * std::max(1.0, share);
       if (cost <= best_cost) { best_cost = cost; best = L; }
     }
@@ -2076,7 +2067,7 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
   // kept singular vectors of B by inverse iteration, then into the columns of P (rows x r)
   constexpr int W = 32;
   const int npan = cdiv(r, W);
-  const int sms = num_sms();
+  const int sms = device_sms();
   // Gram chunk: rows per partial sum, so that the widest Gram has about 2 blocks per SM
   auto gram_chunk = [&](int a) {
     const long long want = (long long)rows * cdiv(a, 32) / (2LL * sms);
@@ -2163,7 +2154,7 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
     const int g = (int)std::max<long long>(0, std::min<long long>(16, room / (rows + 1)));
     const size_t smem =
         sizeof(double) * ((xsm ? (size_t)kApplyCols * rows : 0) + (size_t)g * (rows + 1));
-    bidiag_apply_kernel<<<std::min(cdiv(r, kApplyCols), 4 * num_sms()), 32 * kApplyCols, smem,
+    bidiag_apply_kernel<<<std::min(cdiv(r, kApplyCols), 4 * device_sms()), 32 * kApplyCols, smem,
                           s>>>(A, n, rows, q, left ? tu : tv, left ? 1 : 0, P, r, g, xsm);
     A2_CHECK_LAUNCH();
   }
@@ -2252,14 +2243,14 @@ int hh_lq(const double* M, int rows, int cols, double* L, double* Q, FactorWork&
     A2_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hh_lq_kernel, kFacThreads,
                                                           vbytes));
     A2_REQUIRE(per_sm >= 1, "LQ: kernel does not fit on an SM");
-    const int grid = std::max(1, std::min({rows, num_sms() * per_sm, num_sms()}));
+    const int grid = std::max(1, std::min({rows, device_sms() * per_sm, device_sms()}));
     GridBarrier* bar = w.bar.as<GridBarrier>();
     int* ready = reinterpret_cast<int*>(bar + 1);
     void* args[] = {&A, &rows, &cols, const_cast<int*>(&k), &V, &tau, &beta, &bar, &ready};
     A2_CUDA(cudaLaunchCooperativeKernel((const void*)hh_lq_kernel, dim3(grid), dim3(kFacThreads),
                                         args, vbytes, s));
     count_launch();
-    hh_form_q_kernel<<<std::min(k, 4 * num_sms()), kFacThreads, vbytes, s>>>(V, tau, cols, k, Q);
+    hh_form_q_kernel<<<std::min(k, 4 * device_sms()), kFacThreads, vbytes, s>>>(V, tau, cols, k, Q);
     A2_CHECK_LAUNCH();
     hh_sign_rows_kernel<<<std::min(k, 1024), 128, 0, s>>>(Q, cols, k, beta);
     A2_CHECK_LAUNCH();

@@ -10,6 +10,16 @@
 
 namespace a2 {
 
+int device_sms() {
+  static PerDevice<int> sms;
+  const int dev = current_device();
+  return sms.at(dev, [&] {
+    int n = 0;
+    A2_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    return n > 0 ? n : 1;
+  });
+}
+
 // ----------------------------------------------------------------------------- memory pool
 cudaMemPool_t lib_pool() {
   static std::mutex mu;
@@ -273,17 +283,6 @@ simt_gemm_kernel(SimtGemm<T, OutT> g) {
   }
 }
 
-static int simt_sms() {
-  static int n = 0;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    int dev = 0;
-    A2_CUDA(cudaGetDevice(&dev));
-    A2_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
-  });
-  return n > 0 ? n : 1;
-}
-
 template <typename T, typename OutT, int BM, int BN, int BK, int TM, int TN, int KG>
 static void simt_launch(const SimtGemm<T, OutT>& g, cudaStream_t s) {
   dim3 grid(cdiv(g.N, BN), cdiv(g.M, BM), g.splitk);
@@ -296,7 +295,7 @@ static void simt_launch(const SimtGemm<T, OutT>& g, cudaStream_t s) {
 // rounds of blocks over the SMs times the tile's area, divided by the tile's relative
 // efficiency.  A smaller tile also has to gain something (its loads per product are more).
 static int pick_tile(int M, int N, int splitk, const int* edges, const double* eff, int n) {
-  const int sms = simt_sms();
+  const int sms = device_sms();
   int best = 0;
   double best_cost = 0.0;
   for (int i = 0; i < n; ++i) {
@@ -1239,10 +1238,11 @@ __global__ void jacobi_kernel(double* A, int m, double* evals, double* evecs, in
 
 void jacobi_eig(double* A, int m, double* evals, double* evecs, int* status, cudaStream_t s) {
   A2_REQUIRE(m >= 1 && m <= 63, "jacobi_eig: 1 <= m <= 63");
-  static std::once_flag once;
-  std::call_once(once, [] {
+  static PerDevice<bool> set;
+  set.at(current_device(), [] {
     A2_CUDA(cudaFuncSetAttribute(jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sizeof(JacobiShared)));
+    return true;
   });
   jacobi_kernel<<<1, 256, sizeof(JacobiShared), s>>>(A, m, evals, evecs, status);
   A2_CHECK_LAUNCH();
@@ -1331,10 +1331,11 @@ __global__ void coarse_kernel(const double* A, const double* S, int m, double ep
 void coarse_solve_dev(const double* A, const double* S, int m, double eps, double* c,
                       double* lam, int* rank, int* status, cudaStream_t s) {
   A2_REQUIRE(m >= 1 && m <= 63, "coarse problem: 1 <= m <= 63");
-  static std::once_flag once;
-  std::call_once(once, [] {
+  static PerDevice<bool> set;
+  set.at(current_device(), [] {
     A2_CUDA(cudaFuncSetAttribute(coarse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sizeof(CoarseShared)));
+    return true;
   });
   coarse_kernel<<<1, 256, sizeof(CoarseShared), s>>>(A, S, m, eps, c, lam, rank, status);
   A2_CHECK_LAUNCH();
@@ -1512,7 +1513,7 @@ __global__ void sum_parts_kernel(const double* __restrict__ in, int n, int parts
 // X and Y of at most 64 MB (half of L2).
 int grad_dot_parts(int Dl, int Dr, int Rl, int nw, int n, int nel) {
   const long long bytes = 8LL * Dl * n * Dr * ((long long)Rl + nw);
-  const long long want = std::max<long long>(cdiv(16 * simt_sms(), nel), (bytes >> 26) + 1);
+  const long long want = std::max<long long>(cdiv(16 * device_sms(), nel), (bytes >> 26) + 1);
   return (int)std::min<long long>(want, Dl);
 }
 void grad_dots(const double* X, const double* Y, const int4* el, int nel, int Dl, int Rl, int n,

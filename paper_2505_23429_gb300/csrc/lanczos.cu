@@ -18,7 +18,6 @@
 // Mean of the steps j = 0 .. 20, device time: N = 4096 22 us (208 us as separate kernels),
 // N = 2^20 126 us (380 us; the vectors' traffic alone is ~40 us at this part's copy rate).
 #include <algorithm>
-#include <mutex>
 
 #include "kernels.cuh"
 
@@ -730,17 +729,15 @@ void lanczos_step(double* V, double* w, long long N, int j, double beta_prev, bo
                   double* tri, double* partial, unsigned* bar, unsigned* bar_next,
                   double* out, cudaStream_t s) {
   A2_REQUIRE(j >= 0 && j < 63, "Lanczos step: at most 63 basis vectors");
-  static int sms = 0;
-  static std::once_flag once;
   constexpr size_t kSliceMax = 160 * 1024;
-  std::call_once(once, [] {
-    int dev = 0;
-    A2_CUDA(cudaGetDevice(&dev));
-    A2_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  static PerDevice<bool> set;
+  set.at(current_device(), [] {
     for (const void* f : {(const void*)lanczos_step_kernel<false>,
                           (const void*)lanczos_step_kernel<true>})
       A2_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSliceMax));
+    return true;
   });
+  const int sms = device_sms();
   const int most = std::max(1, std::min(sms - 1, kReduceBlocks / 2));
   LzArgs p;
   p.V = V;

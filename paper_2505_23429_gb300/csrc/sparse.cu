@@ -18,7 +18,6 @@
 // BF16 S2 0.78 -> 0.58, S3 1.01 -> 0.76; FP32 pairs S2 + S3 6.34 -> 5.42; bond 7, split
 // products, S3 (three planes in and out) 4.82 -> 3.68.
 #include <algorithm>
-#include <mutex>
 #include <type_traits>
 
 #include "kernels.cuh"
@@ -271,10 +270,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) sparse_staged_kernel(StArgs a) 
 
 template <int IN, int OUT, bool ADD, bool VEC, int NT>
 void st_launch(const StArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
-  static std::once_flag once;
-  std::call_once(once, [] {
+  static PerDevice<bool> set;
+  set.at(current_device(), [] {
     A2_CUDA(cudaFuncSetAttribute(sparse_staged_kernel<IN, OUT, ADD, VEC, NT>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    return true;
   });
   sparse_staged_kernel<IN, OUT, ADD, VEC, NT><<<grid, NT, smem, s>>>(a);
   A2_CHECK_LAUNCH();

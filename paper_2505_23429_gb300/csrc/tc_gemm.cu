@@ -639,17 +639,6 @@ CUtensorMap make_map_nd(const __nv_bfloat16* ptr, int rank, const cuuint64_t* di
   return m;
 }
 
-int tc_sms() {
-  static int num_sms = 0;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    int dev = 0;
-    A2_CUDA(cudaGetDevice(&dev));
-    A2_CUDA(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
-  });
-  return num_sms;
-}
-
 template <int BN, int STAGES>
 void launch(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* B, long long ldb, int M,
             int N, int K, const TcSeg2* seg, void* C, long long ldc, int out_kind, int splitk,
@@ -681,10 +670,11 @@ void launch(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* B, long 
     maps.b2 = maps.b;
   }
   const size_t smem = sizeof(TcSmem<BN, STAGES>) + 1024;
-  static std::once_flag once;
-  std::call_once(once, [smem] {
+  static PerDevice<bool> set;
+  set.at(current_device(), [smem] {
     A2_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<BN, STAGES>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    return true;
   });
   const int nk1 = (K + BK - 1) / BK;
   const int nk_total = nk1 + nk2;
@@ -719,7 +709,7 @@ void launch(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* B, long 
   }
   const long long units = (long long)cdiv(M, BM) * cdiv(N, BN) * splitk;
   A2_REQUIRE(units < (1LL << 31), "tcgen05 GEMM too large");
-  const int grid = (int)std::min<long long>(units, std::max(1, tc_sms()));
+  const int grid = (int)std::min<long long>(units, device_sms());
   tc_gemm_kernel<BN, STAGES><<<grid, kTcThreads, smem, s>>>(maps, args);
   A2_CHECK_LAUNCH();
 }
@@ -1186,10 +1176,11 @@ void launch_oz(const __nv_bfloat16* A, const __nv_bfloat16* B, int M, int N, int
   maps.a7 = make_oz_map(A, M, nkb, true);
   maps.b7 = make_oz_map(B, N, nkb, true);
   const size_t smem = sizeof(OzSmem) + 1024;
-  static std::once_flag once;
-  std::call_once(once, [smem] {
+  static PerDevice<bool> set;
+  set.at(current_device(), [smem] {
     A2_CUDA(cudaFuncSetAttribute(tc_oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem));
+    return true;
   });
   OzArgs args;
   args.M = M; args.N = N;
@@ -1204,7 +1195,7 @@ void launch_oz(const __nv_bfloat16* A, const __nv_bfloat16* B, int M, int N, int
   args.MN = (long long)M * N;
   const long long units = (long long)cdiv(M, BM) * cdiv(N, kOzBN) * args.splits;
   A2_REQUIRE(units < (1LL << 31), "Ozaki GEMM too large");
-  const int grid = (int)std::min<long long>(units, std::max(1, tc_sms()));
+  const int grid = (int)std::min<long long>(units, device_sms());
   tc_oz_kernel<<<grid, kOzThreads, smem, s>>>(maps, args);
   A2_CHECK_LAUNCH();
 }
@@ -1582,10 +1573,11 @@ void launch_split3(const __nv_bfloat16* const* A, long long lda, const __nv_bflo
     }
   }
   const size_t smem = sizeof(S3Smem<BN>) + 1024;
-  static std::once_flag once;
-  std::call_once(once, [smem] {
+  static PerDevice<bool> set;
+  set.at(current_device(), [smem] {
     A2_CUDA(cudaFuncSetAttribute(tc_split3_kernel<BN>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    return true;
   });
   const int nk_total = args.nk1 + args.nk2;
   splitk = std::max(1, std::min(splitk, nk_total));
@@ -1597,7 +1589,7 @@ void launch_split3(const __nv_bfloat16* const* A, long long lda, const __nv_bflo
   if (!args.tma_store) maps.c = maps.a[0];
   const long long units = (long long)cdiv(M, BM) * cdiv(N, BN) * args.splits;
   A2_REQUIRE(units < (1LL << 31), "tcgen05 GEMM too large");
-  const int grid = (int)std::min<long long>(units, std::max(1, tc_sms()));
+  const int grid = (int)std::min<long long>(units, device_sms());
   tc_split3_kernel<BN><<<grid, kS3Threads, smem, s>>>(maps, args);
   A2_CHECK_LAUNCH();
 }
@@ -2240,7 +2232,7 @@ void ozaki_split(const double* X, long long sr, long long sk, int rows, int K, _
 void tc_gemm_f64emu(const __nv_bfloat16* A, const __nv_bfloat16* B, int M, int N, int K, double* C,
                     long long ldc, DevBuf& slab, cudaStream_t s, float* Cdf, long long df_plane) {
   if (M <= 0 || N <= 0) return;
-  const int num_sms = tc::tc_sms();
+  const int num_sms = device_sms();
   // K splits: at most kOzSplitBlocks K blocks per split (bounds the number of sums per
   // accumulator, hence the rounding of its lo part), and enough work units to fill the GPU
   // when the output has few tiles
