@@ -90,22 +90,27 @@ struct SiteOps {
   struct Part {
     int nrows = 0, nnz = 0;
     int in_rows = 0, in_t = 1;
-    DevBuf ptr, rw, rs, nw, nt, v64, v32, v32lo, sell, sell_lo, sell_row;
+    // all arrays in one buffer (made by one copy), each from a multiple of 256 bytes on
+    enum { PTR, RW, RS, NW, NT, V64, V32, V32LO, SELL, SELL_LO, SELL_ROW, ARRAYS };
+    DevBuf buf;
+    size_t at[ARRAYS] = {};
+    template <typename E> const E* array(int i) const {
+      return reinterpret_cast<const E*>(buf.as<unsigned char>() + at[i]);
+    }
     template <typename V> SparseRows<V> rows() const {
       SparseRows<V> r;
       r.nrows = nrows;
-      r.row_ptr = ptr.as<int>();
-      r.row_w = rw.as<int>();
-      r.row_s = rs.as<int>();
-      r.nz_w = nw.as<int>();
-      r.nz_t = nt.as<int>();
+      r.row_ptr = array<int>(PTR);
+      r.row_w = array<int>(RW);
+      r.row_s = array<int>(RS);
+      r.nz_w = array<int>(NW);
+      r.nz_t = array<int>(NT);
       r.nnz_total = nnz;
-      if constexpr (sizeof(V) == 8) r.nz_val = v64.as<double>();
-      else r.nz_val = v32.as<float>();
-      r.nz_lo = v32lo.as<float>();
-      r.sell = sell.as<int2>();
-      r.sell_lo = sell_lo.as<float>();
-      r.sell_row = sell_row.as<int4>();
+      r.nz_val = array<V>(sizeof(V) == 8 ? V64 : V32);
+      r.nz_lo = array<float>(V32LO);
+      r.sell = array<int2>(SELL);
+      r.sell_lo = array<float>(SELL_LO);
+      r.sell_row = array<int4>(SELL_ROW);
       r.in_rows = in_rows;
       r.in_t = in_t;
       return r;
@@ -163,62 +168,72 @@ void upload(DevBuf& b, const void* h, size_t bytes, cudaStream_t s) {
 void build_part(SiteOps::Part& part, const std::vector<std::vector<std::array<double, 3>>>& rows,
                 const std::vector<std::pair<int, int>>& rowid, int win, int nt_in,
                 cudaStream_t s) {
-  part.nrows = (int)rows.size();
+  using P = SiteOps::Part;
+  const size_t nr = rows.size();
+  part.nrows = (int)nr;
   part.in_rows = win * nt_in;
   part.in_t = nt_in;
-  std::vector<int> order(rows.size());
+  std::vector<int> order(nr);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(),
                    [&](int x, int y) { return rows[x].size() > rows[y].size(); });
-  std::vector<int> ptr(rows.size() + 1, 0), rw, rs, nw, nt;
-  std::vector<double> v64;
-  std::vector<float> v32, v32lo;
-  for (size_t i = 0; i < rows.size(); ++i) {
-    const int r = order[i];
-    rw.push_back(rowid[r].first);
-    rs.push_back(rowid[r].second);
-    for (auto& e : rows[r]) {
-      nw.push_back((int)e[0]);
-      nt.push_back((int)e[1]);
-      v64.push_back(e[2]);
-      const float hi = (float)e[2];
-      v32.push_back(hi);
-      v32lo.push_back((float)(e[2] - (double)hi));
-    }
-    ptr[i + 1] = (int)nw.size();
+  size_t nnz = 0, ngap = 0;              // entries; the same with the gaps of the interleaved form
+  for (size_t i = 0; i < nr; ++i) {
+    nnz += rows[order[i]].size();
+    if (i % kSellRows == 0) ngap += rows[order[i]].size() * kSellRows;
   }
-  part.nnz = (int)nw.size();
-  // the same entries interleaved over kSellRows rows (gaps behind the shorter rows)
-  std::vector<int4> meta(rows.size());
-  std::vector<int2> sell;
-  std::vector<float> sell_lo;
-  for (size_t i0 = 0; i0 < rows.size(); i0 += kSellRows) {
-    const size_t base = sell.size(), len0 = rows[order[i0]].size();   // the longest of them
-    sell.resize(base + len0 * kSellRows, int2{0, 0});
-    sell_lo.resize(sell.size(), 0.f);
-    for (size_t i = i0; i < std::min(rows.size(), i0 + kSellRows); ++i) {
-      const int len = ptr[i + 1] - ptr[i];
-      meta[i] = int4{len, (int)(base + (i - i0)), rw[i], rs[i]};
-      for (int e = 0; e < len; ++e) {
-        const int q = ptr[i] + e;
-        int2& k = sell[base + (size_t)e * kSellRows + (i - i0)];
-        k.x = nw[q] * nt_in + nt[q];
-        std::memcpy(&k.y, &v32[q], sizeof(float));
-        sell_lo[base + (size_t)e * kSellRows + (i - i0)] = v32lo[q];
-      }
+  part.nnz = (int)nnz;
+  const size_t bytes[P::ARRAYS] = {
+      (nr + 1) * sizeof(int), nr * sizeof(int),      nr * sizeof(int),
+      nnz * sizeof(int),      nnz * sizeof(int),     nnz * sizeof(double),
+      nnz * sizeof(float),    nnz * sizeof(float),   ngap * sizeof(int2),
+      ngap * sizeof(float),   nr * sizeof(int4)};
+  size_t total = 0;
+  for (int i = 0; i < P::ARRAYS; ++i) {
+    part.at[i] = total;
+    total = (total + bytes[i] + 255) / 256 * 256;
+  }
+  std::vector<double> host(total / sizeof(double));        // zeros: the gaps
+  auto array = [&](int i) { return reinterpret_cast<unsigned char*>(host.data()) + part.at[i]; };
+  int* ptr = reinterpret_cast<int*>(array(P::PTR));
+  int* rw = reinterpret_cast<int*>(array(P::RW));
+  int* rs = reinterpret_cast<int*>(array(P::RS));
+  int* nw = reinterpret_cast<int*>(array(P::NW));
+  int* nt = reinterpret_cast<int*>(array(P::NT));
+  double* v64 = reinterpret_cast<double*>(array(P::V64));
+  float* v32 = reinterpret_cast<float*>(array(P::V32));
+  float* v32lo = reinterpret_cast<float*>(array(P::V32LO));
+  int2* sell = reinterpret_cast<int2*>(array(P::SELL));
+  float* sell_lo = reinterpret_cast<float*>(array(P::SELL_LO));
+  int4* meta = reinterpret_cast<int4*>(array(P::SELL_ROW));
+  // row by row, and the same entries interleaved over kSellRows rows (gaps behind the shorter
+  // ones of them)
+  int q = 0;
+  size_t base = 0;
+  for (size_t i = 0; i < nr; ++i) {
+    const int r = order[i], lane = (int)(i % kSellRows);
+    if (i > 0 && lane == 0) base += rows[order[i - kSellRows]].size() * kSellRows;
+    ptr[i] = q;
+    rw[i] = rowid[r].first;
+    rs[i] = rowid[r].second;
+    meta[i] = int4{(int)rows[r].size(), (int)(base + lane), rw[i], rs[i]};
+    size_t k = base + lane;
+    for (const auto& e : rows[r]) {
+      const float hi = (float)e[2], lo = (float)(e[2] - (double)hi);
+      nw[q] = (int)e[0];
+      nt[q] = (int)e[1];
+      v64[q] = e[2];
+      v32[q] = hi;
+      v32lo[q] = lo;
+      sell[k].x = nw[q] * nt_in + nt[q];
+      std::memcpy(&sell[k].y, &hi, sizeof(float));
+      sell_lo[k] = lo;
+      k += kSellRows;
+      ++q;
     }
   }
-  upload(part.ptr, ptr.data(), ptr.size() * sizeof(int), s);
-  upload(part.rw, rw.data(), rw.size() * sizeof(int), s);
-  upload(part.rs, rs.data(), rs.size() * sizeof(int), s);
-  upload(part.nw, nw.data(), nw.size() * sizeof(int), s);
-  upload(part.nt, nt.data(), nt.size() * sizeof(int), s);
-  upload(part.v64, v64.data(), v64.size() * sizeof(double), s);
-  upload(part.v32, v32.data(), v32.size() * sizeof(float), s);
-  upload(part.v32lo, v32lo.data(), v32lo.size() * sizeof(float), s);
-  upload(part.sell, sell.data(), sell.size() * sizeof(int2), s);
-  upload(part.sell_lo, sell_lo.data(), sell_lo.size() * sizeof(float), s);
-  upload(part.sell_row, meta.data(), meta.size() * sizeof(int4), s);
+  ptr[nr] = q;
+  upload(part.buf, host.data(), total, s);
 }
 
 // Scan a dense core W[wl][s][t][wr] (minus `sub` = I (x) G when given) into the two
