@@ -2211,9 +2211,13 @@ __global__ void ozaki_combine_kernel(const float* __restrict__ T, long long MN, 
 void ozaki_split_cols(const double* X, long long ldx, int N, int K, __nv_bfloat16* P,
                       cudaStream_t s) {
   if (N <= 0 || K <= 0) return;
-  A2_REQUIRE(cdiv(K, kOzGroup) < 65536, "Ozaki slicing: K too large");
-  ozaki_split_cols_kernel<<<dim3((N + 31) / 32, cdiv(K, kOzGroup)), 256, 0, s>>>(X, ldx, N, K, P);
-  A2_CHECK_LAUNCH();
+  constexpr int kMost = 65535 * kOzGroup;              // grid.y chunks of a launch
+  for (long long k0 = 0; k0 < K; k0 += kMost) {
+    const int kn = (int)std::min<long long>(K - k0, kMost);
+    ozaki_split_cols_kernel<<<dim3((N + 31) / 32, cdiv(kn, kOzGroup)), 256, 0, s>>>(
+        X + k0 * ldx, ldx, N, kn, P + k0 / kOzKBlock * N * kOzRowBlock);
+    A2_CHECK_LAUNCH();
+  }
 }
 
 void ozaki_split(const double* X, long long sr, long long sk, int rows, int K, __nv_bfloat16* P,
