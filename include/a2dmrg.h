@@ -373,6 +373,18 @@ a2_status a2_device_error(a2_ctx* ctx, int reset, int* code_out);
  * out. */
 a2_status a2_selftest_timeout(a2_ctx* ctx, int* code_out);
 
+/* The same for the Lanczos step's grid barrier (not paper content): one step whose blocks
+ * wait for one arrival more than comes, with a limit of 2^14 polls.  The waits give up, every
+ * block leaves, and the call returns A2_ETIMEOUT; A2_ECUDA if the wait did not run out.  The
+ * device error word is not used: a solve whose barrier gives up returns A2_ECUDA. */
+a2_status a2_selftest_lanczos_timeout(a2_ctx* ctx);
+
+/* Lowest eigenpair of the symmetric tridiagonal matrix with diagonal a[k] and off-diagonal
+ * b[k-1], k <= 63 (host arrays), by the solver of the Lanczos step: *theta_out, the unit
+ * vector vec_out[k], and *general_out (may be NULL) = 1 where the general method had to run. */
+a2_status a2_tridiag_lowest(a2_ctx* ctx, int k, const double* a, const double* b,
+                            double* theta_out, double* vec_out, int* general_out);
+
 /* Live kernel timing with CUDA events on the context stream (not paper content;
  * used to report achieved throughput per kernel class).  op: 0 = disable,
  * 1 = enable, 2 = reset totals, 3 = read the totals of `kind` (0 tcgen05 S1,

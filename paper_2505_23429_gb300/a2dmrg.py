@@ -104,6 +104,8 @@ def lib():
                          _P, ctypes.c_longlong, _P, ctypes.c_longlong, ctypes.c_int],
         "a2_device_error": [_P, ctypes.c_int, _I],
         "a2_selftest_timeout": [_P, _I],
+        "a2_selftest_lanczos_timeout": [_P],
+        "a2_tridiag_lowest": [_P, ctypes.c_int, _D, _D, _D, _D, _I],
         "a2_lq": [_P, ctypes.c_int, ctypes.c_int, _P, _P, _P],
         "a2_profile": [_P, ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_longlong), _D, _D,
                        _D],
@@ -131,7 +133,8 @@ def exported_symbols():
             "a2_device_error", "a2_profile", "a2_heff_apply_noalloc", "a2_mpo_fold_split",
             "a2_mpo_fold_info", "a2_mpo_set_fold", "a2_heff_create", "a2_heff_apply_op",
             "a2_heff_destroy", "a2_energy_gradient", "a2_set_autotune", "a2_tt_save",
-            "a2_tt_load", "a2_selftest_timeout", "a2_lq"]
+            "a2_tt_load", "a2_selftest_timeout", "a2_lq", "a2_selftest_lanczos_timeout",
+            "a2_tridiag_lowest"]
 
 
 def _dp(a):
@@ -458,6 +461,22 @@ def selftest_timeout(ctx):
     code = ctypes.c_int(0)
     st = lib().a2_selftest_timeout(ctx._h, ctypes.byref(code))
     return st, code.value
+
+
+def selftest_lanczos_timeout(ctx):
+    """The same for the Lanczos step's grid barrier (a2_selftest_lanczos_timeout): status."""
+    return lib().a2_selftest_lanczos_timeout(ctx._h)
+
+
+def tridiag_lowest(ctx, a, b):
+    """Lowest eigenpair of the symmetric tridiagonal (diagonal a, off-diagonal b) by the
+    Lanczos step's solver (a2_tridiag_lowest): (eigenvalue, vector, general method ran)."""
+    a, b = (np.ascontiguousarray(v, dtype=np.float64) for v in (a, b))
+    th, z, general = ctypes.c_double(), np.zeros(len(a)), ctypes.c_int()
+    p = [v.ctypes.data_as(_D) for v in (a, b, z)]
+    ctx.check(lib().a2_tridiag_lowest(ctx._h, len(a), p[0], p[1], ctypes.byref(th), p[2],
+                                      ctypes.byref(general)))
+    return th.value, z, bool(general.value)
 
 
 PROFILE_KINDS = ["tc_s1", "sparse_s2", "sparse_s3", "tc_s4", "heff_simt", "env", "lanczos",

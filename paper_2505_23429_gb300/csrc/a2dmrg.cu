@@ -3410,6 +3410,41 @@ a2_status a2_lq(a2_ctx* c, int rows, int cols, const double* M, double* L, doubl
   });
 }
 
+a2_status a2_selftest_lanczos_timeout(a2_ctx* c) {
+  if (!c) return A2_EINVAL;
+  bool ran_out = false;
+  a2_status st = guarded(c, [&] {
+    A2_CUDA(cudaSetDevice(c->device));
+    ran_out = lanczos_selftest_timeout(c->partial.as<double>(), c->h_scal + 32, c->stream);
+  });
+  if (st != A2_OK) return st;
+  if (!ran_out)
+    return fail(c, A2_ECUDA, "a2_selftest_lanczos_timeout: the wait did not run out");
+  return fail(c, A2_ETIMEOUT, "Lanczos: a bounded grid barrier gave up");
+}
+
+a2_status a2_tridiag_lowest(a2_ctx* c, int k, const double* a, const double* b, double* theta_out,
+                            double* vec_out, int* general_out) {
+  if (!c) return A2_EINVAL;
+  return guarded(c, [&] {
+    A2_REQUIRE(k >= 1 && k <= 63 && a && (k == 1 || b) && theta_out && vec_out,
+               "a2_tridiag_lowest: bad arguments");
+    double h[65];
+    double* t = scal(c, 1024);
+    A2_CUDA(cudaMemcpyAsync(t, a, sizeof(double) * k, cudaMemcpyHostToDevice, c->stream));
+    if (k > 1)
+      A2_CUDA(cudaMemcpyAsync(t + 64, b, sizeof(double) * (k - 1), cudaMemcpyHostToDevice,
+                              c->stream));
+    tridiag_lowest(t, t + 64, k, t + 128, c->stream);
+    A2_CUDA(cudaMemcpyAsync(h, t + 128, sizeof(double) * (k + 2), cudaMemcpyDeviceToHost,
+                            c->stream));
+    A2_CUDA(cudaStreamSynchronize(c->stream));
+    *theta_out = h[0];
+    if (general_out) *general_out = h[1] != 0.0;
+    std::copy(h + 2, h + 2 + k, vec_out);
+  });
+}
+
 a2_status a2_selftest_timeout(a2_ctx* c, int* code_out) {
   if (!c || !code_out) return A2_EINVAL;
   int code = 0;

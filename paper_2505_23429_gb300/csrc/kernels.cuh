@@ -127,6 +127,12 @@ void jacobi_eig(double* A, int m, double* evals, double* evecs, int* status, cud
 void lanczos_step(double* V, double* w, long long N, int j, double beta_prev, bool write_next,
                   double* tri, double* partial, unsigned* bar, unsigned* bar_next,
                   double* out, cudaStream_t s);
+// The step with one arrival too many expected at its grid barriers and a limit of 2^14 polls:
+// returns whether out[4] reports that the wait ran out.  Synchronous.
+bool lanczos_selftest_timeout(double* partial, double* out, cudaStream_t s);
+// The step's tridiagonal solver by itself (device pointers, k <= 63): out[0] eigenvalue, out[1] 1
+// if the general method ran, out[2 ..] the unit eigenvector.
+void tridiag_lowest(const double* a, const double* b, int k, double* out, cudaStream_t s);
 
 // Coarse problem of Sec. 3.1 (m <= 63) in one CTA; outputs on the device.
 void coarse_solve_dev(const double* A, const double* S, int m, double eps, double* c,

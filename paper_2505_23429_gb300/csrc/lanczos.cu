@@ -42,6 +42,8 @@ struct LzArgs {
   unsigned* bar;        // {arrivals, abort} of this step, zero on entry
   unsigned* bar_next;   // those of the next step, zeroed here
   double* out;          // pinned host: alpha, |w|^2, theta, |last component|, gave-up flag
+  unsigned wait_limit;  // polls of a bounded wait
+  unsigned extra;       // self-test only: arrivals waited for beyond those that come
 };
 
 __device__ __forceinline__ double shfl_xor_d(double v, int o) {
@@ -84,14 +86,14 @@ __device__ void lz_arrive(unsigned* bar) {
   }
 }
 // Bounded wait for `target` arrivals; false if it (or another block) gave up.
-__device__ bool lz_wait(unsigned* bar, unsigned target) {
+__device__ bool lz_wait(unsigned* bar, unsigned target, unsigned limit) {
   __shared__ int ok;
   if (threadIdx.x == 0) {
     ok = 1;
     for (unsigned it = 0;; ++it) {
       if (*(volatile unsigned*)bar >= target) break;
       if (*(volatile unsigned*)(bar + 1)) { ok = 0; break; }
-      if (it >= kLzWaitLimit) {
+      if (it >= limit) {
         atomicExch(bar + 1, 1u);
         ok = 0;
         break;
@@ -566,7 +568,7 @@ __global__ void __launch_bounds__(kLzThreads) lanczos_step_kernel(LzArgs p) {
       S.a[tid] = p.tri[tid];
       S.b[tid] = tid < k - 2 ? p.tri[64 + tid] : p.beta_prev;
     }
-    if (!lz_wait(p.bar, (unsigned)G)) {
+    if (!lz_wait(p.bar, (unsigned)G + p.extra, p.wait_limit)) {
       if (tid == 0) p.out[4] = 1.0;
       return;
     }
@@ -602,7 +604,7 @@ __global__ void __launch_bounds__(kLzThreads) lanczos_step_kernel(LzArgs p) {
   // ---- alpha = <v_j, w>
   lz_dots(V + (long long)p.j * p.N, p.N, x, n, 1, false, part_a + b, G, red);
   lz_arrive(p.bar);
-  if (!lz_wait(p.bar, ++epoch * G)) {
+  if (!lz_wait(p.bar, ++epoch * G + p.extra, p.wait_limit)) {
     if (tid == 0) p.out[4] = 1.0;
     return;
   }
@@ -624,7 +626,7 @@ __global__ void __launch_bounds__(kLzThreads) lanczos_step_kernel(LzArgs p) {
   for (int pass = 0; pass < 2; ++pass) {
     lz_dots(V, p.N, x, n, k, true, part_h + b, G, red);
     lz_arrive(p.bar);
-    if (!lz_wait(p.bar, ++epoch * G)) {
+    if (!lz_wait(p.bar, ++epoch * G + p.extra, p.wait_limit)) {
       if (tid == 0) p.out[4] = 1.0;
       return;
     }
@@ -666,7 +668,7 @@ __global__ void __launch_bounds__(kLzThreads) lanczos_step_kernel(LzArgs p) {
     __syncthreads();
     lz_dots(x, 0, x, n, 0, true, part_n + b, G, red);
     lz_arrive(p.bar);
-    if (!lz_wait(p.bar, ++epoch * G)) {
+    if (!lz_wait(p.bar, ++epoch * G + p.extra, p.wait_limit)) {
       if (tid == 0) p.out[4] = 1.0;
       return;
     }
@@ -723,11 +725,29 @@ void dot_multi(const double* V, long long ldv, int k, const double* w, long long
   A2_CHECK_LAUNCH();
 }
 
+namespace {
+
+__global__ void __launch_bounds__(kLzThreads)
+tridiag_kernel(const double* a, const double* b, int k, double* out) {
+  extern __shared__ __align__(16) double lz_smem[];
+  TriShared& S = *reinterpret_cast<TriShared*>(lz_smem);
+  const int tid = threadIdx.x;
+  if (tid < k) S.a[tid] = a[tid];
+  if (tid + 1 < k) S.b[tid] = b[tid];
+  __syncthreads();
+  tri_lowest(S, k);
+  if (tid < k) out[2 + tid] = S.z[tid];
+  if (tid == 0) {
+    out[0] = S.theta;
+    out[1] = k > 1 && S.state != 1 ? 1.0 : 0.0;
+  }
+}
+
 // The slice of a worker: at least 128 entries (four warps' worth), at most what spreads N
 // over all SMs but the one of the tridiagonal block.
-void lanczos_step(double* V, double* w, long long N, int j, double beta_prev, bool write_next,
-                  double* tri, double* partial, unsigned* bar, unsigned* bar_next,
-                  double* out, cudaStream_t s) {
+void launch_step(double* V, double* w, long long N, int j, double beta_prev, bool write_next,
+                 double* tri, double* partial, unsigned* bar, unsigned* bar_next, double* out,
+                 unsigned wait_limit, unsigned extra, cudaStream_t s) {
   A2_REQUIRE(j >= 0 && j < 63, "Lanczos step: at most 63 basis vectors");
   constexpr size_t kSliceMax = 160 * 1024;
   static PerDevice<bool> set;
@@ -757,12 +777,45 @@ void lanczos_step(double* V, double* w, long long N, int j, double beta_prev, bo
   p.bar = bar;
   p.bar_next = bar_next;
   p.out = out;
+  p.wait_limit = wait_limit;
+  p.extra = extra;
   const size_t smem = std::max(sizeof(TriShared),
                                p.in_smem ? sizeof(double) * (size_t)chunk : (size_t)0);
   void* args[] = {&p};
   const void* kernel = p.workers > 64 ? (const void*)lanczos_step_kernel<true>
                                       : (const void*)lanczos_step_kernel<false>;
   A2_CUDA(cudaLaunchCooperativeKernel(kernel, dim3(p.workers + 1), dim3(kLzThreads), args, smem, s));
+  A2_CHECK_LAUNCH();
+}
+
+}  // namespace
+
+void lanczos_step(double* V, double* w, long long N, int j, double beta_prev, bool write_next,
+                  double* tri, double* partial, unsigned* bar, unsigned* bar_next,
+                  double* out, cudaStream_t s) {
+  launch_step(V, w, N, j, beta_prev, write_next, tri, partial, bar, bar_next, out, kLzWaitLimit, 0,
+              s);
+}
+
+bool lanczos_selftest_timeout(double* partial, double* out, cudaStream_t s) {
+  constexpr long long N = 4096;
+  DevBuf v, tri, bar;
+  v.ensure(sizeof(double) * 3 * N, s);
+  tri.ensure(sizeof(double) * 192, s);
+  bar.ensure(sizeof(unsigned) * 4, s);
+  fill_zero(v.p, sizeof(double) * 3 * N, s);
+  fill_zero(bar.p, sizeof(unsigned) * 4, s);
+  double* V = v.as<double>();
+  out[4] = 0.0;
+  launch_step(V, V + 2 * N, N, 0, 0.0, false, tri.as<double>(), partial, bar.as<unsigned>(),
+              bar.as<unsigned>() + 2, out, 1u << 14, 1, s);
+  A2_CUDA(cudaStreamSynchronize(s));
+  return out[4] != 0.0;
+}
+
+void tridiag_lowest(const double* a, const double* b, int k, double* out, cudaStream_t s) {
+  A2_REQUIRE(k >= 1 && k <= 63, "tridiagonal size 1..63");
+  tridiag_kernel<<<1, kLzThreads, sizeof(TriShared), s>>>(a, b, k, out);
   A2_CHECK_LAUNCH();
 }
 
