@@ -1478,88 +1478,74 @@ __global__ void tgk_invit_kernel(const double* d, const double* e, int n, const 
 // entries A[row][col] read by `left` (column i below the diagonal: rows i+1.., off = 0) or
 // by the right side (row i beyond the superdiagonal: columns i+2.., off = 1).  One warp per
 // column (kApplyCols per block): a lane always owns the entries j = lane mod 32, so a
-// reflection needs only the warp's shuffles.  The reflections are staged in shared memory
-// g at a time (g >= 1, rows padded to p + 1 against bank conflicts), read from global
-// memory once per block, coalesced; g = 0 reads them from global memory directly.  With
-// xsm the block's columns are held in shared memory, otherwise they are updated in place.
+// reflection needs only the warp's shuffles; the columns are updated in place.  The reflections
+// are staged in shared memory g at a time (rows padded to p + 1 against bank conflicts), read
+// from global memory once per block, coalesced.  (For p so large that lq_rows_kernel's three
+// rows do not fit; then one or two reflections do, and no column beside them.)
 constexpr int kApplyCols = 4;
+constexpr int kApplyStage = 2;
+constexpr size_t kApplySmem = 200 * 1024;
 __global__ void __launch_bounds__(32 * kApplyCols)
 bidiag_apply_kernel(const double* A, int lda, int p, int q, const double* tau, int left, double* X,
-                    int r, int g, int xsm) {
-  extern __shared__ double x[];           // [kApplyCols x p if xsm], then g x (p + 1)
-  __shared__ double taus[16];             // tau of the staged reflections (g <= 16)
-  double* vs = x + (xsm ? (size_t)kApplyCols * p : 0);
+                    int r, int g) {
+  extern __shared__ double vs[];          // g x (p + 1)
+  __shared__ double taus[kApplyStage];    // tau of the staged reflections
   const int off = left ? 0 : 1;
   const int ps = p + 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  auto vglob = [&](int i, int j) {        // entry j of v_i, j >= i + off
-    return j == i + off ? 1.0 : (left ? A[(size_t)j * lda + i] : A[(size_t)i * lda + j]);
-  };
   for (int k0 = blockIdx.x * kApplyCols; k0 < r; k0 += gridDim.x * kApplyCols) {
     const bool active = k0 + warp < r;
-    double* xk = xsm ? x + (size_t)warp * p : X + k0 + warp;   // entry j at xk[j * xs]
-    const long long xs = xsm ? 1 : r;
-    if (xsm)
-      for (int j = threadIdx.x; j < p; j += blockDim.x)
+    double* xk = X + k0 + warp;           // entry j at xk[j * r]
+    for (int ihi = q; ihi > 0; ihi -= g) {
+      const int ilo = max(0, ihi - g), cnt = ihi - ilo;
+      // stage v_ilo .. v_{ihi-1} (entries from row ilo + off on) and tau
+      const int j0 = ilo + off;
+      if (threadIdx.x < cnt) taus[threadIdx.x] = tau[ilo + threadIdx.x];
+      // eight loads in flight per thread (the copy is latency-bound otherwise)
+      const int tot = (p - j0) * cnt;
+      for (int e0 = threadIdx.x; e0 < tot; e0 += 8 * blockDim.x) {
+        double v[8];
 #pragma unroll
-        for (int v = 0; v < kApplyCols; ++v)
-          x[v * p + j] = k0 + v < r ? X[(size_t)j * r + k0 + v] : 0.0;
-    __syncthreads();
-    const int gs = g > 0 ? g : 1;
-    for (int ihi = q; ihi > 0; ihi -= gs) {
-      const int ilo = max(0, ihi - gs), cnt = ihi - ilo;
-      if (g > 0) {   // stage v_ilo .. v_{ihi-1} (entries from row ilo + off on) and tau
-        const int j0 = ilo + off;
-        if (threadIdx.x < cnt) taus[threadIdx.x] = tau[ilo + threadIdx.x];
-        // eight loads in flight per thread (the copy is latency-bound otherwise)
-        const int tot = (p - j0) * cnt;
-        for (int e0 = threadIdx.x; e0 < tot; e0 += 8 * blockDim.x) {
-          double v[8];
+        for (int u = 0; u < 8; ++u) {
+          const int e = e0 + u * blockDim.x;
+          int j = 0, t = 0;
+          if (left) { j = j0 + e / cnt; t = e % cnt; }          // row-major: v_i's across
+          else { t = e / (p - j0); j = j0 + e % (p - j0); }     // one reflection per row
+          const int i = ilo + t;
+          v[u] = 0.0;
+          if (e < tot && j >= i + off)
+            v[u] = j == i + off ? 1.0 : (left ? A[(size_t)j * lda + i] : A[(size_t)i * lda + j]);
+        }
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int e = e0 + u * blockDim.x;
-            int j = 0, t = 0;
-            if (left) { j = j0 + e / cnt; t = e % cnt; }          // row-major: v_i's across
-            else { t = e / (p - j0); j = j0 + e % (p - j0); }     // one reflection per row
-            v[u] = (e < tot && j >= ilo + t + off) ? vglob(ilo + t, j) : 0.0;
-          }
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int e = e0 + u * blockDim.x;
-            if (e < tot) {
-              const int j = left ? j0 + e / cnt : j0 + e % (p - j0);
-              const int t = left ? e % cnt : e / (p - j0);
-              vs[t * ps + j] = v[u];
-            }
+        for (int u = 0; u < 8; ++u) {
+          const int e = e0 + u * blockDim.x;
+          if (e < tot) {
+            const int j = left ? j0 + e / cnt : j0 + e % (p - j0);
+            const int t = left ? e % cnt : e / (p - j0);
+            vs[t * ps + j] = v[u];
           }
         }
-        __syncthreads();
       }
+      __syncthreads();
       if (active)
         for (int i = ihi - 1; i >= ilo; --i) {
-          const double ti = g > 0 ? taus[i - ilo] : tau[i];
+          const double ti = taus[i - ilo];
           if (ti == 0.0) continue;
-          const int j0 = i + off, jb = j0 & ~31;
+          const int ji = i + off, jb = ji & ~31;
           const double* vi = vs + (size_t)(i - ilo) * ps;
           double s0 = 0.0, s1 = 0.0;
           for (int j = jb + lane; j < p; j += 64) {
-            if (j >= j0) s0 = fma(g > 0 ? vi[j] : vglob(i, j), xk[j * xs], s0);
-            if (j + 32 < p) s1 = fma(g > 0 ? vi[j + 32] : vglob(i, j + 32), xk[(j + 32) * xs], s1);
+            if (j >= ji) s0 = fma(vi[j], xk[(size_t)j * r], s0);
+            if (j + 32 < p) s1 = fma(vi[j + 32], xk[(size_t)(j + 32) * r], s1);
           }
           double sum = s0 + s1;
           for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
           const double f = ti * sum;
           for (int j = jb + lane; j < p; j += 32)
-            if (j >= j0) xk[j * xs] = fma(-f, g > 0 ? vi[j] : vglob(i, j), xk[j * xs]);
+            if (j >= ji) xk[(size_t)j * r] = fma(-f, vi[j], xk[(size_t)j * r]);
         }
       __syncthreads();
     }
-    if (xsm)
-      for (int j = threadIdx.x; j < p; j += blockDim.x)
-#pragma unroll
-        for (int v = 0; v < kApplyCols; ++v)
-          if (k0 + v < r) X[(size_t)j * r + k0 + v] = x[v * p + j];
-    __syncthreads();
   }
 }
 
@@ -1848,7 +1834,7 @@ void set_attributes() {
   set.at(current_device(), [] {
     set_smem((const void*)hh_lq_kernel, 200 * 1024);
     set_smem((const void*)hh_form_q_kernel, 200 * 1024);
-    set_smem((const void*)bidiag_apply_kernel, 200 * 1024);
+    set_smem((const void*)bidiag_apply_kernel, kApplySmem);
     set_smem((const void*)tgk_bisect32_kernel<32>, 200 * 1024);
     set_smem((const void*)tgk_refine64_kernel<8>, 200 * 1024);
     set_smem((const void*)tgk_refine64_kernel<16>, 200 * 1024);
@@ -2074,7 +2060,6 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
     return (int)std::max<long long>(32, (want + 31) / 32 * 32);
   };
   const size_t wmax = (size_t)cdiv(rows, 32) * r * W;      // partial sums of any Gram
-  w.x.ensure(sizeof(double) * (size_t)n * rows, s);
   w.v.ensure(sizeof(double) * ((size_t)r * n + (size_t)r * W + W * W + wmax) +
                  sizeof(int) * npan, s);
   double* vecs = w.v.as<double>();
@@ -2136,6 +2121,7 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
     if (3 * sizeof(double) * (size_t)rows <= kLqSmem) {
       // the reflections as explicit rows, then a few columns of P per block in shared memory
       // (lq_rows_kernel on P^T)
+      w.x.ensure(sizeof(double) * (size_t)n * rows, s);
       double* vx = w.x.as<double>();
       reflectors_kernel<<<dim3(cdiv(rows, 32), cdiv(std::max(q, 1), 32)), dim3(32, 8), 0, s>>>(
           A, n, rows, q, left ? 1 : 0, vx);
@@ -2146,16 +2132,11 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
                 s);
       return r;
     }
-    // the block's columns in shared memory when they fit; reflections staged per pass: as
-    // many as fit beside them (at most 16)
-    const long long cap = 200LL * 1024 / 8;
-    const int xsm = (long long)kApplyCols * rows <= cap / 2 ? 1 : 0;
-    const long long room = cap - (xsm ? (long long)kApplyCols * rows : 0);
-    const int g = (int)std::max<long long>(0, std::min<long long>(16, room / (rows + 1)));
-    const size_t smem =
-        sizeof(double) * ((xsm ? (size_t)kApplyCols * rows : 0) + (size_t)g * (rows + 1));
-    bidiag_apply_kernel<<<std::min(cdiv(r, kApplyCols), 4 * device_sms()), 32 * kApplyCols, smem,
-                          s>>>(A, n, rows, q, left ? tu : tv, left ? 1 : 0, P, r, g, xsm);
+    // one or two reflections staged per pass, as many as fit (rows <= 12800)
+    const size_t row = sizeof(double) * ((size_t)rows + 1);
+    const int g = (int)std::min<size_t>(kApplyStage, kApplySmem / row);
+    bidiag_apply_kernel<<<std::min(cdiv(r, kApplyCols), 4 * device_sms()), 32 * kApplyCols, g * row,
+                          s>>>(A, n, rows, q, left ? tu : tv, left ? 1 : 0, P, r, g);
     A2_CHECK_LAUNCH();
   }
   return r;

@@ -1399,30 +1399,6 @@ void precondition(const double* r, const double* diag, const double* theta, doub
 }
 
 // ----------------------------------------------------------------------------- assorted
-__global__ void cols_rev_to_rows_kernel(const double* __restrict__ G, long long ld, int rows,
-                                        int col_first, int r, double* __restrict__ P) {
-  __shared__ double tile[32][33];
-  const int i0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-  for (int j = threadIdx.y; j < 32; j += 8) {           // read columns (contiguous in i)
-    const int c = c0 + j, i = i0 + threadIdx.x;
-    if (c < r && i < rows) tile[j][threadIdx.x] = G[(long long)(col_first - c) * ld + i];
-  }
-  __syncthreads();
-  for (int j = threadIdx.y; j < 32; j += 8) {           // write rows of P (contiguous in c)
-    const int i = i0 + j, c = c0 + threadIdx.x;
-    if (c < r && i < rows) P[(long long)i * r + c] = tile[threadIdx.x][j];
-  }
-}
-void cols_rev_to_rows(const double* G, long long ld, int rows, int col_first, int r, double* P,
-                      cudaStream_t s) {
-  if (rows <= 0 || r <= 0) return;
-  A2_REQUIRE(col_first - (r - 1) >= 0, "cols_rev_to_rows: column range");
-  dim3 grid(cdiv(rows, 32), cdiv(r, 32));
-  A2_REQUIRE(grid.y < 65536, "cols_rev_to_rows: grid too large");
-  cols_rev_to_rows_kernel<<<grid, dim3(32, 8), 0, s>>>(G, ld, rows, col_first, r, P);
-  A2_CHECK_LAUNCH();
-}
-
 __global__ void gather_axpy_atomic_kernel(const double* __restrict__ G,
                                           const long long* __restrict__ index,
                                           const long long* __restrict__ param,
@@ -1530,34 +1506,6 @@ void grad_dots(const double* X, const double* Y, const int4* el, int nel, int Dl
 
 void fill_zero(void* p, size_t bytes, cudaStream_t s) {
   if (bytes) A2_CUDA(cudaMemsetAsync(p, 0, bytes, s));
-}
-
-// Q: rows x k column-major (ld ldq) from orgqr; R: k x k upper (col-major, ld ldr) from geqrf.
-// Flip signs so that diag(R) >= 0: column j of Q and row j of R change sign if R_jj < 0.
-__global__ void sign_fix_kernel(double* Q, int ldq, int rows, double* R, int ldr, int k) {
-  const int j = blockIdx.x;
-  const double d = R[(long long)j * ldr + j];
-  if (d >= 0.0) return;
-  for (int i = threadIdx.x; i < rows; i += blockDim.x) Q[(long long)j * ldq + i] *= -1.0;
-  for (int c = j + threadIdx.x; c < k; c += blockDim.x) R[(long long)c * ldr + j] *= -1.0;
-}
-void sign_fix_qr(double* Q, int ldq, int rows, double* R, int ldr, int k, cudaStream_t s) {
-  if (!k) return;
-  sign_fix_kernel<<<k, 128, 0, s>>>(Q, ldq, rows, R, ldr, k);
-  A2_CHECK_LAUNCH();
-}
-
-__global__ void scale_rows_kernel(double* M, int rows, int cols, const double* sv) {
-  const long long n = (long long)rows * cols;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-       e += (long long)gridDim.x * blockDim.x)
-    M[e] *= sv[e / cols];
-}
-void scale_rows(double* M, int rows, int cols, const double* svals, cudaStream_t s) {
-  long long n = (long long)rows * cols;
-  if (!n) return;
-  scale_rows_kernel<<<grid_for(n), 256, 0, s>>>(M, rows, cols, svals);
-  A2_CHECK_LAUNCH();
 }
 
 // dst[(o0 + i)*dst_s0 + j*dst_s1 + (o2 + k)] = alpha * src[(i*d1 + j)*d2 + k]

@@ -147,10 +147,6 @@ void precondition(const double* r, const double* diag, const double* theta, doub
                   long long n, cudaStream_t s);
 
 // ---- assorted
-// P[i][c] = G[(col_first - c) * ld + i] for i < rows, c < r (P row-major rows x r): the
-// columns col_first, col_first - 1, ... of a column-major matrix, as rows of P.
-void cols_rev_to_rows(const double* G, long long ld, int rows, int col_first, int r, double* P,
-                      cudaStream_t s);
 void fill_zero(void* p, size_t bytes, cudaStream_t s);
 // Enable / disable (default) the rows-per-CTA autotuner of the sparse stages (disabling
 // also forgets its choices).
@@ -172,8 +168,6 @@ int grad_dot_parts(int Dl, int Dr, int Rl, int nw, int n, int nel);
 // out[i]: element el[i]; part: parts * nel values of scratch.
 void grad_dots(const double* X, const double* Y, const int4* el, int nel, int Dl, int Rl, int n,
                int nw, int Dr, int parts, double* part, double* out, cudaStream_t s);
-void sign_fix_qr(double* Q, int ldq, int rows, double* R, int ldr, int k, cudaStream_t s);
-void scale_rows(double* M, int rows, int cols, const double* svals, cudaStream_t s); // M[r,:]*=s[r]
 // TT-sum block copy: dst[(o0 + i)*dst_s0 + j*dst_s1 + o2 + k] = alpha * src[i][j][k]
 // (added to dst when add is set)
 void copy_block3(const double* src, int d0, int d1, int d2, double* dst, long long dst_s0,

@@ -18,7 +18,6 @@
 // BF16 S2 0.78 -> 0.58, S3 1.01 -> 0.76; FP32 pairs S2 + S3 6.34 -> 5.42; bond 7, split
 // products, S3 (three planes in and out) 4.82 -> 3.68.
 #include <algorithm>
-#include <type_traits>
 
 #include "kernels.cuh"
 #include "sparse.cuh"
@@ -76,8 +75,8 @@ __device__ __forceinline__ void df_fma(float& ah, float& al, float wh, float wl,
 }
 
 // OUT: ST_BF16, ST_PLANES (three BF16 planes), ST_DF (FP32 pair), ST_F64 (sum of the pair).
-// ADD: added to the output (BF16).  VEC: every row segment
-// is 16-byte (8-byte for planes) aligned and whole; otherwise element by element.
+// ADD: added to the output (BF16).  VEC: every row segment is 16-byte (8-byte for planes) aligned
+// and whole; otherwise element by element (not for planes).
 template <int IN, int OUT, bool ADD, bool VEC, int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT) sparse_staged_kernel(StArgs a) {
   using TI = typename StIn<IN>::T;
@@ -118,21 +117,15 @@ __global__ void __launch_bounds__(NT, 1024 / NT) sparse_staged_kernel(StArgs a) 
     }
     if constexpr (IN != ST_PLANES) cp_async_wait();
   } else {
-    using SE = typename std::conditional<IN == ST_PLANES, float, TI>::type;
-    SE* eh = reinterpret_cast<SE*>(sh);
-    SE* el = reinterpret_cast<SE*>(sl);
+    TI* eh = reinterpret_cast<TI*>(sh);
+    TI* el = reinterpret_cast<TI*>(sl);
     const int wsh = a.lsh + (NV == 8 ? 3 : 2);         // log2 of the slice's width
     for (int it = threadIdx.x; it < rows << wsh; it += NT) {
       const int row = it >> wsh, v = it & ((1 << wsh) - 1);
       if (v >= nvec) continue;
       const TI* src = in + (long long)(row / nt) * g.in_sw + (long long)(row % nt) * g.in_st + v;
-      if constexpr (IN == ST_PLANES) {
-        eh[it] = __bfloat162float(src[0]) + (__bfloat162float(src[a.in_plane]) +
-                                             __bfloat162float(src[2 * a.in_plane]));
-      } else {
-        eh[it] = __ldg(src);
-        if constexpr (kPair) el[it] = __ldg(src + a.in_plane);
-      }
+      eh[it] = __ldg(src);
+      if constexpr (kPair) el[it] = __ldg(src + a.in_plane);
     }
   }
   __syncthreads();
@@ -219,19 +212,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) sparse_staged_kernel(StArgs a) 
       for (int i = 0; i < NV; ++i) {
         split3f(acc[i], h[i], m[i], l3[i]);
       }
-      if constexpr (VEC) {
-        *reinterpret_cast<uint2*>(p) = *reinterpret_cast<const uint2*>(h);
-        *reinterpret_cast<uint2*>(p + a.out_plane) = *reinterpret_cast<const uint2*>(m);
-        *reinterpret_cast<uint2*>(p + 2 * a.out_plane) = *reinterpret_cast<const uint2*>(l3);
-      } else {
-#pragma unroll
-        for (int i = 0; i < NV; ++i)
-          if (i < nst) {
-            p[i] = h[i];
-            p[a.out_plane + i] = m[i];
-            p[2 * a.out_plane + i] = l3[i];
-          }
-      }
+      *reinterpret_cast<uint2*>(p) = *reinterpret_cast<const uint2*>(h);
+      *reinterpret_cast<uint2*>(p + a.out_plane) = *reinterpret_cast<const uint2*>(m);
+      *reinterpret_cast<uint2*>(p + 2 * a.out_plane) = *reinterpret_cast<const uint2*>(l3);
     } else if constexpr (OUT == ST_DF) {
       float* p = reinterpret_cast<float*>(a.out) + o;
       float h[NV], lo[NV];
@@ -283,10 +266,13 @@ void st_launch(const StArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
 template <int IN, int OUT, bool ADD>
 void st_launch_vec(const StArgs& a, bool vec, dim3 grid, size_t smem, cudaStream_t s) {
   const bool one = smem > kStTwo;        // one block on an SM: twice the threads
-  if (vec && one) st_launch<IN, OUT, ADD, true, 1024>(a, grid, smem, s);
-  else if (vec) st_launch<IN, OUT, ADD, true, 512>(a, grid, smem, s);
-  else if (one) st_launch<IN, OUT, ADD, false, 1024>(a, grid, smem, s);
-  else st_launch<IN, OUT, ADD, false, 512>(a, grid, smem, s);
+  if (vec) {
+    if (one) st_launch<IN, OUT, ADD, true, 1024>(a, grid, smem, s);
+    else st_launch<IN, OUT, ADD, true, 512>(a, grid, smem, s);
+  } else if constexpr (IN != ST_PLANES) {
+    if (one) st_launch<IN, OUT, ADD, false, 1024>(a, grid, smem, s);
+    else st_launch<IN, OUT, ADD, false, 512>(a, grid, smem, s);
+  }
 }
 
 }  // namespace
@@ -336,6 +322,7 @@ bool sparse_staged(const SparseRows<float>& sp, const SparseGeom& g, int in_kind
                    reinterpret_cast<uintptr_t>(out) % std::min(16, osz * nv) == 0;
   if (in_kind == ST_BF16 && (blocks < 128 || (!vec && sp.nnz_total < 16LL * sp.nrows)))
     return false;
+  if (in_kind == ST_PLANES && !vec) return false;   // (its callers' rows are padded)
   StArgs a;
   a.sp = sp;
   a.g = g;
