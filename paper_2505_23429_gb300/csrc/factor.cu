@@ -1900,8 +1900,12 @@ void lq_rows(RowsArgs p, cudaStream_t s, int per_sm = 2) {
 }  // namespace
 
 // Launch shape of the shared-memory bidiagonalisation: blocks (0: the rows do not fit), cluster
-// size and shared memory.  Clusters of kBdCluster where there are rows for two of them; the blocks
-// of all clusters that the device holds at once (about 144 of 152 SMs).
+// size and shared memory.  Clusters of kBdCluster (the blocks of all clusters that the device
+// holds at once, about 144 of 152 SMs) save atomics and arrivals, for two more cluster barriers a
+// step.  That pays above 128 columns (ms, single blocks / clusters: 1024 x 1024 23.9 / 23.6, 256 x
+// 1024 4.03 / 3.89, 160 x 1536 2.75 / 2.61; 128 x 1024 1.77 / 1.83, 32 x 1024 0.52 / 0.54, 8 x 1024 0.244
+// / 0.253), unless the eight SMs less cost a block's warps one more round over its rows (9300 x 256
+// 9.20 / 9.42, 9300 x 160 5.24 / 5.41; 4000 x 256 with the same rounds 6.11 / 5.97).
 struct BdShape {
   int blocks = 0, cluster = 1;
   size_t smem = 0;
@@ -1929,19 +1933,16 @@ BdShape bd_shape(int m, int n) {
     A2_CUDA(cudaOccupancyMaxActiveClusters(&n, hh_bidiag_smem_kernel, &cfg));
     return n;
   });
-  if (m >= 2 * kBdCluster) {
-    const int nb = std::min(m / kBdCluster, nclusters) * kBdCluster;
-    if (nb >= kBdCluster && bytes(nb) <= most) {
-      sh.blocks = nb;
-      sh.cluster = kBdCluster;
-      sh.smem = bytes(nb);
-      return sh;
-    }
-  }
-  const int nb = std::max(1, std::min(m, device_sms()));
-  if (bytes(nb) <= most) {
+  const int single = std::max(1, std::min(m, device_sms()));
+  const int nb = std::min(m / kBdCluster, nclusters) * kBdCluster;
+  auto rounds = [&](int blocks) { return cdiv(cdiv(m, blocks), kFacThreads / 32); };
+  if (n > 128 && nb >= 2 * kBdCluster && bytes(nb) <= most && rounds(nb) == rounds(single)) {
     sh.blocks = nb;
+    sh.cluster = kBdCluster;
     sh.smem = bytes(nb);
+  } else if (bytes(single) <= most) {
+    sh.blocks = single;
+    sh.smem = bytes(single);
   }
   return sh;
 }
