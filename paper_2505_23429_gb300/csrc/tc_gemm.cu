@@ -2066,7 +2066,10 @@ __device__ __forceinline__ uint2 oz_pack(int a, int b, int c, int d, float sc) {
 // One warp per row and 256-wide K chunk, whose entries stay in registers (eight per lane): one
 // read, the chunk's largest exponent by a warp reduction, then each slice of four
 // consecutive entries as one 8-byte vector.  The last K block is filled with zeros.  Bound by
-// HBM: 8 bytes read and 14 written per entry.  With one scale for a whole row (read twice, one
+// HBM: 8 bytes read and 14 written per entry.  Rows whose entries lie far apart (sk > 1, sr = 1: x,
+// ket, bra) take this kernel too: neighbouring warps read neighbouring rows, whose sectors meet in
+// L1 and L2 (x at D = 256, 4096 x 256: 12 us, by ozaki_split_cols_kernel 23; D = 64 7, 9; D = 512
+// 27, 44).  With one scale for a whole row (read twice, one
 // warp for 143872 entries of T3) the slicing of S4's operand took 2.75 ms at D = 256 with the
 // slicing of x, now 1.82.
 constexpr int kOzGroup = 256;              // entries that share a scale (tc_oz_kernel's chunk)
@@ -2209,10 +2212,6 @@ void ozaki_split_cols(const double* X, long long ldx, int N, int K, __nv_bfloat1
 void ozaki_split(const double* X, long long sr, long long sk, int rows, int K, __nv_bfloat16* P,
                  cudaStream_t s) {
   if (rows <= 0 || K <= 0) return;
-  if (sr == 1 && sk > 1) {               // entries of a row far apart: the transposed kernel
-    ozaki_split_cols(X, sk, rows, K, P, s);
-    return;
-  }
   const long long ntasks = (long long)rows * cdiv(K, kOzGroup);
   const int grid = (int)std::min<long long>((ntasks + 7) / 8, 152 * 32);   // eight warps per block
   ozaki_split_kernel<<<grid, 256, 0, s>>>(X, sr, sk, rows, K, P, ntasks);
