@@ -54,9 +54,10 @@ REF_COUNTS = dict(iterations=64,
 # classes reported by time share only (latency-bound FP64 factorisations)
 LATENCY_BOUND = ("svd", "lq")
 # DRAM traffic / algorithmic bytes of a kernel class, from its ncu capture (the sparse
-# stages at D = 128, one FP64-class environment update at D = 256: all its launches);
+# stages with FP32 inputs at D = 128; one FP64-class environment update at D = 256: all its
+# launches);
 # the bench scales it to its own launches
-DRAM_TRAFFIC_RATIO = {"emu_s2": 0.963, "emu_s3": 0.961, "env": 3.78}
+DRAM_TRAFFIC_RATIO = {"emu_s2": 0.963, "emu_s3": 0.961, "env": 2.10}
 DRAM_TRAFFIC_CAPTURE = {"emu_s2": "profiles/sparse_rows_kernel_heff_D128.md",
                         "emu_s3": "profiles/sparse_rows_kernel_heff_D128.md",
                         "env": "profiles/env_update_f64e_D256.md"}

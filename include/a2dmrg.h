@@ -63,11 +63,11 @@ typedef enum {
   A2_F64EMU = 5  /* H_eff to FP64-class accuracy (~2^-48) on tcgen05 (Ozaki scheme): FP64
                    operands split row by row and 256 entries at a time into seven slices
                    of balanced 8-bit digits (BF16), the 28 slice pairs of level <= 8
-                   accumulated in FP32 per 256 entries (exact up to the two highest levels'
-                   units of 2^-46) and summed by error-free two-sums into FP32 pairs; operands of
-                   2^128 and more and non-finite ones give NaN, below 2^-72 their accuracy is
-                   about 2^-126 absolute; the
-                   sparse MPO stages in double-float (FP32 pairs); environments FP64,
+                   accumulated in FP32 per 256 entries (levels 2 to 5 exactly, 6 to 8 up to
+                   the rounding of their own sums where digits are extreme) and summed by
+                   error-free two-sums into FP32 pairs; operands of 2^128 and more and
+                   non-finite ones give NaN, below 2^-72 their accuracy is about 2^-126
+                   absolute; the sparse MPO stages in double-float (FP32 pairs); environments FP64,
                    their updates emulated the same way (two Ozaki GEMMs and a double-float
                    sparse stage) above a small size, plain FP64 below; vectors, SVD and
                    coarse problem in FP64 */

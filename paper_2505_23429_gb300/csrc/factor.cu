@@ -804,8 +804,8 @@ hh_bidiag_kernel(double* A, int m, int n, double* d, double* e, double* tau_u,
 // its products itself: 27.7 thousand, of them 9.3 in the products and their 150000 atomics,
 // 6.1 in reading 148 partial norms and the reflection's scalars, 5.8 in the barrier of 148
 // arrivals; 13.4 ms in all.  With clusters of four a quarter of the atomics and arrivals
-// remain and the norm is one number: 10.5 ms (clusters of eight leave room for 120 blocks only:
-// 12.0); 796 x 597: 6.4 -> 5.1 ms.
+// remain and the norm is one number: 10.6 ms (clusters of eight leave room for 120 blocks only:
+// 12.0); 796 x 597: 6.4 -> 5.2 ms.  bd_shape says where clusters are taken.
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;

@@ -15,7 +15,7 @@
 //     took more than half of the squared norm (the criterion of Daniel, Gragg, Kaufman and
 //     Stewart, Math. Comp. 30, 1976): w is then orthogonal to working precision;
 //   * one more block solves the tridiagonal while the workers re-orthogonalise.
-// Mean of the steps j = 0 .. 20, device time: N = 4096 22 us (208 us as separate kernels),
+// Mean of the steps j = 0 .. 20, device time: N = 4096 23 us (208 us as separate kernels),
 // N = 2^20 126 us (380 us; the vectors' traffic alone is ~40 us at this part's copy rate).
 #include <algorithm>
 
@@ -188,9 +188,9 @@ __device__ __forceinline__ void lz_total_loop(const double* part, int workers, i
 // tot[q] = sum over the workers of part[q * stride + i], q < kk, in a fixed order.  WIDE (above 64
 // workers): a warp takes every eighth value and its lanes the workers; four threads per value,
 // each adding a quarter of the partial sums one after the other, wait for 38 loads and adds at
-// 150 workers (chemistry L = 8, D = 64, mean of a sweep's steps: 28.3 -> 26.3 us).  With fewer the
+// 150 workers (chemistry L = 8, D = 64, mean of a sweep's steps: 30.1 -> 28.0 us).  With fewer the
 // four threads are the faster form, as they need no sums over a warp (Heisenberg, D = 32, 32
-// workers: 24.5 us, by warps 25.7).
+// workers: 26.8 us, by warps 27.6).
 template <bool WIDE>
 __device__ void lz_totals(const double* part, int workers, int stride, int kk, double* tot,
                           double (*red)[64]) {

@@ -721,9 +721,13 @@ void launch(const __nv_bfloat16* A, long long lda, const __nv_bfloat16* B, long 
 //  * MMAs on the same A slice follow each other and take it from the collector buffer.
 // Exactness: |digit| <= 128, so level l's sum over a chunk is an integer below
 // 256 (l - 1) 2^14 units, at most 2^24 for l <= 5: exact in FP32.  Level 6 reaches 1.25 x
-// 2^24 only if all digits are extreme and is then off by one unit, 2^-46 of the row and
-// column scale, per addition; levels 7 and 8 share an accumulator (level 8 is rounded at
-// 2^-24 of the level 7 sum, ~2^-60).
+// 2^24 only if all digits are extreme; its last additions are then off by up to one unit each, 2^-46
+// of the row and column scale.  Levels 7 and 8 share an accumulator, so that an addition is off by
+// up to 2^-24 of the level 7 sum: up to 2^-53 of the scales where all digits are extreme, ~2^-60
+// where their signs are random.  Measured over operands whose digits all lie in [112, 127], [96, 127],
+// [64, 127], [126, 127], [0, 127] or [-128, 127], against exact integers: at most 2^-46.6, 2^-46.0, 2^-45.2 of sum |a| |b| at
+// K = 256, 512, 1024, where 36 pairs with exact level sums were off by up to 2^-45.4, 2^-44.7, 2^-43.7.
+// Both are the rounding of the pairs' low part, which has an error for every drained accumulator.
 // The epilogue adds every accumulator into a double-float register pair (hi + lo, Knuth's
 // error-free two-sum), so no per-level tile reaches memory.
 //
@@ -2008,8 +2012,9 @@ void tc_heff1_f32emu(cudaStream_t s, int n, int Rl, int Rr, int Dl, int Dr,
 // significand (7 slices for 55 bits; digits of one sign would need 8 slices and 36 pairs for
 // the same products of 2^14).  A product of slice i of A with slice j of B is an integer
 // multiple of the unit 2^(e_A + e_B + 2 - 8 (i + j)) of the chunk; the pairs with i + j <= 8 are
-// kept (28; the rest lie below 2^-58 of the scales), see tc_oz_kernel for their exact
-// accumulation chunk by chunk.
+// kept (28).  Of those left out, level 9 counts: six pairs of at most 2^-56 of the scales each, in
+// all at most 2^-53.4 a product (eight slices of 7 bits and 36 pairs left out as much).  See
+// tc_oz_kernel for the accumulation chunk by chunk.
 // Range: slices are BF16 values, so a chunk that holds a NaN, an infinity or an entry of 2^128 or
 // more has no slices.  Its first slice is written as NaN, which reaches every product of
 // the row.  At the other end, slices whose scale lies below 2^-126 are zero: chunks whose largest
