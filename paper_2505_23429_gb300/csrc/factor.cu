@@ -3,15 +3,16 @@
 // Householder LQ (Golub & Van Loan, Matrix Computations, 4th ed., Sec. 5.1.2-5.1.3 and
 // 5.2.1, applied to the rows of M instead of the columns): reflection i maps the trailing
 // part of row i onto a multiple of e_i and is applied from the right to the rows below.
-// One cooperative persistent kernel walks the k reflections; every block owns the rows
+// hh_lq_kernel, one cooperative persistent kernel, walks the k reflections; every block owns the rows
 // r with r % gridDim.x == blockIdx.x, so a row is only ever touched by one block, and the
 // block that owns row i + 1 forms and publishes the next reflection as soon as it has
 // updated that row.  The blocks synchronise on those publications alone (one flag per
 // reflection, bounded waits: after kBarrierLimit polls a wait raises the error word and
 // every block leaves), so they pipeline behind the owners instead of meeting at a
-// grid-wide barrier per reflection.  Q is then formed row by row: row j of
-// Q is e_j^T H_j H_{j-1} ... H_0 (the reflections H_i with i > j leave e_j unchanged),
-// so every row is independent.
+// grid-wide barrier per reflection.  It takes the matrices with many more rows than columns and
+// rows beyond shared memory, the kernels by panels further below the others (lq_by_panels).  Q is
+// then formed row by row: row j of Q is e_j^T H_j H_{j-1} ... H_0 (the reflections H_i with i > j
+// leave e_j unchanged), so every row is independent.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -352,12 +353,11 @@ __device__ __forceinline__ double ld_cluster(const double* p, unsigned rank) {
 //     the block's rows.  The same kernel forms Q from e_j.
 // Bound: the FP64 pipe in the rows (two multiply-adds per entry and reflection), latency in the
 // panel (~5000 cycles a reflection: chains of FP64 instructions at 64 cycles each, the cluster
-// exchange ~1000).  As one cooperative kernel, each reflection handed from the block that
-// owned a row to all others through device memory, a reflection took 13 us.
+// exchange ~1000).  In the cooperative kernel, each reflection handed from the block that
+// owned a row to all others through device memory, a reflection takes 13 us at this width.
 // 597 x 2388: reflections 7.9 -> 5.6 ms (panels 2.8), Q 3.0 -> 2.6 ms; with the next panel beside
 // the update of the rows below it 5.1 (forming Q beside the panels as well gains nothing: it
-// takes the FP64 pipe from them).  The whole call at 256 x 1024 2.63 -> 2.15 ms, 1024 x 256 1.78 ->
-// 1.77 (1.90 one after the other).
+// takes the FP64 pipe from them).  The whole call at 256 x 1024 2.63 -> 2.20 ms.
 constexpr int kLqPanel = 32;
 constexpr int kLqCluster = 16;
 constexpr int kLqAhead = 64;       // rows below the next panel that are worth a second stream
@@ -2143,6 +2143,19 @@ int svd_trunc(const double* M, int rows, int cols, int D_max, double tol, double
   return r;
 }
 
+// Whether the reflections are formed panel by panel.  Beside a panel (32 reflections of about
+// 2.6 us) the rows below it take the reflections of the one before; where there are many more rows
+// than columns these updates are the longer part, and the cooperative kernel, whose blocks each
+// update their own rows as soon as a reflection is published, is the faster form: 768 x 256 1.77 ms, by
+// panels 1.81; 2400 x 200 1.41, 1.65; 512 x 128 0.859, 0.874; 2400 x 400 3.36, 3.56; 1280 x 64 0.452,
+// 0.464.  Below these lines and from 480 columns on, where a vector fetched once for several rows
+// counts, it loses: 400 x 200 1.39, 1.36; 384 x 128 0.861, 0.856; 1600 x 400 3.25, 3.15; 768 x 64 0.453,
+// 0.447; 4096 x 512 6.63, 6.49; 4608 x 768 12.6, 11.7.
+bool lq_by_panels(int rows, int cols) {
+  if (cols < 48 || cols >= 480) return true;
+  return rows < (long long)(cols < 96 ? 16 : cols < 200 ? 4 : cols <= 320 ? 3 : 6) * cols;
+}
+
 int hh_lq(const double* M, int rows, int cols, double* L, double* Q, FactorWork& w,
           cudaStream_t s) {
   const int k = std::min(rows, cols);
@@ -2158,7 +2171,8 @@ int hh_lq(const double* M, int rows, int cols, double* L, double* Q, FactorWork&
   double* beta = tau + k;
   A2_CUDA(cudaMemcpyAsync(A, M, sizeof(double) * (size_t)rows * cols, cudaMemcpyDeviceToDevice, s));
   set_attributes();
-  if (3 * vbytes <= kLqSmem) {
+  const bool fits = 3 * vbytes <= kLqSmem;
+  if (fits && lq_by_panels(rows, cols)) {
     // A panel's reflections go to the rows of the next panel first; the next panel then runs
     // beside the update of the other rows, on the second stream (a panel is bound by latency and
     // takes at most 16 SMs).
@@ -2214,10 +2228,8 @@ int hh_lq(const double* M, int rows, int cols, double* L, double* Q, FactorWork&
       i0 += b;
     }
     wait_side();
-    lq_rows(RowsArgs{Q, cols, 1, k, cols, V, cols, tau, k - 1, k, -1, 0, beta, 0}, s);
   } else {
-    // rows of more than 9200 entries (three do not fit in shared memory): the kernels that
-    // keep the rows in device memory
+    // the rows stay in device memory, each with its owner
     w.bar.ensure(sizeof(GridBarrier) + sizeof(int) * (size_t)k, s);
     A2_CUDA(cudaMemsetAsync(w.bar.p, 0, sizeof(GridBarrier) + sizeof(int) * (size_t)k, s));
     // cooperative launch: every block resident at once (the ready flags rely on it)
@@ -2232,6 +2244,10 @@ int hh_lq(const double* M, int rows, int cols, double* L, double* Q, FactorWork&
     A2_CUDA(cudaLaunchCooperativeKernel((const void*)hh_lq_kernel, dim3(grid), dim3(kFacThreads),
                                         args, vbytes, s));
     count_launch();
+  }
+  if (fits) {
+    lq_rows(RowsArgs{Q, cols, 1, k, cols, V, cols, tau, k - 1, k, -1, 0, beta, 0}, s);
+  } else {
     hh_form_q_kernel<<<std::min(k, 4 * device_sms()), kFacThreads, vbytes, s>>>(V, tau, cols, k, Q);
     A2_CHECK_LAUNCH();
     hh_sign_rows_kernel<<<std::min(k, 1024), 128, 0, s>>>(Q, cols, k, beta);
